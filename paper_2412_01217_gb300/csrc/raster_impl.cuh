@@ -193,10 +193,31 @@ __device__ __forceinline__ TileInfo tile_info(const RasterArgs &a, int item) {
 constexpr int kFwdHalfChunk = 32;
 constexpr int kFwdHalfQueue = kFwdHalfChunk + 32;  // < kFwdHalfChunk pending + one 32-entry scan
 
+// acc[0 .. 3] += w f where w != 0 (a lane without a contribution takes nothing from a
+// non-finite feature), predicated instead of branched around: the four entries of a group
+// then share one instruction stream and their loads and sums overlap.
+__device__ __forceinline__ void fma4_if(float *acc, float w, const float4 &f) {
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.f32 p, %4, 0f00000000;\n\t"
+        "@p fma.rn.f32 %0, %4, %5, %0;\n\t@p fma.rn.f32 %1, %4, %6, %1;\n\t"
+        "@p fma.rn.f32 %2, %4, %7, %2;\n\t@p fma.rn.f32 %3, %4, %8, %3;\n}\n"
+        : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3])
+        : "f"(w), "f"(f.x), "f"(f.y), "f"(f.z), "f"(f.w));
+}
+
+template <int N>
+struct IntC {
+    static constexpr int value = N;
+};
+
+// Entries whose alpha the forward evaluates together (before their serial recurrence).
+template <int PPT>
+__host__ __device__ constexpr int fwd_group() { return PPT == 1 ? 4 : 2; }
+
 template <int C, int PPT, bool HALF = false>
 __global__ void __launch_bounds__(kMaxTileThreads) raster_fwd_kernel(RasterArgs a) {
     pdl_begin();
     constexpr int NF = 4 + C;
+    constexpr int GF = fwd_group<PPT>();
     constexpr bool hm = HALF;
     static_assert(!HALF || PPT == 1, "half mode runs one pixel per thread");
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -243,43 +264,52 @@ __global__ void __launch_bounds__(kMaxTileThreads) raster_fwd_kernel(RasterArgs 
             done[k] = !(px < vw.W && py < vw.H);
             n_done += done[k];
         }
-        // staged row j, list position pos: alpha at the thread's pixels, front to back
-        auto entry = [&](const int j, const int pos) {
-            const float4 g0 = s_geo0[j];
-            const float4 g1 = s_geo1[j];
-            float w[PPT];
-            bool any = false;
+        // n staged rows row_of(i) at list positions pos_of(i), front to back: first every alpha of
+        // the group (no dependence between entries), then the recurrence in T and the feature sums
+        auto group = [&](auto n_c, auto row_of, auto pos_of) {
+            constexpr int n = decltype(n_c)::value;
+            float al[n][PPT];  // 0: no contribution
 #pragma unroll
-            for (int k = 0; k < PPT; ++k) {
-                w[k] = 0.f;
-                if (done[k]) continue;
-                AlphaEval e;
-                if (!eval_alpha(fx - g0.x, (float)(wt.ly + 4 * k) - g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w,
-                                a.alpha_max, a.alpha_min, e))
-                    continue;
-                const float Tn = __fmul_rn(T[k], __fsub_rn(1.f, e.alpha));
-                if (Tn < a.T_min) {
-                    done[k] = true;
-                    ++n_done;
-                    continue;
-                }
-                w[k] = e.alpha * T[k];
-                T[k] = Tn;
-                last[k] = pos + 1;
-                ++nc[k];
-                any = true;
-            }
-            if (!any) return;
-            const float4 *f4 = reinterpret_cast<const float4 *>(s_feat + (size_t)j * NF);
-#pragma unroll
-            for (int q = 0; q < NF / 4; ++q) {
-                const float4 f = f4[q];
+            for (int i = 0; i < n; ++i) {
+                const float4 g0 = s_geo0[row_of(i)];
+                const float4 g1 = s_geo1[row_of(i)];
 #pragma unroll
                 for (int k = 0; k < PPT; ++k) {
-                    acc[k][4 * q + 0] = fmaf(w[k], f.x, acc[k][4 * q + 0]);
-                    acc[k][4 * q + 1] = fmaf(w[k], f.y, acc[k][4 * q + 1]);
-                    acc[k][4 * q + 2] = fmaf(w[k], f.z, acc[k][4 * q + 2]);
-                    acc[k][4 * q + 3] = fmaf(w[k], f.w, acc[k][4 * q + 3]);
+                    AlphaEval e;
+                    const bool hit = eval_alpha(fx - g0.x, (float)(wt.ly + 4 * k) - g0.y, g0.z, g0.w, g1.x, g1.y,
+                                                g1.z, g1.w, a.alpha_max, a.alpha_min, e);
+                    al[i][k] = hit ? e.alpha : 0.f;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < n; ++i) {
+                float w[PPT];
+                bool any = false;
+#pragma unroll
+                for (int k = 0; k < PPT; ++k) {
+                    const float A = al[i][k];
+                    const float Tn = __fmul_rn(T[k], __fsub_rn(1.f, A));
+                    bool hit = A > 0.f && !done[k];
+                    if (hit && Tn < a.T_min) {
+                        done[k] = true;
+                        ++n_done;
+                        hit = false;
+                    }
+                    w[k] = hit ? A * T[k] : 0.f;
+                    if (hit) {
+                        T[k] = Tn;
+                        last[k] = pos_of(i) + 1;
+                        ++nc[k];
+                        any = true;
+                    }
+                }
+                if (!__any_sync(SG_FULL_MASK, any)) continue;
+                const float4 *f4 = reinterpret_cast<const float4 *>(s_feat + (size_t)row_of(i) * NF);
+#pragma unroll
+                for (int q = 0; q < NF / 4; ++q) {
+                    const float4 f = f4[q];
+#pragma unroll
+                    for (int k = 0; k < PPT; ++k) fma4_if(&acc[k][4 * q], w[k], f);
                 }
             }
         };
@@ -297,10 +327,18 @@ __global__ void __launch_bounds__(kMaxTileThreads) raster_fwd_kernel(RasterArgs 
                     if (__all_sync(SG_FULL_MASK, n_done == PPT)) break;
                     const int jl = j0 + lane;
                     uint32_t cm = __ballot_sync(SG_FULL_MASK, jl < cnt && !wt.misses(s_geo2[jl], s_geo1[jl], ln_amin));
-                    while (cm) {
-                        const int j = j0 + __ffs(cm) - 1;
-                        cm &= cm - 1;
-                        entry(j, b0 + j);
+                    for (int m = __popc(cm); m >= GF; m -= GF) {
+                        int row[GF];
+#pragma unroll
+                        for (int i = 0; i < GF; ++i) {
+                            row[i] = j0 + __ffs(cm) - 1;
+                            cm &= cm - 1;
+                        }
+                        group(IntC<GF>(), [&](int i) { return row[i]; }, [&](int i) { return b0 + row[i]; });
+                    }
+                    for (; cm; cm &= cm - 1) {
+                        const int row = j0 + __ffs(cm) - 1;
+                        group(IntC<1>(), [row](int) { return row; }, [b0, row](int) { return b0 + row; });
                     }
                 }
             }
@@ -333,10 +371,13 @@ __global__ void __launch_bounds__(kMaxTileThreads) raster_fwd_kernel(RasterArgs 
                 stage_rows_warp<NF>(a, C, [&](int j) { return s_qr[j]; }, c, ti.px0, ti.py0, rec_base, s_geo0, s_geo1,
                                     nullptr, s_feat, nullptr);
                 __syncwarp();
-                for (int j = 0; j < c; ++j) {
+                int j = 0;
+                for (; j + GF <= c; j += GF) {
                     if (__all_sync(SG_FULL_MASK, n_done == PPT)) break;
-                    entry(j, s_q[j]);
+                    group(IntC<GF>(), [j](int i) { return j + i; }, [s_q, j](int i) { return s_q[j + i]; });
                 }
+                if (j + GF > c)  // (else the pixels are saturated)
+                    for (; j < c; ++j) group(IntC<1>(), [j](int) { return j; }, [s_q, j](int) { return s_q[j]; });
                 __syncwarp();
                 // drop the staged entries from the queue
                 const int rest = qn - c;  // (< 32)
@@ -387,7 +428,7 @@ __global__ void __launch_bounds__(kMaxTileThreads) raster_fwd_kernel(RasterArgs 
 // with w = alpha T and P = (1, X, Y, X^2, XY, Y^2) the pixel offsets from the warp centre.
 // The 2D-mean, conic and opacity gradients are linear in the moments (see moment_grads).
 constexpr int kChunk = 16;
-constexpr int kHalfQueue = kChunk + 32;  // half mode: list positions pending (< 16 + one 32-entry scan)
+constexpr int kHalfQueue = kChunk + 32;  // entries pending (< 16 + one 32-entry scan)
 
 template <int NPX>
 __host__ __device__ constexpr int chunk_pitch() { return NPX + 4; }  // 4 mod 32: conflict-free fragments
@@ -401,25 +442,16 @@ __host__ __device__ constexpr int padded_features() { return (NF + 7) / 8 * 8; }
 template <int NF>
 __host__ __device__ constexpr int g_pitch() { return (NF / 4) % 2 == 1 ? NF : NF + 4; }
 
-// shared memory of one warp: G (NPX x g_pitch) and two chunk buffers (16 x chunk_pitch)
-template <int C, int PPT>
-__host__ __device__ constexpr int bwd_warp_floats() {
-    return 32 * PPT * g_pitch<4 + C>() + 2 * kChunk * chunk_pitch<32 * PPT>();
+// shared memory of one warp (4-byte words): the chunk's rows and the queue (with records in
+// half mode), G (NPX x g_pitch) and two chunk buffers (16 x chunk_pitch); a multiple of 16 bytes
+template <int C, int PPT, bool HALF>
+__host__ __device__ constexpr int bwd_warp_words() {
+    return kChunk + (HALF ? 2 : 1) * kHalfQueue + 32 * PPT * g_pitch<4 + C>() + 2 * kChunk * chunk_pitch<32 * PPT>();
 }
 
-// A fragment (16 x 8, row-major, pitch ld) at column k0: a0 (gid, tig), a1 (gid + 8, tig),
-// a2 (gid, tig + 4), a3 (gid + 8, tig + 4); rows outside `keep` read as zero, and so do
-// columns k0 + 4 .. k0 + 7 unless `upper` (the part of the last feature tile that is not
-// stored).
-__device__ __forceinline__ void load_a_split(const float *m, int ld, int k0, int gid, int tig, bool keep0,
-                                             bool keep1, uint32_t (&ah)[4], uint32_t (&al)[4],
-                                             bool upper = true) {
-    const float *p = m + gid * ld + k0 + tig;
-    const float v[4] = {keep0 ? p[0] : 0.f, keep1 ? p[8 * ld] : 0.f, keep0 && upper ? p[4] : 0.f,
-                        keep1 && upper ? p[8 * ld + 4] : 0.f};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) split_tf32(v[i], ah[i], al[i]);
-}
+// Entries whose alpha the backward evaluates together (before their serial recurrence).
+template <int PPT>
+__host__ __device__ constexpr int bwd_group() { return PPT == 1 ? 8 : 4; }
 
 // Gradients of the 2D mean (u, v), the conic (a, b, c) and the opacity from the moments
 // M = (sum s, sum s X, sum s Y, sum s X^2, sum s XY, sum s Y^2) of s = dL/dsigma over the
@@ -447,13 +479,8 @@ __device__ __forceinline__ void moment_grads(const float (&M)[6], float U, float
     }
 }
 
-// One pixel per thread and C = 4 or 16: at most 72 registers, so that occupancy is set by
-// shared memory rather than registers (the adjoint is latency-bound and gains from warps):
-// 13 CTAs of an 8 x 8 tile fit both (13 x 64 threads x 72 registers); 64 registers spilled
-// nothing but measured 1 % slower, 80 cost a CTA.  The other widths keep the compiler's
-// choice (with C >= 32 the staged entries hold occupancy lower than registers anyway).
 template <int C, int PPT>
-__host__ __device__ constexpr int bwd_max_regs() { return PPT == 1 && (C == 4 || C == 16) ? 72 : 255; }
+__host__ __device__ constexpr int bwd_max_regs() { return PPT == 1 ? (C <= 16 ? 96 : 128) : 255; }
 
 template <int C, int PPT, bool HALF = false>
 __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterArgs a) {
@@ -463,7 +490,7 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
     constexpr int NT = NFP / 8;                   // 8-feature tiles
     constexpr int NPX = 32 * PPT;                 // pixels of one warp (pixel q = 32 k + lane)
     constexpr int KS = NPX / 8;                   // 8-pixel steps
-    constexpr int MT = NPX / 16;                  // 16-pixel tiles
+    constexpr int GR = bwd_group<PPT>();
     constexpr int WQ = chunk_pitch<NPX>();
     constexpr int GP = g_pitch<NF>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -484,14 +511,14 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
     float4 *s_geo2 = hm ? nullptr : s_geo1 + batch;
     float *s_feat = reinterpret_cast<float *>(s_geo1 + (hm ? batch : 2 * batch));
     uint32_t *s_rec = reinterpret_cast<uint32_t *>(s_feat + (size_t)batch * NF);
-    // half mode: the list position of each staged row, and the queue of pending entries
-    // (list position, record)
-    int *s_pos = reinterpret_cast<int *>(s_rec + batch);
-    int *s_q = s_pos + (hm ? kChunk : 0);
-    uint32_t *s_qr = reinterpret_cast<uint32_t *>(s_q + (hm ? kHalfQueue : 0));
+    // per warp: the list position (half mode) or staged row (shared batches) of each chunk row,
+    // and the queue of pending entries: (list position, record), or staged rows
     const int nthreads = hm ? 32 : a.tile_w * a.tile_h / PPT;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float *s_G = reinterpret_cast<float *>(s_qr + (hm ? kHalfQueue : 0)) + (size_t)warp * bwd_warp_floats<C, PPT>();
+    int *s_pos = reinterpret_cast<int *>(s_rec + batch) + (size_t)warp * bwd_warp_words<C, PPT, HALF>();
+    int *s_q = s_pos + kChunk;
+    uint32_t *s_qr = reinterpret_cast<uint32_t *>(s_q + kHalfQueue);
+    float *s_G = reinterpret_cast<float *>(s_qr + (hm ? kHalfQueue : 0));
     float *s_gw = s_G + NPX * GP;     // per chunk row: gf, then overwritten with w = alpha T
     float *s_sg = s_gw + kChunk * WQ; // per chunk row: s = dL/dsigma
     const int gid = lane >> 2, tig = lane & 3;
@@ -510,6 +537,7 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
     // half mode: a work item is one half tile, or (half_pairs) a whole tile whose halves the
     // warp takes in turn, so that the second half's staging loads can hit L1
     const bool pairs = hm && a.half_pairs;
+    const uint32_t lt = (1u << lane) - 1u;
     const int n_items = hm && !pairs ? 2 * a.n_tiles : a.n_tiles;
     for (int iter = 0;; ++iter) {
         if (!a.persistent && iter > 0) break;
@@ -557,127 +585,121 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
             for (int f = 0; f < NF; f += 4) row[f / 4] = make_float4(g[f], g[f + 1], g[f + 2], g[f + 3]);
         }
         const int warp_last = __reduce_max_sync(SG_FULL_MASK, thread_last);
-        // One chunk of staged rows [jc0, jc0 + 16) (rows past jmax are left out), back to
-        // front; pos_of(j) is the list position of row j.
-        auto chunk = [&](const int jc0, const int jmax, auto pos_of) {
-                // entries of the chunk whose footprint reaches the warp (lane r tests entry jc0 + r)
-                bool cand = false;
-                if (lane < kChunk)
-                    cand = jc0 + lane < jmax && (hm || !wt.misses(s_geo2[jc0 + lane], s_geo1[jc0 + lane], ln_amin));
-                uint32_t cmask = __ballot_sync(SG_FULL_MASK, cand);
-                if (!cmask) return;
-                // ---- gf = G F^T for the chunk (M = pixels, N = entries, K = features) ----
-                if constexpr (MT <= 2) {
-                    // features outside, pixel tiles inside: every F fragment is split once
-                    float d[MT][2][4];
+        __syncwarp();
+        // One chunk of c <= 16 list entries, back to front: chunk row r (ascending list position)
+        // is staged row row_of(r) at list position pos_of(r) (pos_of(r) >= warp_last for r >= c).
+        auto chunk = [&](const int c, auto row_of, auto pos_of) {
+                // ---- gf = F G^T for the chunk (M = entries, N = pixels, K = features) ----
+                // ldmatrix row addresses: lanes 0-15 rows 0-15 of the first four columns, lanes
+                // 16-31 the same rows four columns further (A); lanes 8 m + i row i of matrix m (B)
+                {
+                    const float *fa = s_feat + (size_t)row_of(lane & 15) * NF + 4 * (lane >> 4);
+                    const float *ga = s_G + ((lane & 7) + 8 * (lane >> 4)) * GP + 4 * ((lane >> 3) & 1);
+                    float d[KS][4];
 #pragma unroll
-                    for (int mt = 0; mt < MT; ++mt)
+                    for (int nt = 0; nt < KS; ++nt) d[nt][0] = d[nt][1] = d[nt][2] = d[nt][3] = 0.f;
 #pragma unroll
-                        for (int nt = 0; nt < 2; ++nt) d[mt][nt][0] = d[mt][nt][1] = d[mt][nt][2] = d[mt][nt][3] = 0.f;
+                    for (int kk = 0; kk < NF / 8; ++kk) {
+                        uint32_t ar[4], ah[4], al[4];
+                        ldsm_x4(fa + 8 * kk, ar);
 #pragma unroll
-                    for (int kk = 0; kk < NT; ++kk) {
-                        const int f0 = 8 * kk + tig;
-                        uint32_t bh[2][2], bl[2][2];
+                        for (int i = 0; i < 4; ++i) split_tf32(__uint_as_float(ar[i]), ah[i], al[i]);
 #pragma unroll
-                        for (int nt = 0; nt < 2; ++nt) {
-                            const float *fr = s_feat + (size_t)(jc0 + 8 * nt + gid) * NF;
-                            split_tf32(f0 < NF ? fr[f0] : 0.f, bh[nt][0], bl[nt][0]);
-                            split_tf32(f0 + 4 < NF ? fr[f0 + 4] : 0.f, bh[nt][1], bl[nt][1]);
-                        }
+                        for (int n2 = 0; n2 < KS / 2; ++n2) {
+                            uint32_t br[4], bh[4], bl[4];
+                            ldsm_x4(ga + 16 * n2 * GP + 8 * kk, br);
 #pragma unroll
-                        for (int mt = 0; mt < MT; ++mt) {
-                            uint32_t ah[4], al[4];
-                            load_a_split(s_G + 16 * mt * GP, GP, 8 * kk, gid, tig, true, true, ah, al,
-                                         8 * kk + 4 < NF);
-#pragma unroll
-                            for (int nt = 0; nt < 2; ++nt)
-                                mma_tf32x3(d[mt][nt], ah, al, bh[nt][0], bh[nt][1], bl[nt][0], bl[nt][1]);
+                            for (int i = 0; i < 4; ++i) split_tf32(__uint_as_float(br[i]), bh[i], bl[i]);
+                            mma_tf32x3(d[2 * n2], ah, al, bh[0], bh[1], bl[0], bl[1]);
+                            mma_tf32x3(d[2 * n2 + 1], ah, al, bh[2], bh[3], bl[2], bl[3]);
                         }
                     }
+                    if constexpr (NF % 8 != 0) {
+                        // the last four features: K = 4 products
+                        const float *f4 = s_feat + (size_t)row_of(lane & 15) * NF + 8 * (NF / 8);
+                        uint32_t ar[2], ah[2], al[2];
+                        ldsm_x2(f4, ar[0], ar[1]);
 #pragma unroll
-                    for (int mt = 0; mt < MT; ++mt)
+                        for (int i = 0; i < 2; ++i) split_tf32(__uint_as_float(ar[i]), ah[i], al[i]);
 #pragma unroll
-                        for (int nt = 0; nt < 2; ++nt)
+                        for (int n4 = 0; n4 < KS / 4; ++n4) {
+                            uint32_t br[4];
+                            ldsm_x4(s_G + (32 * n4 + lane) * GP + 8 * (NF / 8), br);
 #pragma unroll
-                            for (int i = 0; i < 4; ++i)
-                                s_gw[(8 * nt + 2 * tig + (i & 1)) * WQ + 16 * mt + gid + 8 * (i >> 1)] = d[mt][nt][i];
-                } else
-#pragma unroll 1
-                for (int mt = 0; mt < MT; ++mt) {
-                    float d[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll
-                    for (int kk = 0; kk < NT; ++kk) {
-                        // B (8 x 8): b0 (tig, gid), b1 (tig + 4, gid) = F[entry][feature]
-                        const int f0 = 8 * kk + tig;
-                        uint32_t ah[4], al[4];
-                        load_a_split(s_G + 16 * mt * GP, GP, 8 * kk, gid, tig, true, true, ah, al,
-                                     8 * kk + 4 < NF);
-#pragma unroll
-                        for (int nt = 0; nt < 2; ++nt) {
-                            const float *fr = s_feat + (size_t)(jc0 + 8 * nt + gid) * NF;
-                            uint32_t bh0, bl0, bh1, bl1;
-                            split_tf32(f0 < NF ? fr[f0] : 0.f, bh0, bl0);
-                            split_tf32(f0 + 4 < NF ? fr[f0 + 4] : 0.f, bh1, bl1);
-                            mma_tf32x3(d[nt], ah, al, bh0, bh1, bl0, bl1);
+                            for (int i = 0; i < 4; ++i) {
+                                uint32_t bh, bl;
+                                split_tf32(__uint_as_float(br[i]), bh, bl);
+                                mma_tf32x3_k4(d[4 * n4 + i], ah, al, bh, bl);
+                            }
                         }
                     }
-                    // D (16 x 8): d0 (gid, 2 tig), d1 (gid, 2 tig + 1), d2 (gid + 8, 2 tig), d3 (gid + 8, 2 tig + 1)
+                    // D (16 x 8): d0, d1 (gid, 2 tig + 0 / 1), d2, d3 (gid + 8, ..)
 #pragma unroll
-                    for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            s_gw[(8 * nt + 2 * tig + (i & 1)) * WQ + 16 * mt + gid + 8 * (i >> 1)] = d[nt][i];
+                    for (int nt = 0; nt < KS; ++nt) {
+                        *reinterpret_cast<float2 *>(s_gw + gid * WQ + 8 * nt + 2 * tig) = make_float2(d[nt][0], d[nt][1]);
+                        *reinterpret_cast<float2 *>(s_gw + (gid + 8) * WQ + 8 * nt + 2 * tig) =
+                            make_float2(d[nt][2], d[nt][3]);
+                    }
                 }
                 __syncwarp();
-                // ---- back to front over the candidates: T, dL/dalpha, w and s per pixel ----
-                uint32_t mask = 0;
-                while (cmask) {
-                    const int r = 31 - __clz(cmask);
-                    cmask &= ~(1u << r);
-                    const int j = jc0 + r;
-                    const float4 g0 = s_geo0[j];
-                    const float4 g1 = s_geo1[j];
-                    const int pos = pos_of(j);
-                    AlphaEval e[PPT];
-                    bool hit[PPT];
-                    bool any = false;
+                // ---- back to front, GR entries at a time: first every alpha of the group (no
+                // dependence between entries), then the recurrence in T and a ----
+                uint32_t hits = 0;  // rows that contribute to one of the lane's pixels
+#pragma unroll 1
+                for (int rg = (c - 1) / GR * GR; rg >= 0; rg -= GR) {
+                    float al[PPT][GR];  // 0: no contribution
+                    uint32_t hb = 0;
 #pragma unroll
-                    for (int k = 0; k < PPT; ++k) {
-                        hit[k] = pos < my_last[k] &&
-                                 eval_alpha(fx - g0.x, (float)(wt.ly + 4 * k) - g0.y, g0.z, g0.w, g1.x, g1.y, g1.z,
-                                            g1.w, a.alpha_max, a.alpha_min, e[k]);
-                        any |= hit[k];
-                    }
-                    if (!__any_sync(SG_FULL_MASK, any)) continue;
-                    mask |= 1u << r;
+                    for (int i = 0; i < GR; ++i) {
+                        const int j = row_of(rg + i), pos = pos_of(rg + i);
+                        const float4 g0 = s_geo0[j];
+                        const float4 g1 = s_geo1[j];
 #pragma unroll
-                    for (int k = 0; k < PPT; ++k) {
-                        float *gw = s_gw + r * WQ + 32 * k + lane;
-                        float w = 0.f, sg = 0.f;
-                        if (hit[k]) {
-                            const float gf = *gw;
-                            // transmittance before this Gaussian (only gradients depend on it)
-                            T[k] = __fdividef(T[k], __fsub_rn(1.f, e[k].alpha));
-                            const float dalpha = T[k] * (gf - acc_a[k]);
-                            acc_a[k] = e[k].alpha * gf + (1.f - e[k].alpha) * acc_a[k];
-                            w = e[k].alpha * T[k];
-                            if (e[k].raw < a.alpha_max) sg = -dalpha * e[k].raw;
+                        for (int k = 0; k < PPT; ++k) {
+                            AlphaEval e;
+                            const bool hit = eval_alpha(fx - g0.x, (float)(wt.ly + 4 * k) - g0.y, g0.z, g0.w, g1.x,
+                                                        g1.y, g1.z, g1.w, a.alpha_max, a.alpha_min, e) &&
+                                             pos < my_last[k];
+                            al[k][i] = hit ? e.alpha : 0.f;
+                            if (hit) hb |= 1u << i;
                         }
-                        *gw = w;
-                        s_sg[r * WQ + 32 * k + lane] = sg;
+                    }
+                    hits |= hb << rg;
+#pragma unroll
+                    for (int i = GR - 1; i >= 0; --i) {
+                        float *gw = s_gw + (rg + i) * WQ + lane;
+#pragma unroll
+                        for (int k = 0; k < PPT; ++k) {
+                            const float A = al[k][i], om = 1.f - A;
+                            // (a pixel without a contribution keeps T and a: A = 0, gf taken as 0)
+                            const float gf = A > 0.f ? gw[32 * k] : 0.f;
+                            // transmittance before this Gaussian (only gradients depend on it)
+                            T[k] *= rcp_fast(om);
+                            const float dalpha = T[k] * (gf - acc_a[k]);
+                            acc_a[k] = fmaf(om, acc_a[k], A * gf);
+                            gw[32 * k] = A * T[k];
+                            // (alpha = alpha_max: clamped, no gradient; else alpha = o G)
+                            s_sg[(rg + i) * WQ + 32 * k + lane] = A < a.alpha_max ? -dalpha * A : 0.f;
+                        }
                     }
                 }
+                const uint32_t mask = __reduce_or_sync(SG_FULL_MASK, hits);
                 if (!mask) return;  // (warp-uniform)
                 __syncwarp();
                 // ---- dF = W G (M = entries, N = features, K = pixels), moments M = S P ----
+                // (rows without a contribution may hold stale values: they are not written out)
                 const bool keep0 = (mask >> gid) & 1u, keep1 = (mask >> (gid + 8)) & 1u;
+                const float *wa = s_gw + (lane & 15) * WQ + 4 * (lane >> 4);
+                const float *sa = s_sg + (lane & 15) * WQ + 4 * (lane >> 4);
                 float df[NT][4], mom[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                 for (int nt = 0; nt < NT; ++nt) df[nt][0] = df[nt][1] = df[nt][2] = df[nt][3] = 0.f;
 #pragma unroll
                 for (int ks = 0; ks < KS; ++ks) {
-                    uint32_t ah[4], al[4];
-                    load_a_split(s_gw, WQ, 8 * ks, gid, tig, keep0, keep1, ah, al);
+                    uint32_t ar[4], ah[4], al[4];
+                    ldsm_x4(wa + 8 * ks, ar);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) split_tf32(__uint_as_float(ar[i]), ah[i], al[i]);
 #pragma unroll
                     for (int nt = 0; nt < NT; ++nt) {
                         // B (8 x 8): b0 (tig, gid), b1 (tig + 4, gid) = G[pixel][feature]
@@ -688,7 +710,9 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
                         split_tf32(stored ? gp[4 * GP] : 0.f, bh1, bl1);
                         mma_tf32x3(df[nt], ah, al, bh0, bh1, bl0, bl1);
                     }
-                    load_a_split(s_sg, WQ, 8 * ks, gid, tig, keep0, keep1, ah, al);
+                    ldsm_x4(sa + 8 * ks, ar);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) split_tf32(__uint_as_float(ar[i]), ah[i], al[i]);
                     const float Y = (float)((ks & 3) + 4 * (ks >> 2)) - (2.f * PPT - 0.5f);
                     const uint32_t pb0 = __float_as_uint(fmaf(Y, fmaf(Y, P2, P1a), P0a));
                     const uint32_t pb1 = __float_as_uint(fmaf(Y, fmaf(Y, P2, P1b), P0b));
@@ -699,7 +723,7 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
 #pragma unroll
                 for (int hr = 0; hr < 2; ++hr) {
                     if (!(hr ? keep1 : keep0)) continue;
-                    const uint32_t rec = s_rec[jc0 + gid + 8 * hr];
+                    const uint32_t rec = s_rec[row_of(gid + 8 * hr)];
                     const uint32_t gi = rec - rec_base;
                     const size_t si = (size_t)C * (a.sem_rec ? rec : gi);
 #pragma unroll
@@ -739,15 +763,14 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
 #pragma unroll
                     for (int hr = 0; hr < 2; ++hr) {
                         if (!(hr ? keep1 : keep0)) continue;
-                        const int j = jc0 + gid + 8 * hr;
+                        const int j = row_of(gid + 8 * hr);
                         const float4 g0 = s_geo0[j];
                         const float4 g1 = s_geo1[j];
                         const float U = (g0.x - wt.cxw) + g0.z, V = (g0.y - wt.cyw) + g0.w;
                         float r0, r1;
                         moment_grads(Mr[hr], U, V, g1, tig, r0, r1);
-                        float *dst = a.g2d + 8 * (size_t)s_rec[j] + 2 * tig;
-                        atomicAdd(dst, r0);
-                        atomicAdd(dst + 1, r1);
+                        // (records are 32 bytes of the 16-byte aligned workspace)
+                        red_add_v2(a.g2d + 8 * (size_t)s_rec[j] + 2 * tig, r0, r1);
                     }
                 }
                 __syncwarp();  // the chunk buffers are rewritten next
@@ -766,16 +789,38 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
                 load_batch<NF>(a, C, range.x, b0, cnt, ti.px0, ti.py0, rec_base, s_geo0, s_geo1, s_geo2, s_feat,
                                s_rec, nthreads);
                 __syncthreads();
+                // rows of the batch whose footprint reaches the warp's pixels, back to front: (the
+                // exact ellipse test, 32 rows at a time), processed 16 at a time
                 const int jmax = min(cnt, warp_last - b0);  // warp-uniform
-                for (int jc0 = jmax > 0 ? (jmax - 1) & ~(kChunk - 1) : -kChunk; jc0 >= 0; jc0 -= kChunk)
-                    chunk(jc0, jmax, [b0](int j) { return b0 + j; });
+                int qn = 0;
+                for (int top = jmax; top > 0 || qn > 0;) {
+                    while (qn < kChunk && top > 0) {
+                        const int j = top - 1 - lane;
+                        const bool sel = j >= 0 && !wt.misses(s_geo2[j], s_geo1[j], ln_amin);
+                        const uint32_t bal = __ballot_sync(SG_FULL_MASK, sel);
+                        if (sel) s_q[qn + __popc(bal & lt)] = j;
+                        qn += __popc(bal);
+                        top -= 32;
+                    }
+                    if (qn == 0) break;
+                    __syncwarp();
+                    const int c = min(kChunk, qn);
+                    // chunk row r is queue entry c - 1 - r; rows past c stay out of reach
+                    if (lane < kChunk) s_pos[lane] = lane < c ? s_q[c - 1 - lane] : 0;
+                    const int rest = qn - c;  // (< 32)
+                    const int keep = lane < rest ? s_q[c + lane] : 0;
+                    __syncwarp();
+                    if (lane < rest) s_q[lane] = keep;
+                    qn = rest;
+                    chunk(c, [s_pos](int r) { return s_pos[r]; },
+                          [s_pos, b0, c](int r) { return r < c ? b0 + s_pos[r] : 0x7fffffff; });
+                }
             }
             __syncthreads();
         } else {
             // list positions < warp_last whose half mask holds this half, in descending order:
             // (s_q, s_qr)[0 .. qn) is the queue of (position, record), top the next position
             // scanned (exclusive)
-            const uint32_t lt = (1u << lane) - 1u;
             int top = warp_last, qn = 0;
             for (;;) {
                 while (qn < kChunk && top > 0) {
@@ -801,7 +846,7 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
                 // rows 0 .. c-1 in ascending list position: row r is queue entry c - 1 - r
                 stage_rows_warp<NF>(a, C, [&](int j) { return s_qr[c - 1 - j]; }, c, ti.px0, ti.py0, rec_base, s_geo0,
                                     s_geo1, s_geo2, s_feat, s_rec);
-                if (lane < c) s_pos[lane] = s_q[c - 1 - lane];
+                if (lane < kChunk) s_pos[lane] = lane < c ? s_q[c - 1 - lane] : 0x7fffffff;
                 const int rest = qn - c;  // (< 32)
                 const int keep = lane < rest ? s_q[c + lane] : 0;
                 const uint32_t keep_rec = lane < rest ? s_qr[c + lane] : 0u;
@@ -812,7 +857,7 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
                 }
                 qn = rest;
                 __syncwarp();
-                chunk(0, c, [s_pos](int j) { return s_pos[j]; });
+                chunk(c, [](int r) { return r; }, [s_pos](int r) { return s_pos[r]; });
             }
             __syncwarp();
         }
@@ -828,14 +873,13 @@ inline size_t fwd_smem(int batch) {
 }
 template <int C, int PPT>
 inline size_t bwd_smem(int batch, int threads) {
-    return fwd_smem<C>(batch) + (size_t)batch * 4 + sizeof(float) * (threads / 32) * bwd_warp_floats<C, PPT>();
+    return fwd_smem<C>(batch) + (size_t)batch * 4 + sizeof(float) * (threads / 32) * bwd_warp_words<C, PPT, false>();
 }
 // half mode: one 16-entry chunk staged without its (u, v, ex, ey) rows (+ its list positions),
 // the (position, record) queue, one warp
 template <int C>
 inline size_t bwd_half_smem() {
-    return fwd_smem<C>(kChunk) - (size_t)kChunk * 16 + (size_t)kChunk * 4 * 2 + (size_t)kHalfQueue * 4 * 2 +
-           sizeof(float) * bwd_warp_floats<C, 1>();
+    return fwd_smem<C>(kChunk) - (size_t)kChunk * 16 + (size_t)kChunk * 4 + sizeof(float) * bwd_warp_words<C, 1, true>();
 }
 
 // forward half mode: one 32-entry chunk staged without its (u, v, ex, ey) rows, and the

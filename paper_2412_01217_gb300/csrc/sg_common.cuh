@@ -136,6 +136,42 @@ __device__ __forceinline__ void mma_tf32x3(float (&d)[4], const uint32_t (&ah)[4
     mma_tf32(d, ah, bh0, bh1);
 }
 
+// The same with four-deep operands (m16n8k4): A (16 x 4) a0 (gid, tig), a1 (gid + 8, tig);
+// B (4 x 8) b0 (tig, gid).
+__device__ __forceinline__ void mma_tf32_k4(float (&d)[4], const uint32_t (&a)[2], uint32_t b) {
+    asm(
+        "mma.sync.aligned.m16n8k4.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};\n"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(b));
+}
+__device__ __forceinline__ void mma_tf32x3_k4(float (&d)[4], const uint32_t (&ah)[2], const uint32_t (&al)[2],
+                                              uint32_t bh, uint32_t bl) {
+    mma_tf32_k4(d, al, bh);
+    mma_tf32_k4(d, ah, bl);
+    mma_tf32_k4(d, ah, bh);
+}
+
+// 32-bit operand tiles through ldmatrix: an 8 x 4 tile of 32-bit words is an 8 x 8 tile of
+// 16-bit halves, and thread t receives the word at row t / 4, column t % 4 of each tile, the
+// (gid, tig) element of the fragments above.  Lane 8 m + i gives the (16-byte aligned)
+// address of row i of tile m.
+__device__ __forceinline__ void ldsm_x2(const float *p, uint32_t &r0, uint32_t &r1) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];\n" : "=r"(r0), "=r"(r1) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ldsm_x4(const float *p, uint32_t (&r)[4]) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+
+// 1 / x, approximate (x normal; 1 ulp, exact for 1)
+__device__ __forceinline__ float rcp_fast(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;\n" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // Two float additions to consecutive, 8-byte aligned addresses in one vector reduction.
 __device__ __forceinline__ void red_add_v2(float *addr, float a, float b) {
     asm volatile("red.global.add.v2.f32 [%0], {%1, %2};\n" ::"l"(addr), "f"(a), "f"(b) : "memory");
