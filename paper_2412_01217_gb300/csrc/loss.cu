@@ -509,15 +509,6 @@ __host__ __device__ constexpr int ce_mma_smem_floats() {
     return CeLayout<C, K>::W_FLOATS + (kLossThreads / 32) * (CeLayout<C, K>::WARP_FLOATS + CeLayout<C, K>::STAGE_FLOATS);
 }
 
-// 4-byte asynchronous copy global -> shared (zero-filled when !valid; src must still be a
-// mapped address), and its group fences.
-__device__ __forceinline__ void cp_async4(void *dst, const void *src, bool valid) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all_groups() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
 // Two CTAs per SM (up to 128 registers): with the per-warp stage, three CTAs at 80 registers
 // spilled the warp's fragments and measured slower (loss 0.975 against 0.954 ms on the batched
 // workload), and four at 64 slower still.
@@ -597,7 +588,7 @@ __global__ void __launch_bounds__(kLossThreads, 2) ce_decoder_mma_kernel(PixelAr
         const int v = x.v, HW = x.HW, pw = x.pw;
         const size_t p0 = x.p0;
         const int nd = a.counts[2 * v], nl = a.counts[2 * v + 1];
-        cp_async_wait_all_groups();
+        cp_async_wait_groups<0>();
         __syncwarp();
         float l1d = 0.f, ce = 0.f;
         {

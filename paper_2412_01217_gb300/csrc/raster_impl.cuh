@@ -66,43 +66,73 @@ __device__ __forceinline__ void load_batch(const RasterArgs &a, int C, int list_
         if (s_rec) s_rec[j] = rec;
     }
 }
-// The same rows for one warp and at most 32 entries whose records are known (rec_of(j) is
-// row j's record): lanes 0-15 stage the geometry of rows lane, lane + 16, lanes 16-31 their
-// features.  s_geo2 and s_rec may be null (not staged).
-template <int NF, class RecOf>
-__device__ __forceinline__ void stage_rows_warp(const RasterArgs &a, int C, RecOf rec_of, int cnt, int px0,
-                                                int py0, uint32_t rec_base, float4 *s_geo0, float4 *s_geo1,
-                                                float4 *s_geo2, float *s_feat, uint32_t *s_rec) {
-    const int lane = threadIdx.x & 31;
-    for (int j = lane & 15; j < cnt; j += 16) {
-        const uint32_t rec = rec_of(j);
-        float *f = s_feat + (size_t)j * NF;
-        if (lane < 16) {
-            const float4 g0 = a.geo[2 * (size_t)rec];
-            const float4 g1 = a.geo[2 * (size_t)rec + 1];
-            const uint32_t packed = __float_as_uint(g1.w);
-            const float uI = (float)((int)(short)(packed & 0xffffu) - px0);
-            const float vI = (float)((int)(short)(packed >> 16) - py0);
-            s_geo0[j] = make_float4(uI, vI, g0.x, g0.y);
-            s_geo1[j] = make_float4(g1.x, g1.y, g1.z, g0.w);
-            if (s_geo2) {
-                const float2 ex = a.ext[rec];
-                s_geo2[j] = make_float4(uI + g0.x, vI + g0.y, ex.x, ex.y);
-            }
-            if (s_rec) s_rec[j] = rec;
-            f[3] = g0.z;  // depth (camera z of the mean, Eq. 8)
-        } else {
-            const uint32_t gi = rec - rec_base;
-            const size_t ci = a.col_rec ? rec : gi;
-            f[0] = a.rgb[3 * ci];
-            f[1] = a.rgb[3 * ci + 1];
-            f[2] = a.rgb[3 * ci + 2];
-            const float4 *s4 = reinterpret_cast<const float4 *>(a.sem + (size_t)(a.sem_rec ? rec : gi) * C);
-            float4 *f4 = reinterpret_cast<float4 *>(f + 4);
+
+// Features of a warp's 16 chunk rows into s_feat by asynchronous copies: colour into f[0..2],
+// semantics into f[4..]; f[3] (the depth) is left to the caller.  Lanes r and r + 16 copy row r
+// (record rec), half of its words each.
+template <int NF>
+__device__ __forceinline__ void stage_features_async(const RasterArgs &a, uint32_t rec, uint32_t rec_base,
+                                                     float *s_feat) {
+    constexpr int C = NF - 4, NS = C / 4;
+    const int lane = threadIdx.x & 31, h = lane >> 4;
+    float *f = s_feat + (lane & 15) * NF;
+    const float *sem = a.sem + (size_t)(a.sem_rec ? rec : rec - rec_base) * C;
+    const float *rgb = a.rgb + 3 * (size_t)(a.col_rec ? rec : rec - rec_base);
 #pragma unroll
-            for (int k = 0; k < (NF - 4) / 4; ++k) f4[k] = s4[k];
+    for (int q = 0; q < (NS + 1) / 2; ++q)
+        if (2 * q + h < NS) cp_async16(f + 4 + 4 * (2 * q + h), sem + 4 * (2 * q + h));
+    cp_async4(f + h, rgb + h, true);
+    if (h) cp_async4(f + 2, rgb + 2, true);
+}
+
+// One list entry's geometry, relative to the tile: integer part (exact in float) and float
+// fraction of the 2D mean, the conic form and the opacity.
+struct EntryGeo {
+    float ui, vi, uf, vf, m00, m10, m11, o;
+};
+__device__ __forceinline__ EntryGeo entry_geo(const float4 &g0, const float4 &g1) {  // staged rows
+    return {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+}
+__device__ __forceinline__ EntryGeo record_geo(const float4 &g0, const float4 &g1, int px0, int py0) {
+    const uint32_t packed = __float_as_uint(g1.w);
+    return {(float)((int)(short)(packed & 0xffffu) - px0), (float)((int)(short)(packed >> 16) - py0), g0.x, g0.y,
+            g1.x, g1.y, g1.z, g0.w};
+}
+
+// Alphas of a chunk of 16 entries at the warp's 32 PPT pixels.  Lane l evaluates entry l % 16
+// at the four columns x0 .. x0 + 3 (x0 = lx0, the left or the right half of the sub-tile by
+// l / 16) of every row ly0 .. ly0 + 4 PPT - 1, so that dx and its square terms are formed once
+// per column and dy once per row, and writes alpha (0 below alpha_min) to
+// s_A[pixel * kAPitch + entry]; pixel 32 k + lane then reads its 16 alphas back as float4s.
+// With a lane per pixel instead, every entry's eight geometry floats would be broadcast to all
+// lanes through shared memory (8 data-pipe cycles per entry and warp), which bound both
+// kernels (l1tex data pipe 80 % busy).  kAPitch: rows of 16 plus 4, conflict-free both ways.
+// Returns whether the entry contributes to any of the lane's pixels.
+constexpr int kAPitch = 20;
+template <int PPT>
+__device__ __forceinline__ bool chunk_alphas(const EntryGeo &g, float lx0, float ly0, float alpha_max, float alpha_min,
+                                             float *s_A) {
+    const int lane = threadIdx.x & 31;
+    float *out = s_A + 4 * (lane >> 4) * kAPitch + (lane & 15);
+    float dx[4], p1[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        dx[c] = __fsub_rn(__fsub_rn(lx0 + (float)c, g.ui), g.uf);
+        const float p = __fmul_rn(g.m00, dx[c]);
+        p1[c] = __fmul_rn(p, p);
+    }
+    float top = 0.f;
+#pragma unroll
+    for (int r = 0; r < 4 * PPT; ++r) {
+        const float q = __fmul_rn(g.m11, __fsub_rn(__fsub_rn(ly0 + (float)r, g.vi), g.vf));
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float al = entry_alpha(g.m10, dx[c], q, p1[c], g.o, alpha_max, alpha_min);
+            out[(8 * r + c) * kAPitch] = al;
+            top = fmaxf(top, al);
         }
     }
+    return top > 0.f;
 }
 
 // Persistent work queue: work_counter[0] hands out slots, work_counter[1] counts the CTAs
@@ -184,56 +214,120 @@ __device__ __forceinline__ TileInfo tile_info(const RasterArgs &a, int item) {
     return t;
 }
 
+// Both kernels work on chunks of 16 consecutive entries of a warp's list.
+constexpr int kChunk = 16;
+// Ring of pending entries of a warp (< 16 pending + one 32-entry scan).
+constexpr int kRing = 64;
+
 // Half mode of the forward (8 x 8 tiles, one pixel per thread, lists with half masks): a
 // CTA is one warp that owns one half (8 x 4 pixels) of a tile; it walks the tile's list front
-// to back, queues (position, record) of the entries whose mask holds its half, and stages and
-// composites them 32 at a time with no block barrier, stopping as soon as its own 32 pixels
-// are saturated.  The per-pixel sequence of contributing entries, and so the output, is the
-// same as with shared batches.
-constexpr int kFwdHalfChunk = 32;
-constexpr int kFwdHalfQueue = kFwdHalfChunk + 32;  // < kFwdHalfChunk pending + one 32-entry scan
+// to back, queues (position, record) of the entries whose mask holds its half, and composites
+// them 16 at a time with no block barrier, stopping as soon as its own 32 pixels are
+// saturated; the next chunk's geometry (registers) and features (asynchronous copies into the
+// other of two buffers) are requested before the current one is composited.  The per-pixel
+// sequence of contributing entries, and so the output, is the same as with shared batches.
 
-// acc[0 .. 3] += w f where w != 0 (a lane without a contribution takes nothing from a
-// non-finite feature), predicated instead of branched around: the four entries of a group
-// then share one instruction stream and their loads and sums overlap.
-__device__ __forceinline__ void fma4_if(float *acc, float w, const float4 &f) {
-    asm("{\n\t.reg .pred p;\n\tsetp.ne.f32 p, %4, 0f00000000;\n\t"
-        "@p fma.rn.f32 %0, %4, %5, %0;\n\t@p fma.rn.f32 %1, %4, %6, %1;\n\t"
-        "@p fma.rn.f32 %2, %4, %7, %2;\n\t@p fma.rn.f32 %3, %4, %8, %3;\n}\n"
-        : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3])
-        : "f"(w), "f"(f.x), "f"(f.y), "f"(f.z), "f"(f.w));
+// acc[i] += w f[i] where w != 0 (a pixel without a contribution takes nothing from a
+// non-finite feature)
+template <int N>
+__device__ __forceinline__ void fma_if(float *acc, float w, const float *f) {
+    if constexpr (N >= 5) {
+        asm("{\n\t.reg .pred p;\n\tsetp.ne.f32 p, %5, 0f00000000;\n\t"
+            "@p fma.rn.f32 %0, %5, %6, %0;\n\t@p fma.rn.f32 %1, %5, %7, %1;\n\t@p fma.rn.f32 %2, %5, %8, %2;\n\t"
+            "@p fma.rn.f32 %3, %5, %9, %3;\n\t@p fma.rn.f32 %4, %5, %10, %4;\n}\n"
+            : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3]), "+f"(acc[4])
+            : "f"(w), "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]), "f"(f[4]));
+        fma_if<N - 5>(acc + 5, w, f + 5);
+    } else if constexpr (N == 4) {
+        asm("{\n\t.reg .pred p;\n\tsetp.ne.f32 p, %4, 0f00000000;\n\t"
+            "@p fma.rn.f32 %0, %4, %5, %0;\n\t@p fma.rn.f32 %1, %4, %6, %1;\n\t@p fma.rn.f32 %2, %4, %7, %2;\n\t"
+            "@p fma.rn.f32 %3, %4, %8, %3;\n}\n"
+            : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3])
+            : "f"(w), "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]));
+    } else if constexpr (N >= 1) {
+        asm("{\n\t.reg .pred p;\n\tsetp.ne.f32 p, %1, 0f00000000;\n\t@p fma.rn.f32 %0, %1, %2, %0;\n}\n"
+            : "+f"(acc[0])
+            : "f"(w), "f"(f[0]));
+        fma_if<N - 1>(acc + 1, w, f + 1);
+    }
 }
 
-template <int N>
-struct IntC {
-    static constexpr int value = N;
+// The four lanes of a quad share the feature sums of their pixels: lane s of the quad sums a
+// quarter of the channels (one of r, g, b, depth; sem[16 q + 4 s ..], then sem[16 (C / 16) +
+// (C % 16) / 4 s ..]) at all four pixels, whose weights it takes by shuffles.  Every feature is
+// then loaded by one lane in four, a quarter of the shared-memory traffic of a lane that sums
+// every channel of its own pixel; each pixel and channel still sums its entries in list order.
+template <int C>
+struct QuadChannels {
+    static constexpr int NQ = C / 16, REM = C % 16 / 4, N = 1 + 4 * NQ + REM;
+    static __device__ __forceinline__ void load(const float *row, int s, float (&f)[N]) {
+        f[0] = row[s];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const float4 t = *reinterpret_cast<const float4 *>(row + 4 + 16 * q + 4 * s);
+            f[1 + 4 * q] = t.x; f[2 + 4 * q] = t.y; f[3 + 4 * q] = t.z; f[4 + 4 * q] = t.w;
+        }
+        if constexpr (REM == 2) {
+            const float2 t = *reinterpret_cast<const float2 *>(row + 4 + 16 * NQ + 2 * s);
+            f[1 + 4 * NQ] = t.x; f[2 + 4 * NQ] = t.y;
+        } else if constexpr (REM == 1) {
+            f[1 + 4 * NQ] = row[4 + 16 * NQ + s];
+        }
+    }
+    // semantic channel of f[1 + i]
+    static __device__ __forceinline__ int sem(int i, int s) {
+        return i < 4 * NQ ? 16 * (i / 4) + 4 * s + i % 4 : 16 * NQ + REM * s + i - 4 * NQ;
+    }
 };
 
-// Entries whose alpha the forward evaluates together (before their serial recurrence).
-template <int PPT>
-__host__ __device__ constexpr int fwd_group() { return PPT == 1 ? 4 : 2; }
+// v[0 .. 3] to the pixels x .. x + 3 of a row (p points at x; those from n_in on are outside)
+__device__ __forceinline__ void store_quad(float *p, const float (&v)[4], int n_in) {
+    if (n_in >= 4 && ((uintptr_t)p & 15) == 0) {
+        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (j < n_in) p[j] = v[j];
+    }
+}
+
+// shared memory of one forward warp (4-byte words): the ring (rows, or positions and records),
+// the chunk's rows (or positions), the alphas, and in half mode two feature buffers
+template <int C, int PPT, bool HALF>
+__host__ __device__ constexpr int fwd_warp_words() {
+    return (HALF ? 2 : 1) * kRing + kChunk + 32 * PPT * kAPitch + (HALF ? 2 * kChunk * (4 + C) : 0);
+}
+
+// One pixel per thread, C <= 16: 80 registers, i.e. 25 one-warp CTAs per SM in half mode (batched
+// workload: 1151 us at 80, 1216 at 72, 1286 at 64 with spills, 1232 at the compiler's 99).
+template <int C, int PPT>
+__host__ __device__ constexpr int fwd_max_regs() { return PPT == 1 ? (C <= 16 ? 80 : 128) : PPT == 2 ? 168 : 255; }
 
 template <int C, int PPT, bool HALF = false>
-__global__ void __launch_bounds__(kMaxTileThreads) raster_fwd_kernel(RasterArgs a) {
+__global__ void __launch_bounds__(kMaxTileThreads) __maxnreg__((fwd_max_regs<C, PPT>())) raster_fwd_kernel(RasterArgs a) {
     pdl_begin();
     constexpr int NF = 4 + C;
-    constexpr int GF = fwd_group<PPT>();
+    using QC = QuadChannels<C>;
     constexpr bool hm = HALF;
     static_assert(!HALF || PPT == 1, "half mode runs one pixel per thread");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_item;
-    const int batch = hm ? kFwdHalfChunk : a.batch;
+    const int batch = hm ? 0 : a.batch;
     float4 *s_geo0 = reinterpret_cast<float4 *>(smem_raw);
     float4 *s_geo1 = s_geo0 + batch;
-    float4 *s_geo2 = hm ? nullptr : s_geo1 + batch;
-    float *s_feat = reinterpret_cast<float *>(s_geo1 + (hm ? batch : 2 * batch));
-    int *s_q = reinterpret_cast<int *>(s_feat + (size_t)batch * NF);  // half mode: the queue
-    uint32_t *s_qr = reinterpret_cast<uint32_t *>(s_q + kFwdHalfQueue);
+    float4 *s_geo2 = s_geo1 + batch;
+    float *s_feat = reinterpret_cast<float *>(s_geo2 + batch);
     const int nthreads = hm ? 32 : a.tile_w * a.tile_h / PPT;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane & 3;
+    int *s_q = reinterpret_cast<int *>(s_feat + (size_t)batch * NF) + (size_t)warp * fwd_warp_words<C, PPT, HALF>();
+    uint32_t *s_qr = reinterpret_cast<uint32_t *>(s_q + kRing);  // (half mode)
+    int *s_row = s_q + (hm ? 2 : 1) * kRing;
+    float *s_A = reinterpret_cast<float *>(s_row + kChunk);
+    float *s_hf = s_A + 32 * PPT * kAPitch;  // half mode: 2 x 16 feature rows
     const WarpTile<PPT> wt(a.tile_w);
-    const float fx = (float)wt.lx;
     const float ln_amin = __logf(a.alpha_min);
+    const float ax = (float)(wt.lx - (lane & 7) + 4 * (lane >> 4)), ay = (float)(wt.ly - (lane >> 3));
+    const uint32_t lt = (1u << lane) - 1u;
     const int n_items = hm ? 2 * a.n_tiles : a.n_tiles;
     for (int iter = 0;; ++iter) {
         if (!a.persistent && iter > 0) break;
@@ -248,166 +342,219 @@ __global__ void __launch_bounds__(kMaxTileThreads) raster_fwd_kernel(RasterArgs 
         const int2 range = a.ranges[item];
         const int n = range.y - range.x;
         const uint32_t rec_base = (uint32_t)ti.v * (uint32_t)a.N;
-        float acc[PPT][NF];
-        float T[PPT];
+        float acc[PPT][4][QC::N];  // [k][x]: the lane's channels at the pixel of lane ^ x
+        float T[PPT], Tl[PPT];  // transmittance; the same while the pixel is live, then -1
         int last[PPT], nc[PPT];
-        bool done[PPT];
-        int n_done = 0;
 #pragma unroll
         for (int k = 0; k < PPT; ++k) {
-            const int py = ti.py0 + wt.ly + 4 * k;
 #pragma unroll
-            for (int c = 0; c < NF; ++c) acc[k][c] = 0.f;
+            for (int x = 0; x < 4; ++x)
+#pragma unroll
+                for (int c = 0; c < QC::N; ++c) acc[k][x][c] = 0.f;
             T[k] = 1.f;
             last[k] = 0;
             nc[k] = 0;
-            done[k] = !(px < vw.W && py < vw.H);
-            n_done += done[k];
+            Tl[k] = px < vw.W && ti.py0 + wt.ly + 4 * k < vw.H ? 1.f : -1.f;
         }
-        // n staged rows row_of(i) at list positions pos_of(i), front to back: first every alpha of
-        // the group (no dependence between entries), then the recurrence in T and the feature sums
-        auto group = [&](auto n_c, auto row_of, auto pos_of) {
-            constexpr int n = decltype(n_c)::value;
-            float al[n][PPT];  // 0: no contribution
+        // The chunk whose alphas are in s_A: hits has a bit for each entry that contributes to
+        // some pixel of the warp; entry e has its features at feat_of(e) and list position
+        // pos_of(e).  The recurrence in T, then the feature sums.
+        auto composite = [&](const uint32_t hits, auto feat_of, auto pos_of) {
+            uint32_t hit[PPT];  // the entries that contribute to the pixel
 #pragma unroll
-            for (int i = 0; i < n; ++i) {
-                const float4 g0 = s_geo0[row_of(i)];
-                const float4 g1 = s_geo1[row_of(i)];
+            for (int k = 0; k < PPT; ++k) hit[k] = 0;
+#pragma unroll 1
+            for (int e0 = 0; e0 < kChunk; e0 += 4) {
+                const uint32_t h4 = (hits >> e0) & 15u;
+                if (!h4) continue;
+                float tl = -1.f;
 #pragma unroll
-                for (int k = 0; k < PPT; ++k) {
-                    AlphaEval e;
-                    const bool hit = eval_alpha(fx - g0.x, (float)(wt.ly + 4 * k) - g0.y, g0.z, g0.w, g1.x, g1.y,
-                                                g1.z, g1.w, a.alpha_max, a.alpha_min, e);
-                    al[i][k] = hit ? e.alpha : 0.f;
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < n; ++i) {
-                float w[PPT];
-                bool any = false;
+                for (int k = 0; k < PPT; ++k) tl = fmaxf(tl, Tl[k]);
+                if (!__any_sync(SG_FULL_MASK, tl >= 0.f)) break;
+                float al[PPT][4];
 #pragma unroll
                 for (int k = 0; k < PPT; ++k) {
-                    const float A = al[i][k];
-                    const float Tn = __fmul_rn(T[k], __fsub_rn(1.f, A));
-                    bool hit = A > 0.f && !done[k];
-                    if (hit && Tn < a.T_min) {
-                        done[k] = true;
-                        ++n_done;
-                        hit = false;
-                    }
-                    w[k] = hit ? A * T[k] : 0.f;
-                    if (hit) {
-                        T[k] = Tn;
-                        last[k] = pos_of(i) + 1;
-                        ++nc[k];
-                        any = true;
+                    const float4 t = *reinterpret_cast<const float4 *>(s_A + (32 * k + lane) * kAPitch + e0);
+                    al[k][0] = t.x; al[k][1] = t.y; al[k][2] = t.z; al[k][3] = t.w;
+                }
+                uint32_t hb[PPT];
+#pragma unroll
+                for (int k = 0; k < PPT; ++k) hb[k] = 0;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (!((h4 >> i) & 1u)) continue;  // (warp-uniform)
+                    float f[QC::N];
+                    QC::load(feat_of(e0 + i), sub, f);
+#pragma unroll
+                    for (int k = 0; k < PPT; ++k) {
+                        const float A = al[k][i];
+                        const float Tn = __fmul_rn(Tl[k], __fsub_rn(1.f, A));
+                        const bool stop = Tn < a.T_min;  // (and again for a stopped pixel: Tl = -1)
+                        const float w = stop ? 0.f : A * Tl[k];
+                        if (!stop && A > 0.f) hb[k] |= 1u << i;
+                        T[k] = stop ? T[k] : Tn;
+                        Tl[k] = stop ? -1.f : Tn;
+#pragma unroll
+                        for (int x = 0; x < 4; ++x)
+                            fma_if<QC::N>(acc[k][x], x ? __shfl_xor_sync(SG_FULL_MASK, w, x) : w, f);
                     }
                 }
-                if (!__any_sync(SG_FULL_MASK, any)) continue;
-                const float4 *f4 = reinterpret_cast<const float4 *>(s_feat + (size_t)row_of(i) * NF);
 #pragma unroll
-                for (int q = 0; q < NF / 4; ++q) {
-                    const float4 f = f4[q];
-#pragma unroll
-                    for (int k = 0; k < PPT; ++k) fma4_if(&acc[k][4 * q], w[k], f);
-                }
+                for (int k = 0; k < PPT; ++k) hit[k] |= hb[k] << e0;
             }
+#pragma unroll
+            for (int k = 0; k < PPT; ++k) {
+                nc[k] += __popc(hit[k]);
+                if (hit[k]) last[k] = pos_of(31 - __clz(hit[k])) + 1;
+            }
+        };
+        auto any_live = [&]() {
+            bool r = false;
+#pragma unroll
+            for (int k = 0; k < PPT; ++k) r |= Tl[k] >= 0.f;
+            return r;
         };
         if (!hm) {
             for (int b0 = 0; b0 < n; b0 += batch) {
-                if (__syncthreads_count(n_done == PPT) == nthreads) break;
+                if (__syncthreads_count(!any_live()) == nthreads) break;
                 const int cnt = min(batch, n - b0);
                 load_batch<NF>(a, C, range.x, b0, cnt, ti.px0, ti.py0, rec_base, s_geo0, s_geo1, s_geo2, s_feat,
                                nullptr, nthreads);
                 __syncthreads();
-                if (__all_sync(SG_FULL_MASK, n_done == PPT)) continue;
-                // 32 entries at a time: lane l tests entry j0 + l against the warp's sub-tile, and
-                // the warp walks the entries that can reach it, front to back
-                for (int j0 = 0; j0 < cnt; j0 += 32) {
-                    if (__all_sync(SG_FULL_MASK, n_done == PPT)) break;
-                    const int jl = j0 + lane;
-                    uint32_t cm = __ballot_sync(SG_FULL_MASK, jl < cnt && !wt.misses(s_geo2[jl], s_geo1[jl], ln_amin));
-                    for (int m = __popc(cm); m >= GF; m -= GF) {
-                        int row[GF];
-#pragma unroll
-                        for (int i = 0; i < GF; ++i) {
-                            row[i] = j0 + __ffs(cm) - 1;
-                            cm &= cm - 1;
-                        }
-                        group(IntC<GF>(), [&](int i) { return row[i]; }, [&](int i) { return b0 + row[i]; });
+                // rows whose footprint can reach the warp's sub-tile (32 tested at once), queued
+                // front to back and composited 16 at a time
+                int top = 0, head = 0, qn = 0;
+                while (__any_sync(SG_FULL_MASK, any_live())) {
+                    while (qn < kChunk && top < cnt) {
+                        const int j = top + lane;
+                        const bool sel = j < cnt && !wt.misses(s_geo2[j], s_geo1[j], ln_amin);
+                        const uint32_t bal = __ballot_sync(SG_FULL_MASK, sel);
+                        if (sel) s_q[(head + qn + __popc(bal & lt)) & (kRing - 1)] = j;
+                        qn += __popc(bal);
+                        top += 32;
                     }
-                    for (; cm; cm &= cm - 1) {
-                        const int row = j0 + __ffs(cm) - 1;
-                        group(IntC<1>(), [row](int) { return row; }, [b0, row](int) { return b0 + row; });
-                    }
+                    if (qn == 0) break;
+                    __syncwarp();
+                    const int c = min(kChunk, qn), e = lane & 15;
+                    const int j = s_q[(head + min(e, c - 1)) & (kRing - 1)];
+                    EntryGeo g = entry_geo(s_geo0[j], s_geo1[j]);
+                    if (e >= c) g.o = 0.f;
+                    if (lane < kChunk) s_row[lane] = j;
+                    const uint32_t bal = __ballot_sync(
+                        SG_FULL_MASK, chunk_alphas<PPT>(g, ax, ay, a.alpha_max, a.alpha_min, s_A));
+                    __syncwarp();
+                    composite((bal | (bal >> 16)) & 0xffffu, [&](int r) { return s_feat + (size_t)s_row[r] * NF; },
+                              [&](int r) { return b0 + s_row[r]; });
+                    __syncwarp();
+                    head += c;
+                    qn -= c;
                 }
             }
         } else {
-            // list positions whose half mask holds this half, ascending: (s_q, s_qr)[0 .. qn)
-            // is the queue of (position, record), top the next position scanned
-            const uint32_t lt = (1u << lane) - 1u;
-            int top = 0, qn = 0;
-            while (!__all_sync(SG_FULL_MASK, n_done == PPT)) {
-                while (qn < kFwdHalfChunk && top < n) {
+            // list positions whose half mask holds this half, ascending: (s_q, s_qr) is a ring
+            // of (position, record), top the next position scanned, word its list word (loaded
+            // one scan ahead)
+            int top = 0, head = 0, qn = 0;
+            uint32_t word = lane < n ? a.record[range.x + lane] : 0u;  // record | half mask << 30
+            auto fill = [&]() {
+                while (qn < kChunk && top < n) {
+                    const uint32_t w = word;
                     const int pos = top + lane;
-                    uint32_t rec = 0u;
-                    bool sel = false;
-                    if (pos < n) {
-                        const uint32_t word = a.record[range.x + pos];  // record | half mask << 30
-                        rec = word & 0x3fffffffu;
-                        sel = (word >> (30 + hf)) & 1u;
-                    }
+                    top += 32;
+                    word = top + lane < n ? a.record[range.x + top + lane] : 0u;
+                    const bool sel = (w >> (30 + hf)) & 1u;  // (0 past the list's end)
                     const uint32_t bal = __ballot_sync(SG_FULL_MASK, sel);
                     if (sel) {
-                        s_q[qn + __popc(bal & lt)] = pos;
-                        s_qr[qn + __popc(bal & lt)] = rec;
+                        const int q = (head + qn + __popc(bal & lt)) & (kRing - 1);
+                        s_q[q] = pos;
+                        s_qr[q] = w & 0x3fffffffu;
                     }
                     qn += __popc(bal);
-                    top += 32;
-                    __syncwarp();
                 }
-                if (qn == 0) break;
-                const int c = min(kFwdHalfChunk, qn);
-                stage_rows_warp<NF>(a, C, [&](int j) { return s_qr[j]; }, c, ti.px0, ti.py0, rec_base, s_geo0, s_geo1,
-                                    nullptr, s_feat, nullptr);
                 __syncwarp();
-                int j = 0;
-                for (; j + GF <= c; j += GF) {
-                    if (__all_sync(SG_FULL_MASK, n_done == PPT)) break;
-                    group(IntC<GF>(), [j](int i) { return j + i; }, [s_q, j](int i) { return s_q[j + i]; });
+            };
+            // requests the next chunk of the ring: geometry of entry lane % 16 and its position
+            // into registers, features into buffer buf
+            float4 g0, g1;
+            int pos = 0;
+            auto request = [&](int buf) {
+                fill();
+                const int c = min(kChunk, qn), e = lane & 15;
+                if (c > 0) {
+                    const int q = (head + min(e, c - 1)) & (kRing - 1);
+                    const uint32_t rec = s_qr[q];
+                    pos = s_q[q];
+                    g0 = a.geo[2 * (size_t)rec];
+                    g1 = a.geo[2 * (size_t)rec + 1];
+                    stage_features_async<NF>(a, rec, rec_base, s_hf + buf * kChunk * NF);
                 }
-                if (j + GF > c)  // (else the pixels are saturated)
-                    for (; j < c; ++j) group(IntC<1>(), [j](int) { return j; }, [s_q, j](int) { return s_q[j]; });
-                __syncwarp();
-                // drop the staged entries from the queue
-                const int rest = qn - c;  // (< 32)
-                const int keep = lane < rest ? s_q[c + lane] : 0;
-                const uint32_t keep_rec = lane < rest ? s_qr[c + lane] : 0u;
-                __syncwarp();
-                if (lane < rest) {
-                    s_q[lane] = keep;
-                    s_qr[lane] = keep_rec;
+                cp_async_commit_group();
+                head += c;
+                qn -= c;
+                return c;
+            };
+            int buf = 0;
+            int c = request(0);
+            while (c > 0 && __any_sync(SG_FULL_MASK, any_live())) {
+                const int e = lane & 15;
+                float *feat = s_hf + buf * kChunk * NF;
+                EntryGeo g = record_geo(g0, g1, ti.px0, ti.py0);
+                if (e >= c) g.o = 0.f;
+                if (lane < kChunk) {
+                    s_row[lane] = pos;
+                    feat[lane * NF + 3] = g0.z;  // depth (camera z of the mean, Eq. 8)
                 }
-                qn = rest;
                 __syncwarp();
+                c = request(buf ^ 1);
+                const uint32_t bal = __ballot_sync(
+                    SG_FULL_MASK, chunk_alphas<PPT>(g, ax, ay, a.alpha_max, a.alpha_min, s_A));
+                cp_async_wait_groups<1>();
+                __syncwarp();
+                composite((bal | (bal >> 16)) & 0xffffu, [&](int r) { return feat + r * NF; },
+                          [&](int r) { return s_row[r]; });
+                __syncwarp();
+                buf ^= 1;
             }
+            cp_async_wait_groups<0>();
         }
+        // the quad's pixels in order: v[j] is the pixel of lane (lane & ~3) + j
         const size_t HW = (size_t)vw.W * vw.H;
         const size_t p0 = (size_t)vw.pixel_offset;
+        const int qx = px - sub;  // first pixel column of the quad
 #pragma unroll
         for (int k = 0; k < PPT; ++k) {
             const int py = ti.py0 + wt.ly + 4 * k;
-            if (!(px < vw.W && py < vw.H)) continue;
-            const size_t p = (size_t)py * vw.W + px;
-            a.img_rgb[3 * p0 + p] = acc[k][0] + T[k] * a.bg0;
-            a.img_rgb[3 * p0 + HW + p] = acc[k][1] + T[k] * a.bg1;
-            a.img_rgb[3 * p0 + 2 * HW + p] = acc[k][2] + T[k] * a.bg2;
-            a.img_depth[p0 + p] = acc[k][3];
+            float Tq[4];
 #pragma unroll
-            for (int c = 0; c < C; ++c) a.img_sem[(size_t)C * p0 + c * HW + p] = acc[k][4 + c];
-            a.T_final[p0 + p] = T[k];
-            a.last[p0 + p] = last[k];
-            a.n_contrib[p0 + p] = nc[k];
+            for (int j = 0; j < 4; ++j) Tq[j] = __shfl_sync(SG_FULL_MASK, T[k], (lane & ~3) | j);
+            if (py >= vw.H) continue;
+            const size_t p = (size_t)py * vw.W + qx;
+#pragma unroll
+            for (int i = 0; i < QC::N; ++i) {
+                float v[4] = {acc[k][0][i], acc[k][1][i], acc[k][2][i], acc[k][3][i]};
+                if (sub & 1) {
+                    float t = v[0]; v[0] = v[1]; v[1] = t;
+                    t = v[2]; v[2] = v[3]; v[3] = t;
+                }
+                if (sub & 2) {
+                    float t = v[0]; v[0] = v[2]; v[2] = t;
+                    t = v[1]; v[1] = v[3]; v[3] = t;
+                }
+                if (i == 0) {
+                    if (sub < 3) {
+                        const float bg = sub == 0 ? a.bg0 : sub == 1 ? a.bg1 : a.bg2;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) v[j] = v[j] + Tq[j] * bg;
+                    }
+                    store_quad(sub < 3 ? a.img_rgb + 3 * p0 + sub * HW + p : a.img_depth + p0 + p, v, vw.W - qx);
+                } else {
+                    store_quad(a.img_sem + (size_t)C * p0 + QC::sem(i - 1, sub) * HW + p, v, vw.W - qx);
+                }
+            }
+            if (px >= vw.W) continue;
+            a.T_final[p0 + p + sub] = T[k];
+            a.last[p0 + p + sub] = last[k];
+            a.n_contrib[p0 + p + sub] = nc[k];
         }
         __syncthreads();
     }
@@ -427,7 +574,6 @@ __global__ void __launch_bounds__(kMaxTileThreads) raster_fwd_kernel(RasterArgs 
 //   M[r][m]  = sum_p s[p][r] P_m(X_p, Y_p)    (moments of s = dL/dsigma)
 // with w = alpha T and P = (1, X, Y, X^2, XY, Y^2) the pixel offsets from the warp centre.
 // The 2D-mean, conic and opacity gradients are linear in the moments (see moment_grads).
-constexpr int kChunk = 16;
 constexpr int kHalfQueue = kChunk + 32;  // entries pending (< 16 + one 32-entry scan)
 
 template <int NPX>
@@ -443,15 +589,18 @@ template <int NF>
 __host__ __device__ constexpr int g_pitch() { return (NF / 4) % 2 == 1 ? NF : NF + 4; }
 
 // shared memory of one warp (4-byte words): the chunk's rows and the queue (with records in
-// half mode), G (NPX x g_pitch) and two chunk buffers (16 x chunk_pitch); a multiple of 16 bytes
+// half mode), their list positions, G (NPX x g_pitch), two chunk buffers (16 x chunk_pitch) and
+// the chunk's alphas; a multiple of 16 bytes.  At one pixel per thread the second chunk buffer
+// reuses the alphas' (read into registers first): 20 instead of 17 one-warp CTAs per SM in half
+// mode (batched workload 2072 -> 2009 us); with more pixels the registers cost more than that.
+template <int PPT>
+__host__ __device__ constexpr bool bwd_overlay() { return PPT == 1; }
 template <int C, int PPT, bool HALF>
 __host__ __device__ constexpr int bwd_warp_words() {
-    return kChunk + (HALF ? 2 : 1) * kHalfQueue + 32 * PPT * g_pitch<4 + C>() + 2 * kChunk * chunk_pitch<32 * PPT>();
+    static_assert(kChunk * chunk_pitch<32 * PPT>() <= 32 * PPT * kAPitch, "the second chunk buffer reuses the alphas'");
+    return 2 * kChunk + (HALF ? 2 : 1) * kHalfQueue + 32 * PPT * g_pitch<4 + C>() +
+           (bwd_overlay<PPT>() ? 1 : 2) * kChunk * chunk_pitch<32 * PPT>() + 32 * PPT * kAPitch;
 }
-
-// Entries whose alpha the backward evaluates together (before their serial recurrence).
-template <int PPT>
-__host__ __device__ constexpr int bwd_group() { return PPT == 1 ? 8 : 4; }
 
 // Gradients of the 2D mean (u, v), the conic (a, b, c) and the opacity from the moments
 // M = (sum s, sum s X, sum s Y, sum s X^2, sum s XY, sum s Y^2) of s = dL/dsigma over the
@@ -490,7 +639,6 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
     constexpr int NT = NFP / 8;                   // 8-feature tiles
     constexpr int NPX = 32 * PPT;                 // pixels of one warp (pixel q = 32 k + lane)
     constexpr int KS = NPX / 8;                   // 8-pixel steps
-    constexpr int GR = bwd_group<PPT>();
     constexpr int WQ = chunk_pitch<NPX>();
     constexpr int GP = g_pitch<NF>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -511,19 +659,22 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
     float4 *s_geo2 = hm ? nullptr : s_geo1 + batch;
     float *s_feat = reinterpret_cast<float *>(s_geo1 + (hm ? batch : 2 * batch));
     uint32_t *s_rec = reinterpret_cast<uint32_t *>(s_feat + (size_t)batch * NF);
-    // per warp: the list position (half mode) or staged row (shared batches) of each chunk row,
-    // and the queue of pending entries: (list position, record), or staged rows
+    // per warp: the staged row of each chunk row (shared batches), its list position, and the
+    // queue of pending entries: (list position, record), or staged rows
     const int nthreads = hm ? 32 : a.tile_w * a.tile_h / PPT;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int *s_pos = reinterpret_cast<int *>(s_rec + batch) + (size_t)warp * bwd_warp_words<C, PPT, HALF>();
-    int *s_q = s_pos + kChunk;
+    int *s_lp = s_pos + kChunk;  // list position of each chunk row (the largest int past its end)
+    int *s_q = s_lp + kChunk;
     uint32_t *s_qr = reinterpret_cast<uint32_t *>(s_q + kHalfQueue);
     float *s_G = reinterpret_cast<float *>(s_qr + (hm ? kHalfQueue : 0));
     float *s_gw = s_G + NPX * GP;     // per chunk row: gf, then overwritten with w = alpha T
-    float *s_sg = s_gw + kChunk * WQ; // per chunk row: s = dL/dsigma
+    float *s_A = s_gw + kChunk * WQ;  // alphas (chunk_alphas)
+    constexpr bool OVER = bwd_overlay<PPT>();
+    float *s_sg = OVER ? s_A : s_A + 32 * PPT * kAPitch;  // per chunk row: s = dL/dsigma
     const int gid = lane >> 2, tig = lane & 3;
     const WarpTile<PPT> wt(a.tile_w);
-    const float fx = (float)wt.lx;
+    const float ax = (float)(wt.lx - (lane & 7) + 4 * (lane >> 4)), ay = (float)(wt.ly - (lane >> 3));
     const float ln_amin = __logf(a.alpha_min);
     // moment polynomials at the B-fragment pixels: pixel 8 ks + tig (+ 4) has X = tig - 3.5
     // (tig + 0.5), Y = (ks % 4) + 4 (ks / 4) - (2 PPT - 0.5); P_gid = P0 + Y (P1 + Y P2)
@@ -587,8 +738,10 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
         const int warp_last = __reduce_max_sync(SG_FULL_MASK, thread_last);
         __syncwarp();
         // One chunk of c <= 16 list entries, back to front: chunk row r (ascending list position)
-        // is staged row row_of(r) at list position pos_of(r) (pos_of(r) >= warp_last for r >= c).
-        auto chunk = [&](const int c, auto row_of, auto pos_of) {
+        // is staged row row_of(r) at list position s_lp[r] (>= warp_last for r >= c), and lane l
+        // holds the geometry g of row l % 16 (rows >= c: opacity 0).
+        auto chunk = [&](const int c, const EntryGeo &g, auto row_of) {
+                chunk_alphas<PPT>(g, ax, ay, a.alpha_max, a.alpha_min, s_A);
                 // ---- gf = F G^T for the chunk (M = entries, N = pixels, K = features) ----
                 // ldmatrix row addresses: lanes 0-15 rows 0-15 of the first four columns, lanes
                 // 16-31 the same rows four columns further (A); lanes 8 m + i row i of matrix m (B)
@@ -642,37 +795,21 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
                     }
                 }
                 __syncwarp();
-                // ---- back to front, GR entries at a time: first every alpha of the group (no
-                // dependence between entries), then the recurrence in T and a ----
+                // ---- back to front: the recurrence in T and a ----
                 uint32_t hits = 0;  // rows that contribute to one of the lane's pixels
-#pragma unroll 1
-                for (int rg = (c - 1) / GR * GR; rg >= 0; rg -= GR) {
-                    float al[PPT][GR];  // 0: no contribution
+                auto recur = [&](const int rg, const float (&al)[PPT][4]) {  // rows rg .. rg + 3
+                    const int4 lp = *reinterpret_cast<const int4 *>(s_lp + rg);
+                    const int pos[4] = {lp.x, lp.y, lp.z, lp.w};
                     uint32_t hb = 0;
 #pragma unroll
-                    for (int i = 0; i < GR; ++i) {
-                        const int j = row_of(rg + i), pos = pos_of(rg + i);
-                        const float4 g0 = s_geo0[j];
-                        const float4 g1 = s_geo1[j];
-#pragma unroll
-                        for (int k = 0; k < PPT; ++k) {
-                            AlphaEval e;
-                            const bool hit = eval_alpha(fx - g0.x, (float)(wt.ly + 4 * k) - g0.y, g0.z, g0.w, g1.x,
-                                                        g1.y, g1.z, g1.w, a.alpha_max, a.alpha_min, e) &&
-                                             pos < my_last[k];
-                            al[k][i] = hit ? e.alpha : 0.f;
-                            if (hit) hb |= 1u << i;
-                        }
-                    }
-                    hits |= hb << rg;
-#pragma unroll
-                    for (int i = GR - 1; i >= 0; --i) {
+                    for (int i = 3; i >= 0; --i) {
                         float *gw = s_gw + (rg + i) * WQ + lane;
 #pragma unroll
                         for (int k = 0; k < PPT; ++k) {
-                            const float A = al[k][i], om = 1.f - A;
+                            const float A = pos[i] < my_last[k] ? al[k][i] : 0.f, om = 1.f - A;
                             // (a pixel without a contribution keeps T and a: A = 0, gf taken as 0)
                             const float gf = A > 0.f ? gw[32 * k] : 0.f;
+                            if (A > 0.f) hb |= 1u << i;
                             // transmittance before this Gaussian (only gradients depend on it)
                             T[k] *= rcp_fast(om);
                             const float dalpha = T[k] * (gf - acc_a[k]);
@@ -682,10 +819,34 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
                             s_sg[(rg + i) * WQ + 32 * k + lane] = A < a.alpha_max ? -dalpha * A : 0.f;
                         }
                     }
+                    hits |= hb << rg;
+                };
+                auto alphas = [&](int rg, float (&al)[PPT][4]) {
+#pragma unroll
+                    for (int k = 0; k < PPT; ++k) {
+                        const float4 t = *reinterpret_cast<const float4 *>(s_A + (32 * k + lane) * kAPitch + rg);
+                        al[k][0] = t.x; al[k][1] = t.y; al[k][2] = t.z; al[k][3] = t.w;
+                    }
+                };
+                if constexpr (OVER) {
+                    float al[kChunk / 4][PPT][4];
+#pragma unroll
+                    for (int q = 0; q < kChunk / 4; ++q) alphas(4 * q, al[q]);
+                    __syncwarp();  // (s_sg reuses s_A)
+#pragma unroll
+                    for (int q = kChunk / 4 - 1; q >= 0; --q)
+                        if (4 * q < c) recur(4 * q, al[q]);  // (warp-uniform)
+                } else {
+#pragma unroll 1
+                    for (int rg = (c - 1) & ~3; rg >= 0; rg -= 4) {
+                        float al[PPT][4];
+                        alphas(rg, al);
+                        recur(rg, al);
+                    }
                 }
                 const uint32_t mask = __reduce_or_sync(SG_FULL_MASK, hits);
-                if (!mask) return;  // (warp-uniform)
                 __syncwarp();
+                if (!mask) return;  // (warp-uniform)
                 // ---- dF = W G (M = entries, N = features, K = pixels), moments M = S P ----
                 // (rows without a contribution may hold stale values: they are not written out)
                 const bool keep0 = (mask >> gid) & 1u, keep1 = (mask >> (gid + 8)) & 1u;
@@ -725,27 +886,27 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
                     if (!(hr ? keep1 : keep0)) continue;
                     const uint32_t rec = s_rec[row_of(gid + 8 * hr)];
                     const uint32_t gi = rec - rec_base;
-                    const size_t si = (size_t)C * (a.sem_rec ? rec : gi);
+                    float *gs = a.g_sem + (size_t)C * (a.sem_rec ? rec : gi);
+                    // features 0-7: colour and depth in lanes 0, 1 of the quad, semantics in 2, 3
+                    float *p0 = a.g_col + (size_t)a.col_stride * (a.col_rec ? rec : gi) + 2 * tig;
+                    float *p1 = tig == 1 ? a.g2d + 8 * (size_t)rec + 6 : p0 + 1;
+                    if (tig >= 2) {
+                        p0 = gs + 2 * tig - 4;
+                        p1 = p0 + 1;
+                    }
+                    atomicAdd(p0, df[0][2 * hr]);
+                    atomicAdd(p1, df[0][2 * hr + 1]);
 #pragma unroll
-                    for (int nt = 0; nt < NT; ++nt) {
-                        // features 2 tig, 2 tig + 1 of this n-tile: both semantic (C even) ->
-                        // one 8-byte vector reduction when the buffer allows it
+                    for (int nt = 1; nt < NT; ++nt) {
+                        // features 2 tig, 2 tig + 1 of this n-tile: one 8-byte vector reduction when
+                        // the buffer allows it
                         const int f0 = 8 * nt + 2 * tig;
-                        if (a.sem_v2 && f0 >= 4 && f0 + 1 < NF) {
-                            red_add_v2(a.g_sem + si + (f0 - 4), df[nt][2 * hr], df[nt][2 * hr + 1]);
-                            continue;
-                        }
-#pragma unroll
-                        for (int c2 = 0; c2 < 2; ++c2) {
-                            const int f = f0 + c2;
-                            const float val = df[nt][2 * hr + c2];
-                            if (f >= NF) continue;
-                            if (f < 3)
-                                atomicAdd(a.g_col + (size_t)a.col_stride * (a.col_rec ? rec : gi) + f, val);
-                            else if (f == 3)
-                                atomicAdd(a.g2d + 8 * (size_t)rec + 6, val);
-                            else
-                                atomicAdd(a.g_sem + si + (f - 4), val);
+                        if (f0 >= NF) continue;
+                        if (a.sem_v2) {
+                            red_add_v2(gs + (f0 - 4), df[nt][2 * hr], df[nt][2 * hr + 1]);
+                        } else {
+                            atomicAdd(gs + (f0 - 4), df[nt][2 * hr]);
+                            atomicAdd(gs + (f0 - 3), df[nt][2 * hr + 1]);
                         }
                     }
                 }
@@ -806,14 +967,19 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
                     __syncwarp();
                     const int c = min(kChunk, qn);
                     // chunk row r is queue entry c - 1 - r; rows past c stay out of reach
-                    if (lane < kChunk) s_pos[lane] = lane < c ? s_q[c - 1 - lane] : 0;
+                    if (lane < kChunk) {
+                        s_pos[lane] = lane < c ? s_q[c - 1 - lane] : 0;
+                        s_lp[lane] = lane < c ? b0 + s_q[c - 1 - lane] : 0x7fffffff;
+                    }
                     const int rest = qn - c;  // (< 32)
                     const int keep = lane < rest ? s_q[c + lane] : 0;
                     __syncwarp();
                     if (lane < rest) s_q[lane] = keep;
                     qn = rest;
-                    chunk(c, [s_pos](int r) { return s_pos[r]; },
-                          [s_pos, b0, c](int r) { return r < c ? b0 + s_pos[r] : 0x7fffffff; });
+                    const int j = s_pos[lane & 15];
+                    EntryGeo g = entry_geo(s_geo0[j], s_geo1[j]);
+                    if ((lane & 15) >= c) g.o = 0.f;
+                    chunk(c, g, [s_pos](int r) { return s_pos[r]; });
                 }
             }
             __syncthreads();
@@ -843,10 +1009,22 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
                 }
                 if (qn == 0) break;
                 const int c = min(kChunk, qn);
-                // rows 0 .. c-1 in ascending list position: row r is queue entry c - 1 - r
-                stage_rows_warp<NF>(a, C, [&](int j) { return s_qr[c - 1 - j]; }, c, ti.px0, ti.py0, rec_base, s_geo0,
-                                    s_geo1, s_geo2, s_feat, s_rec);
-                if (lane < kChunk) s_pos[lane] = lane < c ? s_q[c - 1 - lane] : 0x7fffffff;
+                // rows 0 .. c-1 in ascending list position: row r is queue entry c - 1 - r; lane l
+                // loads the geometry of row l % 16 (lanes 0-15 also stage it)
+                const int q = max(c - 1 - (lane & 15), 0);
+                const uint32_t rec = s_qr[q];
+                const float4 r0 = a.geo[2 * (size_t)rec], r1 = a.geo[2 * (size_t)rec + 1];
+                stage_features_async<NF>(a, rec, rec_base, s_feat);
+                cp_async_commit_group();
+                EntryGeo g = record_geo(r0, r1, ti.px0, ti.py0);
+                if ((lane & 15) >= c) g.o = 0.f;
+                if (lane < kChunk) {
+                    s_geo0[lane] = make_float4(g.ui, g.vi, g.uf, g.vf);
+                    s_geo1[lane] = make_float4(g.m00, g.m10, g.m11, g.o);
+                    s_rec[lane] = rec;
+                    s_feat[lane * NF + 3] = r0.z;  // depth (camera z of the mean, Eq. 8)
+                    s_lp[lane] = lane < c ? s_q[q] : 0x7fffffff;
+                }
                 const int rest = qn - c;  // (< 32)
                 const int keep = lane < rest ? s_q[c + lane] : 0;
                 const uint32_t keep_rec = lane < rest ? s_qr[c + lane] : 0u;
@@ -856,8 +1034,9 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
                     s_qr[lane] = keep_rec;
                 }
                 qn = rest;
+                cp_async_wait_groups<0>();
                 __syncwarp();
-                chunk(c, [](int r) { return r; }, [s_pos](int r) { return s_pos[r]; });
+                chunk(c, g, [](int r) { return r; });
             }
             __syncwarp();
         }
@@ -868,25 +1047,25 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
 // ---------------------------------------------------------------------------------------
 
 template <int C>
-inline size_t fwd_smem(int batch) {
+inline size_t batch_smem(int batch) {
     return (size_t)batch * (3 * 16 + 4 * (4 + C));
 }
 template <int C, int PPT>
-inline size_t bwd_smem(int batch, int threads) {
-    return fwd_smem<C>(batch) + (size_t)batch * 4 + sizeof(float) * (threads / 32) * bwd_warp_words<C, PPT, false>();
+inline size_t fwd_smem(int batch, int threads) {
+    return batch_smem<C>(batch) + sizeof(float) * (threads / 32) * fwd_warp_words<C, PPT, false>();
 }
-// half mode: one 16-entry chunk staged without its (u, v, ex, ey) rows (+ its list positions),
-// the (position, record) queue, one warp
-template <int C>
-inline size_t bwd_half_smem() {
-    return fwd_smem<C>(kChunk) - (size_t)kChunk * 16 + (size_t)kChunk * 4 + sizeof(float) * bwd_warp_words<C, 1, true>();
-}
-
-// forward half mode: one 32-entry chunk staged without its (u, v, ex, ey) rows, and the
-// (position, record) queue
 template <int C>
 inline size_t fwd_half_smem() {
-    return (size_t)kFwdHalfChunk * (2 * 16 + 4 * (4 + C)) + (size_t)kFwdHalfQueue * 4 * 2;
+    return sizeof(float) * fwd_warp_words<C, 1, true>();
+}
+template <int C, int PPT>
+inline size_t bwd_smem(int batch, int threads) {
+    return batch_smem<C>(batch) + (size_t)batch * 4 + sizeof(float) * (threads / 32) * bwd_warp_words<C, PPT, false>();
+}
+// half mode: one 16-entry chunk staged without its (u, v, ex, ey) rows, one warp
+template <int C>
+inline size_t bwd_half_smem() {
+    return batch_smem<C>(kChunk) - (size_t)kChunk * 16 + (size_t)kChunk * 4 + sizeof(float) * bwd_warp_words<C, 1, true>();
 }
 
 inline int resident_grid(const void *fn, int threads, size_t smem) {
@@ -905,7 +1084,7 @@ sg_status launch_raster_cp(RasterArgs &a, bool backward, cudaStream_t st) {
     const bool half = a.half && PPT == 1 && a.tile_w == 8 && a.tile_h == 8 && (backward || a.half_fwd);
     const int threads = half ? 32 : a.tile_w * a.tile_h / PPT;
     const size_t smem = backward ? (half ? bwd_half_smem<C>() : bwd_smem<C, PPT>(a.batch, threads))
-                                 : (half ? fwd_half_smem<C>() : fwd_smem<C>(a.batch));
+                                 : (half ? fwd_half_smem<C>() : fwd_smem<C, PPT>(a.batch, threads));
     const void *fn = backward ? (half ? (const void *)raster_bwd_kernel<C, PPT, PPT == 1>
                                       : (const void *)raster_bwd_kernel<C, PPT>)
                               : (half ? (const void *)raster_fwd_kernel<C, PPT, PPT == 1>

@@ -27,31 +27,26 @@ struct Float3 {
 // m10 = -s01/sqrt(2 s00 det), m11 = sqrt(s00/(2 det)): a sum of squares, so no
 // cancellation for elongated footprints, and 7 flops.  The forward and backward kernels
 // must take bit-identical skip/stop decisions, so every rounding step is spelled out with
-// _rn intrinsics (no compiler contraction can differ between kernels).
+// _rn intrinsics (no compiler contraction can differ between kernels).  The 2D mean is an
+// integer (ui, vi) plus a float fraction (uf, vf): (px - ui) is exact in float and
+// dx = (px - ui) - uf is the correctly rounded offset, whatever the tile.
 // ----------------------------------------------------------------------------------------
-struct AlphaEval {
-    float dx, dy;  // pixel - mean2D
-    float p1, p2;  // m00 dx, m10 dx + m11 dy
-    float G;       // exp(-sigma)
-    float raw;     // o * G
-    float alpha;   // min(alpha_max, raw)
-};
 
-// (px - ui) and (py - vi) are exact integers held in floats, (uf, vf) the float fractions of
-// the 2D mean: dx = (px - ui) - uf is the correctly rounded offset, whatever the tile.
-__device__ __forceinline__ bool eval_alpha(float px_ui, float py_vi, float uf, float vf, float m00,
-                                           float m10, float m11, float o, float alpha_max,
-                                           float alpha_min, AlphaEval &e) {
-    e.dx = __fsub_rn(px_ui, uf);
-    e.dy = __fsub_rn(py_vi, vf);
-    e.p1 = __fmul_rn(m00, e.dx);
-    e.p2 = __fmaf_rn(m10, e.dx, __fmul_rn(m11, e.dy));
-    const float sigma = __fmaf_rn(e.p2, e.p2, __fmul_rn(e.p1, e.p1));
-    if (!(sigma >= 0.f)) return false;
-    e.G = __expf(-sigma);
-    e.raw = __fmul_rn(o, e.G);
-    e.alpha = fminf(alpha_max, e.raw);
-    return e.alpha >= alpha_min;
+// 2^x, approximate (results below the normal range flush to 0)
+__device__ __forceinline__ float ex2_fast(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// alpha from dx, q = m11 dy and (m00 dx)^2, each rounded as above; 0 below alpha_min.
+// exp(-sigma) = 2^(-sigma log2 e).  (A non-finite sigma gives no alpha: the comparison fails.)
+__device__ __forceinline__ float entry_alpha(float m10, float dx, float q, float p1_sq, float o, float alpha_max,
+                                             float alpha_min) {
+    const float p2 = __fmaf_rn(m10, dx, q);
+    const float sigma = __fmaf_rn(p2, p2, p1_sq);
+    const float raw = __fmul_rn(o, ex2_fast(__fmul_rn(sigma, -1.4426950408889634f)));
+    return raw >= alpha_min ? fminf(alpha_max, raw) : 0.f;
 }
 
 // ---- double-float (unevaluated sum hi + lo of two floats) helpers --------------------
@@ -163,6 +158,22 @@ __device__ __forceinline__ void ldsm_x4(const float *p, uint32_t (&r)[4]) {
     const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];\n"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+
+// Asynchronous copies global -> shared (4 bytes, zero-filled when !valid while src must still
+// be a mapped address; 16 bytes, both sides 16-byte aligned) and their group fences.
+__device__ __forceinline__ void cp_async4(void *dst, const void *src, bool valid) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>  // waits until at most the N latest groups are pending
+__device__ __forceinline__ void cp_async_wait_groups() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
 // 1 / x, approximate (x normal; 1 ulp, exact for 1)
