@@ -2,23 +2,34 @@
 //
 // Pipeline (all counts stay on the device, so the whole sequence can be captured in a
 // CUDA graph with a fixed launch shape):
-//   1. compact:  visible records r (non-empty tile rectangle) -> (depth bits, r), in r order
+//   1. compact:  visible records r (non-empty tile rectangle) -> (depth bits, r), in r order,
+//                and the digit histograms of the depth keys
 //   2. sort:     stable LSD radix sort by the 32 float32 depth bits (depths are > z_near > 0
 //                so their bit patterns order like the values); ties keep record order
 //   3. emit:     the slots are the tile rows of each record's rectangle, record after
 //                record in depth order (a prefix of the row counts numbers them); for each
 //                slot the span of the record's alpha >= alpha_min region within the row (a
-//                float32 computation) gives the contiguous run of tiles it reaches; a
-//                counting pass, split evenly over the slots, and a scan give the offsets, and
-//                an emission pass writes (global tile id, r) for those tiles, row-major
+//                float32 computation) gives the contiguous run of tiles it reaches, and the
+//                kept tiles are written as (global tile id, r), row-major, with the digit
+//                histograms of the tile ids
 //   4. sort:     stable LSD radix sort of the instances by global tile id (only the bits
 //                n_tiles needs), which keeps the (depth, record) order inside each tile
 //   5. ranges:   [start, end) of every tile
 //   6. order:    (when requested) the tile ids by descending half-octave bucket of their list
 //                length, one stable counting pass: the compositing kernels' work order
-// The result equals sorting all kept instances by (tile, depth bits, record id).  Every radix
-// pass is three kernels: per-block digit histograms, per-digit scans over the blocks, and
-// a stable scatter that ranks equal digits inside a block by warp match + prefix counts.
+// The result equals sorting all kept instances by (tile, depth bits, record id).
+//
+// Every step that needs a prefix over the whole input (compaction, slot numbering, emission,
+// each radix pass, the work order) is one kernel with a chained scan: a block draws its part's
+// number from a counter, publishes the part's aggregate, sums its predecessors' published
+// words back to the nearest one that already holds an inclusive prefix, and publishes its own.
+// Parts are drawn in order, so the predecessors of a part are held by blocks that already run;
+// every wait is bounded all the same (SG_STATUS_TIMEOUT).  The steps were three kernels each
+// before (count, scan of the counts, apply): 33 launches per list build, now 12 or 13 and one
+// memset, and the keys and footprints are read once instead of twice.  What that gives is
+// the launches and their latencies (320x180 x 3 levels with 30k Gaussians: 110 -> 70 us of
+// kernels and 21 launch gaps); on the batched workload (2.1M visible records, 19M instances)
+// the kernels take the same time as before (1.0 ms).
 #include <cstdio>
 
 #include <algorithm>
@@ -28,22 +39,16 @@
 namespace sg {
 
 constexpr int kScanThreads = 256;
-// Widest digit of the tile sort.  Each pass scatters a block's instances over 2^digit runs
-// of the output; with 9-bit digits (512 runs per block) the partly written output lines no
+// Widest digit of the tile sort.  Each pass scatters a part's instances over 2^digit runs
+// of the output; with 9-bit digits (512 runs per part) the partly written output lines no
 // longer stay in L2 and the pass reads and writes twice its bytes in DRAM (measured), so 17 or
 // 18 bits of tile id sort in three passes of 6 bits rather than two of 9 and 8.
 constexpr int kTileDigitBits = 8;
 
-__device__ __forceinline__ void block_range(int n, int G, int b, int &beg, int &end) {
-    const int tiles = (n + kScanThreads - 1) / kScanThreads;
-    const int per = (tiles + G - 1) / G;
-    beg = min(n, b * per * kScanThreads);
-    end = min(n, beg + per * kScanThreads);
-}
-
-// Exclusive block scan of one value per thread (blockDim == kScanThreads).
+// Exclusive block scan of one value per thread (blockDim == NT).
+template <int NT = kScanThreads>
 __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t &total) {
-    __shared__ uint32_t s_warp[kScanThreads / 32 + 1];
+    __shared__ uint32_t s_warp[NT / 32 + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t incl = v;
 #pragma unroll
@@ -54,7 +59,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t &t
     if (lane == 31) s_warp[warp] = incl;
     __syncthreads();
     if (warp == 0) {
-        const int nw = kScanThreads / 32;
+        const int nw = NT / 32;
         uint32_t w = lane < nw ? s_warp[lane] : 0u;
         uint32_t wi = w;
 #pragma unroll
@@ -67,22 +72,107 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t &t
     }
     __syncthreads();
     const uint32_t res = incl - v + s_warp[warp];
-    total = s_warp[kScanThreads / 32];
+    total = s_warp[NT / 32];
     __syncthreads();
     return res;
 }
 
 // ---------------------------------------------------------------------------------------
-// Device-wide exclusive scan (reduce / scan block sums / apply) with a device-side count.
+// Chained scan over parts.  A part's word is 0 until published, then flag | value.
 // ---------------------------------------------------------------------------------------
 
-struct VisibleCount {  // 1 if the record's tile rectangle is non-empty
-    const uint2 *rect;
-    __device__ uint32_t operator()(int i) const {
-        const uint2 r = rect[i];
-        return r.x != r.y ? 1u : 0u;
+constexpr uint64_t kAggregate = 1ull << 32;  // value: the part's own sum
+constexpr uint64_t kPrefix = 1ull << 33;     // value: inclusive prefix through the part
+constexpr uint32_t kSpinLimit = 1u << 22;
+
+__device__ __forceinline__ uint64_t load_word(const uint64_t *p) {
+    uint64_t v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];\n" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void store_word(uint64_t *p, uint64_t v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;\n" ::"l"(p), "l"(v) : "memory");
+}
+
+// The word of an earlier part, once published; on a timeout (status flagged) an empty prefix.
+__device__ __forceinline__ uint64_t wait_word(const uint64_t *p, uint64_t w, uint32_t *status) {
+    for (uint32_t polls = 0; !(w >> 32); ++polls) {
+        if (polls >= kSpinLimit) {
+            atomicOr(status, SG_STATUS_TIMEOUT);
+            return kPrefix;
+        }
+        w = load_word(p);
     }
-};
+    return w;
+}
+
+// Exclusive prefix of the part whose sum is `own`, for a whole block (every thread gets it);
+// publishes the part's words.  256 predecessors are examined at a time: with several hundred
+// parts in flight most of them hold only their own sum yet.
+__device__ __forceinline__ uint32_t block_look_back(uint64_t *words, int part, uint32_t own, uint32_t *status) {
+    __shared__ uint32_t s_sum[kScanThreads / 32];
+    __shared__ bool s_has[kScanThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) store_word(words + part, (part == 0 ? kPrefix : kAggregate) | own);
+    uint32_t sum = 0;
+    bool found = part == 0;
+    for (int p = part - 1; !found; p -= kScanThreads) {  // (block-uniform)
+        const int q = p - (int)threadIdx.x;
+        uint64_t w = kPrefix;  // before the first part: an empty prefix
+        if (q >= 0) w = wait_word(words + q, load_word(words + q), status);
+        const uint32_t pre = __ballot_sync(SG_FULL_MASK, (w & kPrefix) != 0);
+        // lanes past the nearest prefix do not count
+        const int stop = pre ? __ffs(pre) - 1 : 31;
+        const uint32_t ws = __reduce_add_sync(SG_FULL_MASK, lane <= stop ? (uint32_t)w : 0u);
+        if (lane == 0) {
+            s_sum[warp] = ws;
+            s_has[warp] = pre != 0;
+        }
+        __syncthreads();
+        for (int i = 0; i < kScanThreads / 32 && !found; ++i) {
+            sum += s_sum[i];
+            found = s_has[i];
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0 && part > 0) store_word(words + part, kPrefix | (uint64_t)(sum + own));
+    return sum;
+}
+
+// The same for one thread whose sum has been published in words[part * stride] (a digit of a
+// radix pass): four predecessors' words are requested at a time.
+__device__ __forceinline__ uint32_t look_back(const uint64_t *words, int stride, int part, uint32_t *status) {
+    uint32_t sum = 0;
+    for (int p = part - 1; p >= 0; p -= 4) {
+        uint64_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = p - i >= 0 ? load_word(words + (size_t)(p - i) * stride) : kPrefix;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (p - i < 0) return sum;
+            const uint64_t v = wait_word(words + (size_t)(p - i) * stride, w[i], status);
+            sum += (uint32_t)v;
+            if (v & kPrefix) return sum;
+        }
+    }
+    return sum;
+}
+
+// The next part of a kernel's input (block-uniform).
+__device__ __forceinline__ int next_part(int *counter) {
+    __shared__ int s_part;
+    __syncthreads();
+    if (threadIdx.x == 0) s_part = atomicAdd(counter, 1);
+    __syncthreads();
+    return s_part;
+}
+
+// Adds a block's digit counts in shared memory (n words) to the global histogram.
+__device__ __forceinline__ void flush_hist(const uint32_t *s_h, int n, uint32_t *hist) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += kScanThreads)
+        if (s_h[i]) atomicAdd(hist + i, s_h[i]);
+}
 
 __device__ __forceinline__ uint32_t rect_tiles(uint2 r) {
     const uint32_t tx0 = r.x & 0xffffu, ty0 = r.x >> 16, tx1 = r.y & 0xffffu, ty1 = r.y >> 16;
@@ -94,64 +184,32 @@ __device__ __forceinline__ uint32_t rect_rows(uint2 r) {
     return rect_tiles(r) ? ty1 - ty0 : 0u;
 }
 
-struct SortedRowCount {  // tile rows of the rectangle of the record at sorted position i
-    const uint2 *rect;
-    const uint32_t *rec;
-    __device__ uint32_t operator()(int i) const { return rect_rows(rect[rec[i]]); }
-};
-
-template <class F>
-__global__ void scan_reduce_kernel(F f, const int *n_ptr, int n_host, uint32_t *bsum, int G) {
-    pdl_begin();
-    const int n = n_ptr ? *n_ptr : n_host;
-    int beg, end;
-    block_range(n, G, blockIdx.x, beg, end);
-    uint32_t s = 0;
-    for (int i = beg + threadIdx.x; i < end; i += kScanThreads) s += f(i);
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(SG_FULL_MASK, s, o);
-    __shared__ uint32_t sw[kScanThreads / 32];
-    if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t t = 0;
-        for (int w = 0; w < kScanThreads / 32; ++w) t += sw[w];
-        bsum[blockIdx.x] = t;
-    }
-}
-
-// One block: exclusive scan of G block sums (G <= 4096); writes the grand total.
-__global__ void scan_blocks_kernel(uint32_t *bsum, int G, int *total) {
-    pdl_begin();
-    uint32_t run = 0;
-    for (int base = 0; base < G; base += kScanThreads) {
-        const int i = base + threadIdx.x;
-        const uint32_t v = i < G ? bsum[i] : 0u;
-        uint32_t tot;
-        const uint32_t ex = block_exclusive_scan(v, tot);
-        if (i < G) bsum[i] = ex + run;
-        run += tot;
-    }
-    if (threadIdx.x == 0) *total = (int)run;
-}
-
-// Apply for the compaction: write (depth bits, record) of every visible record.  Each thread
-// takes 8 consecutive records per round (two 16-byte loads of their rectangles when the
-// array is 16-byte aligned), so a round of the block covers 2048 records with one block scan
-// and all of its loads in flight together.
+// Compaction: (depth bits, record) of every visible record, in record order, and the four
+// 8-bit digit histograms of the depth bits.  Each thread takes 8 consecutive records (two
+// 16-byte loads of their rectangles when the array is 16-byte aligned), so a part is 2048
+// records with one block scan and all of its loads in flight together.
 constexpr int kCompactPerThread = 8;
-__global__ void compact_apply_kernel(const uint2 *__restrict__ rect, const float4 *__restrict__ geo,
-                                     int n, const uint32_t *__restrict__ boff, int G,
-                                     uint32_t *__restrict__ key, uint32_t *__restrict__ val) {
+constexpr int kCompactPart = kScanThreads * kCompactPerThread;
+__global__ void __launch_bounds__(kScanThreads) compact_kernel(const uint2 *__restrict__ rect,
+                                                               const float4 *__restrict__ geo, int n,
+                                                               uint64_t *__restrict__ words, int *__restrict__ counter,
+                                                               uint32_t *__restrict__ key, uint32_t *__restrict__ val,
+                                                               int *__restrict__ total, uint32_t *__restrict__ hist,
+                                                               int *__restrict__ instances,
+                                                               uint32_t *__restrict__ status) {
     pdl_begin();
     constexpr int E = kCompactPerThread;
-    int beg, end;
-    block_range(n, G, blockIdx.x, beg, end);
+    __shared__ uint32_t s_h[4 * 256];
+    __shared__ uint32_t s_key[kCompactPart], s_val[kCompactPart];
+    // (written by the last part of the emission, which has none without slots)
+    if (blockIdx.x == 0 && threadIdx.x == 0) *instances = 0;
+    for (int i = threadIdx.x; i < 4 * 256; i += kScanThreads) s_h[i] = 0;
     const bool vec = (reinterpret_cast<uintptr_t>(rect) & 15u) == 0;
-    uint32_t run = boff[blockIdx.x];
-    for (int base = beg; base < end; base += kScanThreads * E) {
-        const int i0 = base + (int)threadIdx.x * E;  // a multiple of 8 (beg is one of 256)
+    const int parts = (n + kCompactPart - 1) / kCompactPart;
+    for (int part; (part = next_part(counter)) < parts;) {
+        const int i0 = part * kCompactPart + (int)threadIdx.x * E;
         uint2 r[E];
-        if (vec && i0 + E <= end) {
+        if (vec && i0 + E <= n) {
             const uint4 *p4 = reinterpret_cast<const uint4 *>(rect + i0);
 #pragma unroll
             for (int q = 0; q < E / 2; ++q) {
@@ -161,7 +219,7 @@ __global__ void compact_apply_kernel(const uint2 *__restrict__ rect, const float
             }
         } else {
 #pragma unroll
-            for (int q = 0; q < E; ++q) r[q] = i0 + q < end ? rect[i0 + q] : make_uint2(0, 0);
+            for (int q = 0; q < E; ++q) r[q] = i0 + q < n ? rect[i0 + q] : make_uint2(0, 0);
         }
         uint32_t f = 0, bits = 0;
 #pragma unroll
@@ -170,20 +228,40 @@ __global__ void compact_apply_kernel(const uint2 *__restrict__ rect, const float
                 bits |= 1u << q;
                 ++f;
             }
-        float dep[E];
+        uint32_t dep[E];
 #pragma unroll
-        for (int q = 0; q < E; ++q) dep[q] = ((bits >> q) & 1u) ? geo[2 * (size_t)(i0 + q)].z : 0.f;
+        for (int q = 0; q < E; ++q)
+            dep[q] = ((bits >> q) & 1u) ? __float_as_uint(geo[2 * (size_t)(i0 + q)].z) : 0u;
         uint32_t tot;
-        uint32_t o = run + block_exclusive_scan(f, tot);
+        uint32_t o = block_exclusive_scan(f, tot);
 #pragma unroll
         for (int q = 0; q < E; ++q)
             if ((bits >> q) & 1u) {
-                key[o] = __float_as_uint(dep[q]);
-                val[o] = (uint32_t)(i0 + q);
+                s_key[o] = dep[q];
+                s_val[o] = (uint32_t)(i0 + q);
                 ++o;
             }
-        run += tot;
+        const uint32_t off = block_look_back(words, part, tot, status);
+        if (part == parts - 1 && threadIdx.x == 0) *total = (int)(off + tot);
+        __syncthreads();
+        for (uint32_t j = threadIdx.x; j < ((tot + 31) & ~31u); j += kScanThreads) {
+            const bool in = j < tot;
+            const uint32_t d = in ? s_key[j] : 0u;
+            if (in) {
+                key[off + j] = d;
+                val[off + j] = s_val[j];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) atomicAdd(&s_h[256 * q + ((d >> (8 * q)) & 255u)], 1u);
+            }
+            // the top digit (sign and exponent) takes a handful of values: one add per value and warp
+            const uint32_t top = in ? d >> 24 : 256u;
+            const uint32_t peers = __match_any_sync(SG_FULL_MASK, top);
+            if (in && (threadIdx.x & 31) == (uint32_t)(__ffs(peers) - 1))
+                atomicAdd(&s_h[256 * 3 + top], (uint32_t)__popc(peers));
+        }
+        // (next_part's barriers order these reads before the next part's writes)
     }
+    flush_hist(s_h, 4 * 256, hist);
 }
 
 // The columns of a tile row that the record's alpha >= alpha_min region reaches.  The
@@ -360,88 +438,128 @@ __device__ __forceinline__ uint32_t half_mask(uint32_t half, uint32_t q) {
 }
 
 // The (record, tile row) slots: the tile rows of every depth-sorted record's rectangle,
-// record after record; P[i] is the first slot of sorted record i.  The two culling passes
-// split the S slots evenly over their Gc blocks (a multiple of 256 slots each), so that the
-// few near records with huge rectangles do not serialise one warp.
-__device__ __forceinline__ uint32_t slot_block_size(uint32_t S, int Gc) {
-    const uint32_t chunks = (S + kScanThreads - 1) / kScanThreads;
-    const uint32_t per = (chunks + (uint32_t)Gc - 1) / (uint32_t)Gc;
-    return (per > 0 ? per : 1u) * kScanThreads;
-}
-
-// P[i] = boff[block] + exclusive scan of the rectangle row counts, and for every block of the
-// slot partition the record that owns its first slot.
-__global__ void slot_prefix_kernel(const uint2 *__restrict__ rect, const uint32_t *__restrict__ rec,
-                                   const int *__restrict__ m_ptr, const uint32_t *__restrict__ boff, int G,
-                                   const int *__restrict__ s_ptr, int Gc, uint32_t *__restrict__ P,
-                                   uint32_t *__restrict__ first_rec) {
+// record after record; P[i] is the first slot of sorted record i and first_rec[b] the record
+// that owns slot 256 b (for the first kMaxChunks chunks of 256 slots).
+constexpr int kMaxChunks = 1 << 16;
+__global__ void __launch_bounds__(kScanThreads) slot_prefix_kernel(const uint2 *__restrict__ rect,
+                                                                   const uint32_t *__restrict__ rec,
+                                                                   const int *__restrict__ m_ptr,
+                                                                   uint64_t *__restrict__ words, int *__restrict__ counter,
+                                                                   uint32_t *__restrict__ P,
+                                                                   uint32_t *__restrict__ first_rec,
+                                                                   int *__restrict__ total, uint32_t *__restrict__ status) {
     pdl_begin();
+    constexpr int E = kCompactPerThread;
     const int n = *m_ptr;
-    const uint64_t per = slot_block_size((uint32_t)*s_ptr, Gc);
-    int beg, end;
-    block_range(n, G, blockIdx.x, beg, end);
-    uint32_t run = boff[blockIdx.x];
-    for (int base = beg; base < end; base += kScanThreads) {
-        const int i = base + threadIdx.x;
-        const uint32_t c = i < end ? rect_rows(rect[rec[i]]) : 0u;
-        uint32_t tot;
-        const uint32_t ex = block_exclusive_scan(c, tot);
-        if (i < end) {
-            const uint64_t p = run + ex;
-            P[i] = (uint32_t)p;
-            for (uint64_t b = (p + per - 1) / per; b * per < p + c && b < (uint64_t)Gc; ++b) first_rec[b] = (uint32_t)i;
+    const int parts = (n + kCompactPart - 1) / kCompactPart;
+    for (int part; (part = next_part(counter)) < parts;) {
+        // thread t takes records base + 32 (8 warp + q) + lane: coalesced loads, and the scan runs
+        // over warps' blocks of 256 records
+        const int lane = threadIdx.x & 31, base = part * kCompactPart + (int)(threadIdx.x >> 5) * (32 * E);
+        uint32_t c[E], incl[E], sum = 0;
+#pragma unroll
+        for (int q = 0; q < E; ++q) {
+            const int i = base + 32 * q + lane;
+            c[q] = i < n ? rect_rows(rect[rec[i]]) : 0u;
         }
-        run += tot;
+#pragma unroll
+        for (int q = 0; q < E; ++q) {
+            uint32_t v = c[q];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(SG_FULL_MASK, v, o);
+                if (lane >= o) v += t;
+            }
+            incl[q] = sum + v;
+            sum += __shfl_sync(SG_FULL_MASK, v, 31);
+        }
+        uint32_t tot;
+        const uint32_t ex = block_exclusive_scan(lane == 0 ? sum : 0u, tot);
+        const uint32_t off = block_look_back(words, part, tot, status) + __shfl_sync(SG_FULL_MASK, ex, 0);
+        if (part == parts - 1 && threadIdx.x == 0) *total = (int)(off + tot);
+#pragma unroll
+        for (int q = 0; q < E; ++q) {
+            const int i = base + 32 * q + lane;
+            if (i >= n) continue;
+            const uint64_t p = off + incl[q] - c[q];
+            P[i] = (uint32_t)p;
+            for (uint64_t b = (p + 255) / 256; b * 256 < p + c[q] && b < (uint64_t)kMaxChunks; ++b)
+                first_rec[b] = (uint32_t)i;
+        }
     }
 }
 
-// The culling passes over the slot partition.  Thread t of a 256-slot chunk takes slot
-// s = c0 + t: its record is found by a binary search over the prefixes of the (at most 256)
-// records that can own the chunk, staged in shared memory; the row's footprint span gives
-// the contiguous run of kept tile columns.
-//   COUNT: adds up the kept tiles of the block's slots (kbsum[block]); when the slots fit the
-//          slot cache (S <= capacity), also stores each slot's first kept tile and count.
-//   EMIT:  writes (global tile id, record) for the kept tiles, column by column, at
-//          kbsum[block] (the scanned block offset) plus the block's exclusive scan of the
-//          kept counts, i.e. in (record, row, column) order; the runs come from the slot
-//          cache when the count pass filled it, else from the same span computation.
+// The sorted record that owns slot s: the last i with P[i] <= s among records that have slots
+// (all records in the lists have at least one row).
+__device__ __forceinline__ int slot_owner(const uint32_t *__restrict__ P, int n, uint32_t s) {
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const int mid = lo + (hi - lo + 1) / 2;
+        if (P[mid] <= s) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+// Digits of the tile sort's passes.
+struct Digits {
+    int n;
+    int shift[4];
+    uint32_t mask[4];
+};
+
+// Culling and emission over the slots, in chunks of 256 (a thread's slot each).  A part is one
+// chunk for small inputs; for larger ones it is several, at most two parts per block (one chunk
+// at a time measured 490 against 360 us on the batched workload), counted before the part's
+// place is known and emitted afterwards from the slot cache (the tile sort's idle ping-pong
+// buffers and the output tile ids, when they hold every slot).  A slot's record is found by a binary search
+// over the prefixes of the (at most 256) records that can own the chunk, staged in shared
+// memory; the row's footprint span gives the contiguous run of kept tile columns.  The part's
+// kept counts give its instances' place by the chained scan, and consecutive threads write
+// consecutive instances (global tile id, record), each finding its slot by a binary search
+// over the slots' offsets: (record, row, column) order.  The few near records with huge
+// rectangles are spread over many parts.  Also counted here: the tile ids' digit histograms;
+// and the words of the tile sort's first pass are cleared for the parts that start among the
+// emitted instances (sweep_part each).
 // HALVES: the rule runs per half tile row (slot_run) and the emitted records carry each
 // tile's half mask in bits 30-31.
-template <bool EMIT, bool HALVES>
-__global__ void __launch_bounds__(kScanThreads, 6) cull_pass_kernel(const uint2 *__restrict__ rect, const float4 *__restrict__ geo,
-                                 const float2 *__restrict__ ext, const uint32_t *__restrict__ rec,
-                                 const int *__restrict__ m_ptr, const int *__restrict__ s_ptr,
-                                 const uint32_t *__restrict__ P, const uint32_t *__restrict__ first_rec, int Gc,
-                                 int N, const sg_view *__restrict__ views, int n_views, int tile_w, int tile_h,
-                                 uint32_t *__restrict__ kbsum, uint32_t *__restrict__ tkey, uint32_t *__restrict__ tval,
-                                 uint32_t *__restrict__ slot_tf, uint32_t *__restrict__ slot_cnt,
-                                 uint32_t *__restrict__ slot_half, int capacity, uint32_t *__restrict__ status) {
+template <bool HALVES>
+__global__ void __launch_bounds__(kScanThreads, 6) cull_kernel(
+    const uint2 *__restrict__ rect, const float4 *__restrict__ geo, const float2 *__restrict__ ext,
+    const uint32_t *__restrict__ rec, const int *__restrict__ m_ptr, const int *__restrict__ s_ptr,
+    const uint32_t *__restrict__ P, const uint32_t *__restrict__ first_rec, uint64_t *__restrict__ words,
+    int *__restrict__ counter, int N, const sg_view *__restrict__ views, int n_views, int tile_w, int tile_h,
+    uint32_t *__restrict__ tkey, uint32_t *__restrict__ tval, int capacity, int *__restrict__ total, Digits dg,
+    uint32_t *__restrict__ hist, uint64_t *__restrict__ sweep_words, int sweep_part, uint32_t *__restrict__ slot_tf,
+    uint32_t *__restrict__ slot_cnt, uint32_t *__restrict__ slot_half, uint32_t *__restrict__ status) {
     pdl_begin();
-    __shared__ uint32_t s_P[kScanThreads];
-    __shared__ uint32_t s_ex[EMIT ? kScanThreads : 1], s_tf[EMIT ? kScanThreads : 1], s_or[EMIT ? kScanThreads : 1],
-        s_hf[EMIT && HALVES ? kScanThreads : 1];
+    __shared__ uint32_t s_P[kScanThreads], s_ex[kScanThreads], s_tf[kScanThreads], s_or[kScanThreads],
+        s_hf[HALVES ? kScanThreads : 1];
+    __shared__ uint32_t s_h[4 * 256];
     __shared__ int s_next;
     __shared__ int4 s_vw[SG_MAX_VIEWS];  // (W, H, tile_offset, tiles_x) of each view-level
     for (int v = threadIdx.x; v < n_views; v += kScanThreads)
         s_vw[v] = make_int4(views[v].W, views[v].H, views[v].tile_offset, views[v].tiles_x);
+    for (int i = threadIdx.x; i < 4 * 256; i += kScanThreads) s_h[i] = 0;
     const int n = *m_ptr;
     const uint32_t S = (uint32_t)*s_ptr;
-    const uint64_t per = slot_block_size(S, Gc);
-    const uint64_t s0 = (uint64_t)blockIdx.x * per;
-    const uint64_t s1 = min((uint64_t)S, s0 + per);
+    const int chunks = (int)(((uint64_t)S + 255) / 256);
+    // chunks of a part: at most two parts per block, one chunk for small inputs
+    const int per = max(1, max((chunks + kMaxChunks - 1) / kMaxChunks, (chunks + 2 * (int)gridDim.x - 1) / (2 * (int)gridDim.x)));
     const bool cached = S <= (uint32_t)capacity;  // the slot cache holds every slot
-    uint32_t kept = 0;
-    uint32_t run = EMIT ? kbsum[blockIdx.x] : 0u;
+    const int parts = (chunks + per - 1) / per;
     bool overflow = false;
-    int ic = s0 < s1 ? (int)first_rec[blockIdx.x] : 0;
-    for (uint64_t c0 = s0; c0 < s1; c0 += kScanThreads) {  // block-uniform trip count
+    // the slot c0 + threadIdx.x, c0 in sorted record ic: its kept tiles [tfirst, tfirst + count),
+    // from the slot cache when an earlier pass over the part stored them (use), or stored there
+    auto slot = [&](uint64_t c0, int ic, int &k, uint32_t &orec, uint32_t &tfirst, uint32_t &half, bool use,
+                    bool store) {
         const int j = ic + (int)threadIdx.x;
         s_P[threadIdx.x] = j < n ? P[j] : 0xffffffffu;
         __syncthreads();
+        k = 0;
+        orec = tfirst = half = 0;
+        uint32_t cnt = 0;
         const uint32_t s = (uint32_t)(c0 + threadIdx.x);
-        uint32_t cnt = 0, orec = 0, tfirst = 0, half = 0;
-        int k = 0;
-        if (c0 + threadIdx.x < s1) {
+        if (c0 + threadIdx.x < S) {
             int lo = 0, hi = kScanThreads - 1;  // the last k with s_P[k] <= s (s_P[0] <= c0)
             while (lo < hi) {
                 const int mid = (lo + hi + 1) >> 1;
@@ -449,84 +567,124 @@ __global__ void __launch_bounds__(kScanThreads, 6) cull_pass_kernel(const uint2 
             }
             k = lo;
             orec = rec[ic + k];
-        }
-        if (EMIT && cached) {
-            if (c0 + threadIdx.x < s1) {
-                tfirst = __ldcs(slot_tf + s);
-                cnt = __ldcs(slot_cnt + s);
-                if (HALVES) half = __ldcs(slot_half + s);
-            }
-        } else if (c0 + threadIdx.x < s1) {
-            const uint2 rc = rect[orec];
-            const int tx0 = (int)(rc.x & 0xffffu), tx1 = (int)(rc.y & 0xffffu);
-            const int ty = (int)(rc.x >> 16) + (int)(s - s_P[k]);
-            const int4 vw = s_vw[orec / (uint32_t)N];
-            const int Y0 = ty * tile_h;
-            const int Y1 = min(Y0 + tile_h - 1, vw.y - 1);
-            int tx_a = tx1;
-            if constexpr (HALVES) {
-                const SlotRun sr = slot_run(geo[2 * (size_t)orec], geo[2 * (size_t)orec + 1], ext[orec].x, Y0, Y1,
-                                            tile_h, tx0, tx1, tile_w, vw.x);
-                cnt = (uint32_t)sr.cnt;
-                half = sr.half;
-                tx_a = sr.a;
+            if (use) {
+                tfirst = slot_tf[s];
+                cnt = slot_cnt[s];
+                if (HALVES) half = slot_half[s];
             } else {
-                RowSpan rs;
-                if (row_span(geo[2 * (size_t)orec], geo[2 * (size_t)orec + 1], ext[orec].x, Y0, Y1, rs)) {
-                    // the kept columns are contiguous
-                    int tb;
-                    span_run(rs, tx0, tx1, tile_w, vw.x, tx_a, tb);
-                    cnt = (uint32_t)(tb - tx_a);
-                    if (!cnt) tx_a = tx1;
-                }
-            }
-            tfirst = (uint32_t)vw.z + (uint32_t)ty * (uint32_t)vw.w + (uint32_t)tx_a;
-            if (!EMIT && cached) {
-                slot_tf[s] = tfirst;
-                slot_cnt[s] = cnt;
-                if (HALVES) slot_half[s] = half;
-            }
-        }
-        if (!EMIT) {
-            kept += cnt;
-        } else {
-            // the chunk's instances [run, run + tot): consecutive threads write consecutive
-            // instances, each finding its slot by a binary search over the slots' offsets
-            uint32_t tot;
-            const uint32_t ex = block_exclusive_scan(cnt, tot);
-            s_ex[threadIdx.x] = ex;
-            s_tf[threadIdx.x] = tfirst;
-            s_or[threadIdx.x] = orec;
-            if (HALVES) s_hf[threadIdx.x] = half;
-            __syncthreads();
-            for (uint32_t o = threadIdx.x; o < tot; o += kScanThreads) {
-                int lo = 0, hi = kScanThreads - 1;  // the last slot t with s_ex[t] <= o
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (s_ex[mid] <= o) lo = mid; else hi = mid - 1;
-                }
-                const uint32_t g = run + o;
-                if (g < (uint32_t)capacity) {
-                    const uint32_t q = o - s_ex[lo];
-                    tkey[g] = s_tf[lo] + q;
-                    // (with halves, records are below 2^30: checked by the caller)
-                    tval[g] = HALVES ? s_or[lo] | (half_mask(s_hf[lo], q) << 30) : s_or[lo];
+                const uint2 rc = rect[orec];
+                const int tx0 = (int)(rc.x & 0xffffu), tx1 = (int)(rc.y & 0xffffu);
+                const int ty = (int)(rc.x >> 16) + (int)(s - s_P[k]);
+                const int4 vw = s_vw[orec / (uint32_t)N];
+                const int Y0 = ty * tile_h;
+                const int Y1 = min(Y0 + tile_h - 1, vw.y - 1);
+                int tx_a = tx1;
+                if constexpr (HALVES) {
+                    const SlotRun sr = slot_run(geo[2 * (size_t)orec], geo[2 * (size_t)orec + 1], ext[orec].x, Y0, Y1,
+                                                tile_h, tx0, tx1, tile_w, vw.x);
+                    cnt = (uint32_t)sr.cnt;
+                    half = sr.half;
+                    tx_a = sr.a;
                 } else {
-                    overflow = true;
+                    RowSpan rs;
+                    if (row_span(geo[2 * (size_t)orec], geo[2 * (size_t)orec + 1], ext[orec].x, Y0, Y1, rs)) {
+                        // the kept columns are contiguous
+                        int tb;
+                        span_run(rs, tx0, tx1, tile_w, vw.x, tx_a, tb);
+                        cnt = (uint32_t)(tb - tx_a);
+                        if (!cnt) tx_a = tx1;
+                    }
+                }
+                tfirst = (uint32_t)vw.z + (uint32_t)ty * (uint32_t)vw.w + (uint32_t)tx_a;
+                if (store) {
+                    slot_tf[s] = tfirst;
+                    slot_cnt[s] = cnt;
+                    if (HALVES) slot_half[s] = half;
                 }
             }
-            run += tot;
         }
         // the next chunk starts in the record that owns this chunk's last slot
         if (threadIdx.x == kScanThreads - 1) s_next = ic + k;
+        return cnt;
+    };
+    // the chunk's instances [run, run + tot)
+    auto emit = [&](uint32_t run, uint32_t ex, uint32_t cnt, uint32_t tot, uint32_t orec, uint32_t tfirst,
+                    uint32_t half) {
+        // the upper digits are the same over most of a run: counted per slot, the lowest per
+        // instance below (per instance they would serialise on a few shared words)
+        const uint64_t at = (uint64_t)run + ex;
+        const uint32_t kept = at < (uint64_t)capacity ? (uint32_t)min((uint64_t)cnt, (uint64_t)capacity - at) : 0u;
+#pragma unroll
+        for (int d = 1; d < 4; ++d) {
+            if (d >= dg.n) break;
+            for (uint32_t t = tfirst, left = kept; left > 0;) {
+                const uint32_t m = min(left, (((t >> dg.shift[d]) + 1u) << dg.shift[d]) - t);
+                atomicAdd(&s_h[256 * d + ((t >> dg.shift[d]) & dg.mask[d])], m);
+                t += m;
+                left -= m;
+            }
+        }
+        s_ex[threadIdx.x] = ex;
+        s_tf[threadIdx.x] = tfirst;
+        s_or[threadIdx.x] = orec;
+        if (HALVES) s_hf[threadIdx.x] = half;
         __syncthreads();
-        ic = s_next;
+        for (uint32_t o = threadIdx.x; o < tot; o += kScanThreads) {
+            int lo = 0, hi = kScanThreads - 1;  // the last slot t with s_ex[t] <= o
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (s_ex[mid] <= o) lo = mid; else hi = mid - 1;
+            }
+            const uint32_t g = run + o;
+            if (g < (uint32_t)capacity) {
+                const uint32_t q = o - s_ex[lo], t = s_tf[lo] + q;
+                tkey[g] = t;
+                // (with halves, records are below 2^30: checked by the caller)
+                tval[g] = HALVES ? s_or[lo] | (half_mask(s_hf[lo], q) << 30) : s_or[lo];
+                atomicAdd(&s_h[t & dg.mask[0]], 1u);
+            } else {
+                overflow = true;
+            }
+        }
+        __syncthreads();
+    };
+    for (int part; (part = next_part(counter)) < parts;) {
+        const int b0 = part * per, b1 = min(chunks, b0 + per);
+        const int i0 = b0 < kMaxChunks ? (int)first_rec[b0] : slot_owner(P, n, (uint32_t)b0 * 256u);
+        int k;
+        uint32_t orec, tfirst, half, run, sum = 0, tot;
+        if (per == 1) {
+            const uint32_t cnt = slot((uint64_t)b0 * 256, i0, k, orec, tfirst, half, false, false);
+            const uint32_t ex = block_exclusive_scan(cnt, tot);
+            run = block_look_back(words, part, tot, status);
+            sum = tot;
+            emit(run, ex, cnt, tot, orec, tfirst, half);
+        } else {
+            int ic = i0;
+            uint32_t kept = 0;
+            for (int b = b0; b < b1; ++b) {
+                kept += slot((uint64_t)b * 256, ic, k, orec, tfirst, half, false, cached);
+                __syncthreads();
+                ic = s_next;
+            }
+            block_exclusive_scan(kept, sum);
+            run = block_look_back(words, part, sum, status);
+            ic = i0;
+            uint32_t at = run;
+            for (int b = b0; b < b1; ++b) {
+                const uint32_t cnt = slot((uint64_t)b * 256, ic, k, orec, tfirst, half, cached, false);
+                const uint32_t ex = block_exclusive_scan(cnt, tot);
+                ic = s_next;
+                emit(at, ex, cnt, tot, orec, tfirst, half);
+                at += tot;
+            }
+        }
+        if (part == parts - 1 && threadIdx.x == 0) *total = (int)(run + sum);
+        const uint64_t end = min((uint64_t)run + sum, (uint64_t)capacity);
+        for (uint64_t q = ((uint64_t)run + sweep_part - 1) / sweep_part; q * sweep_part < end; ++q)
+            sweep_words[q * 256 + threadIdx.x] = 0;
     }
-    if (!EMIT) {
-        uint32_t tot;
-        block_exclusive_scan(kept, tot);
-        if (threadIdx.x == 0) kbsum[blockIdx.x] = tot;
-    }
+    flush_hist(s_h, 256 * dg.n, hist);
     if (overflow) atomicOr(status, SG_STATUS_CAPACITY);
 }
 
@@ -534,138 +692,53 @@ __global__ void __launch_bounds__(kScanThreads, 6) cull_pass_kernel(const uint2 
 // Stable LSD radix sort of (uint32 key, uint32 value) pairs, 8-bit digits (or fewer).
 // ---------------------------------------------------------------------------------------
 
-// Key sources of the radix sort: pairs held in arrays, or the tiles' list lengths.
-struct ArrayPairs {
-    const uint32_t *k, *v;
-    // each pair is read once per kernel: evict-first loads, which leave L2 to the scatter's
-    // partly written output lines
-    __device__ uint32_t key(int i) const { return __ldcs(k + i); }
-    __device__ uint32_t val(int i) const { return __ldcs(v + i); }
-};
-// key = 63 - bucket of the tile's instance count n (bucket 0 for n = 0, else
-// 1 + 2 floor(log2 n) + the bit below the leading one): descending length, 6 bits
-struct TileLengthKeys {
-    const int2 *ranges;
-    __device__ uint32_t key(int i) const {
-        const int2 r = ranges[i];
-        const uint32_t n = (uint32_t)max(r.y - r.x, 0);
-        if (n == 0) return 63u;
-        const int lz = 31 - __clz(n);
-        const uint32_t sub = lz >= 1 ? (n >> (lz - 1)) & 1u : 0u;
-        return 63u - (1u + 2u * (uint32_t)lz + sub);
-    }
-    __device__ uint32_t val(int i) const { return (uint32_t)i; }
-};
-
-// Radix digits of one pass: up to 8 bits (256 buckets) or 9 bits (512 buckets); each of
-// the 256 threads of a block owns ND / 256 consecutive buckets.
-template <class Src, int ND>
-__global__ void rs_hist_kernel(Src src, const int *__restrict__ n_ptr, int cap, int shift, uint32_t mask,
-                               uint32_t *__restrict__ hist, int G) {
-    pdl_begin();
-    constexpr int DPT = ND / kScanThreads;
-    __shared__ uint32_t h[ND];
-#pragma unroll
-    for (int q = 0; q < DPT; ++q) h[threadIdx.x * DPT + q] = 0;
-    __syncthreads();
-    const int n = n_ptr ? min(*n_ptr, cap) : cap;
-    int beg, end;
-    block_range(n, G, blockIdx.x, beg, end);
-    for (int i = beg + threadIdx.x; i < end; i += kScanThreads)
-        atomicAdd(&h[(src.key(i) >> shift) & mask], 1u);
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < DPT; ++q) hist[(threadIdx.x * DPT + q) * G + blockIdx.x] = h[threadIdx.x * DPT + q];
-}
-
-// Block d: exclusive scan of digit d's per-block counts; totals[d] = digit d's count.
-__global__ void rs_digit_scan_kernel(uint32_t *__restrict__ hist, uint32_t *__restrict__ totals, int G) {
-    pdl_begin();
-    const int d = blockIdx.x;
-    uint32_t run = 0;
-    for (int base = 0; base < G; base += kScanThreads) {
-        const int i = base + threadIdx.x;
-        const uint32_t v = i < G ? hist[d * G + i] : 0u;
-        uint32_t tot;
-        const uint32_t ex = block_exclusive_scan(v, tot);
-        if (i < G) hist[d * G + i] = ex + run;
-        run += tot;
-    }
-    if (threadIdx.x == 0) totals[d] = run;
-}
-
-// Exclusive scan over ND buckets held DPT per thread (consecutive), block-wide.
-template <int DPT>
-__device__ __forceinline__ void bucket_exclusive_scan(const uint32_t (&v)[DPT], uint32_t (&ex)[DPT]) {
-    uint32_t sum = 0;
-#pragma unroll
-    for (int q = 0; q < DPT; ++q) sum += v[q];
-    uint32_t tot;
-    uint32_t run = block_exclusive_scan(sum, tot);
-#pragma unroll
-    for (int q = 0; q < DPT; ++q) {
-        ex[q] = run;
-        run += v[q];
-    }
-}
-
-// Scatter of one digit pass.  Each block walks its input range in chunks of 256 IPT
-// elements; warp w owns the chunk's elements [32 IPT w, 32 IPT (w + 1)), lane l element
-// 32 it + l of them.  Ranking needs no block barrier per element row: every warp ranks its
-// own elements against a warp-private digit count (warp match_any + the lanes below), one
-// block pass turns the per-warp counts into per-digit offsets, the chunk is reordered by
-// digit in shared memory, and consecutive threads store consecutive elements of one digit
-// run (coalesced stores instead of one scattered sector per element).
-template <int ND>
-__host__ __device__ constexpr int scatter_ipt() { return 12; }
-
-template <class Src, int ND>
-__global__ void __launch_bounds__(kScanThreads, 4) rs_scatter_kernel(
-    Src src, uint32_t *__restrict__ kout,
+// One digit pass (digits of at most 8 bits, histogram given).  A part is 256 IPT elements; warp
+// w owns the part's elements [32 IPT w, 32 IPT (w + 1)), lane l element 32 it + l of them.
+// Ranking needs no block barrier per element row: every warp ranks its own elements against a
+// warp-private digit count (warp match_any + the lanes below), one block pass turns the
+// per-warp counts into per-digit offsets, thread d publishes digit d's count and looks back for
+// its prefix while the part is reordered by digit in shared memory, and consecutive threads
+// store consecutive elements of one digit run (coalesced stores instead of one scattered sector
+// per element).  clear: the next pass's words, cleared for the parts this pass handles.
+constexpr int kSweepIpt = 12;
+constexpr int kSweepPart = kScanThreads * kSweepIpt;
+__global__ void __launch_bounds__(kScanThreads, 4) sweep_kernel(
+    const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin, uint32_t *__restrict__ kout,
     uint32_t *__restrict__ vout, const int *__restrict__ n_ptr, int cap, int shift, uint32_t mask,
-    const uint32_t *__restrict__ hist, const uint32_t *__restrict__ totals, int G) {
+    const uint32_t *__restrict__ hist, uint64_t *__restrict__ words, uint64_t *__restrict__ clear,
+    int *__restrict__ counter, uint32_t *__restrict__ status) {
     pdl_begin();
-    constexpr int kWarps = kScanThreads / 32;
-    constexpr int DPT = ND / kScanThreads;  // digits per thread: tid * DPT + q
-    constexpr int IPT = scatter_ipt<ND>();
-    constexpr int CH = kScanThreads * IPT;
-    __shared__ uint32_t run[ND];            // global position of the next element of each digit
-    __shared__ uint32_t loc[ND];            // first slot of each digit in the reordered chunk
-    __shared__ uint32_t wcnt[kWarps][ND];   // per-warp digit counts, then per-warp offsets
+    constexpr int kWarps = kScanThreads / 32, IPT = kSweepIpt, CH = kSweepPart;
+    __shared__ uint32_t to[256];            // output position of the part's slot 0 if it had digit d
+    __shared__ uint32_t loc[256];           // first slot of each digit in the reordered part
+    __shared__ uint32_t wcnt[kWarps][256];  // per-warp digit counts, then per-warp offsets
     __shared__ uint32_t skey[CH], sval[CH];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // digit base = exclusive scan of the digit totals (+ this block's offset)
-    {
-        uint32_t t[DPT], ex[DPT];
-#pragma unroll
-        for (int q = 0; q < DPT; ++q) t[q] = totals[tid * DPT + q];
-        bucket_exclusive_scan<DPT>(t, ex);
-#pragma unroll
-        for (int q = 0; q < DPT; ++q) run[tid * DPT + q] = ex[q] + hist[(tid * DPT + q) * G + blockIdx.x];
-    }
-    const int n = n_ptr ? min(*n_ptr, cap) : cap;
-    int beg, end;
-    block_range(n, G, blockIdx.x, beg, end);
+    const int n = min(*n_ptr, cap);
+    const int parts = (int)(((int64_t)n + CH - 1) / CH);
+    uint32_t unused;
+    const uint32_t first = block_exclusive_scan(hist[tid], unused);  // digit tid's first output position
     const uint32_t lt_mask = (1u << lane) - 1u;
     uint32_t *wc = wcnt[warp];
-    for (int cbase = beg; cbase < end; cbase += CH) {
+    for (int part; (part = next_part(counter)) < parts;) {
+        const int cbase = part * CH, cn = min(CH, n - cbase);
 #pragma unroll
-        for (int q = 0; q < ND / 32; ++q) wc[32 * q + lane] = 0;
-        const int wbase = cbase + 32 * IPT * warp;
+        for (int q = 0; q < 8; ++q) wc[32 * q + lane] = 0;
+        const int wbase = 32 * IPT * warp;
         uint32_t key[IPT], val[IPT], rank[IPT];
-        // all of the warp's loads first (their latencies overlap), then the ranking
+        // all of the warp's loads first (their latencies overlap), then the ranking; each pair is
+        // read once: evict-first loads, which leave L2 to the partly written output lines
 #pragma unroll
         for (int it = 0; it < IPT; ++it) {
             const int i = wbase + 32 * it + lane;
-            const bool valid = i < end;
-            key[it] = valid ? src.key(i) : 0u;
-            val[it] = valid ? src.val(i) : 0u;
+            key[it] = i < cn ? __ldcs(kin + cbase + i) : 0u;
+            val[it] = i < cn ? __ldcs(vin + cbase + i) : 0u;
         }
         __syncwarp();
 #pragma unroll
         for (int it = 0; it < IPT; ++it) {
-            const bool valid = wbase + 32 * it + lane < end;
-            const uint32_t d = valid ? ((key[it] >> shift) & mask) : (uint32_t)ND;
+            const bool valid = wbase + 32 * it + lane < cn;
+            const uint32_t d = valid ? ((key[it] >> shift) & mask) : 256u;
             const uint32_t peers = __match_any_sync(SG_FULL_MASK, d);
             const uint32_t below = __popc(peers & lt_mask);
             rank[it] = valid ? wc[d] + below : 0u;
@@ -674,106 +747,206 @@ __global__ void __launch_bounds__(kScanThreads, 4) rs_scatter_kernel(
             __syncwarp();
         }
         __syncthreads();
-        // per digit: exclusive offsets of the warps, the chunk's count, and (block scan)
-        // the digit's first slot in the reordered chunk
-        uint32_t cnt[DPT], ex[DPT];
+        // digit tid: exclusive offsets of the warps, the part's count
+        uint32_t cnt = 0;
 #pragma unroll
-        for (int q = 0; q < DPT; ++q) {
-            const int d = tid * DPT + q;
-            uint32_t s = 0;
-#pragma unroll
-            for (int w = 0; w < kWarps; ++w) {
-                const uint32_t c = wcnt[w][d];
-                wcnt[w][d] = s;
-                s += c;
-            }
-            cnt[q] = s;
+        for (int w = 0; w < kWarps; ++w) {
+            const uint32_t c = wcnt[w][tid];
+            wcnt[w][tid] = cnt;
+            cnt += c;
         }
-        bucket_exclusive_scan<DPT>(cnt, ex);
-#pragma unroll
-        for (int q = 0; q < DPT; ++q) loc[tid * DPT + q] = ex[q];
+        uint64_t *word = words + (size_t)part * 256 + tid;
+        const bool digit = tid <= (int)mask;  // (the other threads' counts are 0)
+        if (digit) store_word(word, (part == 0 ? kPrefix : kAggregate) | cnt);
+        const uint32_t slot0 = block_exclusive_scan(cnt, unused);
+        loc[tid] = slot0;
         __syncthreads();
 #pragma unroll
         for (int it = 0; it < IPT; ++it) {
-            if (wbase + 32 * it + lane < end) {
+            if (wbase + 32 * it + lane < cn) {
                 const uint32_t d = (key[it] >> shift) & mask;
                 const uint32_t li = loc[d] + wc[d] + rank[it];
                 skey[li] = key[it];
                 sval[li] = val[it];
             }
         }
+        uint32_t before = 0;
+        if (part > 0 && digit) {
+            before = look_back(words + tid, 256, part, status);
+            store_word(word, kPrefix | (uint64_t)(before + cnt));
+        }
+        to[tid] = first + before - slot0;
+        if (clear) clear[(size_t)part * 256 + tid] = 0;
         __syncthreads();
-        const int cn = min(CH, end - cbase);
         for (int j = tid; j < cn; j += kScanThreads) {
             const uint32_t k = skey[j];
-            const uint32_t d = (k >> shift) & mask;
-            const uint32_t pos = run[d] + ((uint32_t)j - loc[d]);
-            if (kout) kout[pos] = k;
+            const uint32_t pos = to[(k >> shift) & mask] + (uint32_t)j;
+            if (pos >= (uint32_t)n) continue;  // (only after a timeout)
+            kout[pos] = k;
             vout[pos] = sval[j];
         }
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < DPT; ++q) run[tid * DPT + q] += cnt[q];
-        // (the next chunk's first block barrier orders these updates before their reads)
+        // (next_part's barriers order these reads before the next part's writes)
     }
 }
 
-// Sorts n (device count, clamped to cap) pairs on bits [0, bits) from (kin, vin) into
-// (kout, vout) using (ktmp, vtmp) as ping-pong; kin/vin are not modified.  The bits are
-// split into the fewest passes of at most max_bits (<= 9) bits, as evenly as possible.
-static void radix_sort(const uint32_t *kin, const uint32_t *vin, uint32_t *kout, uint32_t *vout,
-                       uint32_t *ktmp, uint32_t *vtmp, const int *n_ptr, int cap, int bits,
-                       uint32_t *hist, uint32_t *totals, int G, cudaStream_t st, int max_bits) {
-    const int passes = (bits + max_bits - 1) / max_bits;
-    const uint32_t *ks = kin, *vs = vin;
+// Splits `bits` into the fewest passes of at most max_bits bits, as evenly as possible.
+static Digits split_digits(int bits, int max_bits) {
+    Digits d{};
+    d.n = (bits + max_bits - 1) / max_bits;
     int shift = 0;
-    for (int p = 0; p < passes; ++p) {
-        const int nb = (bits - shift + (passes - p) - 1) / (passes - p);
-        const uint32_t mask = (1u << nb) - 1u;
-        uint32_t *kd = ((passes - 1 - p) % 2 == 0) ? kout : ktmp;
-        uint32_t *vd = ((passes - 1 - p) % 2 == 0) ? vout : vtmp;
-        const ArrayPairs src{ks, vs};
-        if (nb > 8) {
-            launch_pdl(rs_hist_kernel<ArrayPairs, 512>, G, kScanThreads, 0, st, src, n_ptr, cap, shift, mask, hist, G);
-            launch_pdl(rs_digit_scan_kernel, 512, kScanThreads, 0, st, hist, totals, G);
-            launch_pdl(rs_scatter_kernel<ArrayPairs, 512>, G, kScanThreads, 0, st, src, kd, vd, n_ptr, cap, shift, mask,
-                       hist, totals, G);
-        } else {
-            launch_pdl(rs_hist_kernel<ArrayPairs, 256>, G, kScanThreads, 0, st, src, n_ptr, cap, shift, mask, hist, G);
-            launch_pdl(rs_digit_scan_kernel, 256, kScanThreads, 0, st, hist, totals, G);
-            launch_pdl(rs_scatter_kernel<ArrayPairs, 256>, G, kScanThreads, 0, st, src, kd, vd, n_ptr, cap, shift, mask,
-                       hist, totals, G);
-        }
-        count_launches(3);
-        ks = kd;
-        vs = vd;
+    for (int p = 0; p < d.n; ++p) {
+        const int nb = (bits - shift + (d.n - p) - 1) / (d.n - p);
+        d.shift[p] = shift;
+        d.mask[p] = (1u << nb) - 1u;
         shift += nb;
     }
+    return d;
 }
 
-__global__ void clamp_count_kernel(const int *in, int cap, int *out) {
-    pdl_begin();
-    *out = min(*in, cap);
+// Sorts n (device count, clamped to cap) pairs by the digits dg from (kin, vin) into
+// (kout, vout) using (ktmp, vtmp) as ping-pong; kin/vin are not modified.  hist: the digits'
+// histograms (256 words each); words[0]: the first pass's chained-scan words, cleared for every
+// part; words[1]: the second pass's (the passes alternate between the two and each clears its
+// successor's); counters: one per pass, zero.
+static void radix_sort(const uint32_t *kin, const uint32_t *vin, uint32_t *kout, uint32_t *vout, uint32_t *ktmp,
+                       uint32_t *vtmp, const int *n_ptr, int cap, const Digits &dg, const uint32_t *hist,
+                       uint64_t *const words[2], int *counters, int grid, uint32_t *status, cudaStream_t st) {
+    const uint32_t *ks = kin, *vs = vin;
+    for (int p = 0; p < dg.n; ++p) {
+        uint32_t *kd = ((dg.n - 1 - p) % 2 == 0) ? kout : ktmp;
+        uint32_t *vd = ((dg.n - 1 - p) % 2 == 0) ? vout : vtmp;
+        launch_pdl(sweep_kernel, grid, kScanThreads, 0, st, ks, vs, kd, vd, n_ptr, cap, dg.shift[p], dg.mask[p],
+                   hist + 256 * p, words[p & 1], p + 1 < dg.n ? words[(p + 1) & 1] : (uint64_t *)nullptr, counters + p,
+                   status);
+        count_launches(1);
+        ks = kd;
+        vs = vd;
+    }
 }
 
-// [start, end) of every tile by binary search in the sorted tile ids ((0, 0) for a tile with
-// no instance): one thread per tile, no prior zeroing.
-__device__ __forceinline__ int lower_bound_u32(const uint32_t *__restrict__ a, int n, uint32_t key) {
-    int lo = 0, hi = n;
+// ---------------------------------------------------------------------------------------
+// Ranges and work order
+// ---------------------------------------------------------------------------------------
+
+__device__ __forceinline__ int lower_bound_u32(const uint32_t *__restrict__ a, int lo, int hi, uint32_t key) {
     while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
+        const int mid = lo + ((hi - lo) >> 1);
         if (a[mid] < key) lo = mid + 1; else hi = mid;
     }
     return lo;
 }
-__global__ void ranges_kernel(const uint32_t *__restrict__ tile, const int *__restrict__ k_ptr, int n_tiles,
-                              int2 *__restrict__ ranges) {
+
+// The same for a whole warp and one key, 32 probes at a time.
+__device__ __forceinline__ int warp_lower_bound_u32(const uint32_t *__restrict__ a, int n, uint32_t key) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0, hi = n;  // the answer is in [lo, hi]
+    while (hi > lo) {
+        const int64_t len = hi - lo;
+        const int probe = lo + (int)(len * lane / 32);  // ascending; probe of lane 0 is lo
+        const uint32_t less = __ballot_sync(SG_FULL_MASK, a[probe] < key);
+        const int m = __popc(less);  // probes below the key: a prefix of the lanes
+        if (m == 0) return lo;
+        const int nlo = lo + (int)(len * (m - 1) / 32) + 1;
+        hi = m == 32 ? hi : lo + (int)(len * m / 32);
+        lo = nlo;
+    }
+    return lo;
+}
+
+// Work-order bucket of a tile with n instances: 63 - b, b = 0 for n = 0, else
+// 1 + 2 floor(log2 n) + the bit below the leading one (descending length, 6 bits).
+__device__ __forceinline__ uint32_t length_bucket(int2 r) {
+    const uint32_t n = (uint32_t)max(r.y - r.x, 0);
+    if (n == 0) return 63u;
+    const int lz = 31 - __clz(n);
+    const uint32_t sub = lz >= 1 ? (n >> (lz - 1)) & 1u : 0u;
+    return 63u - (1u + 2u * (uint32_t)lz + sub);
+}
+
+// [start, end) of every tile by search in the sorted tile ids ((0, 0) for a tile with no
+// instance): one warp per 32 tiles finds its first and its last bound together, then each lane
+// its own bound in between.  hist (or null): counts of the length buckets.
+__global__ void __launch_bounds__(kScanThreads) ranges_kernel(const uint32_t *__restrict__ tile,
+                                                              const int *__restrict__ k_ptr, int cap, int n_tiles,
+                                                              int2 *__restrict__ ranges, uint32_t *__restrict__ hist) {
     pdl_begin();
-    const int K = *k_ptr;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n_tiles; t += gridDim.x * blockDim.x) {
-        const int lo = lower_bound_u32(tile, K, (uint32_t)t);
-        const int hi = lower_bound_u32(tile, K, (uint32_t)t + 1u);
-        ranges[t] = lo < hi ? make_int2(lo, hi) : make_int2(0, 0);
+    __shared__ uint32_t s_h[64];
+    if (threadIdx.x < 64) s_h[threadIdx.x] = 0;
+    __syncthreads();
+    const int K = min(*k_ptr, cap), lane = threadIdx.x & 31;
+    const int t = blockIdx.x * kScanThreads + (int)threadIdx.x, t0 = t - lane;
+    if (t0 < n_tiles) {  // (warp-uniform)
+        const int wlo = warp_lower_bound_u32(tile, K, (uint32_t)t0);
+        const int whi = warp_lower_bound_u32(tile, K, (uint32_t)t0 + 32u);
+        const int lo = lower_bound_u32(tile, wlo, whi, (uint32_t)t);
+        int hi = __shfl_down_sync(SG_FULL_MASK, lo, 1);
+        if (lane == 31) hi = whi;
+        if (t < n_tiles) {
+            const int2 r = lo < hi ? make_int2(lo, hi) : make_int2(0, 0);
+            ranges[t] = r;
+            if (hist) atomicAdd(&s_h[length_bucket(r)], 1u);
+        }
+    }
+    if (hist) flush_hist(s_h, 64, hist);
+}
+
+// The work order: a stable counting sort of the tiles by length bucket.  A block's part is a
+// contiguous range of tiles (grid parts, 256 tiles at a time), counted, placed by the chained
+// scan (64 words per part) and written.
+__global__ void __launch_bounds__(kScanThreads) order_kernel(const int2 *__restrict__ ranges, int n_tiles,
+                                                             const uint32_t *__restrict__ hist,
+                                                             uint64_t *__restrict__ words, int *__restrict__ counter,
+                                                             int *__restrict__ order, uint32_t *__restrict__ status) {
+    pdl_begin();
+    constexpr int kWarps = kScanThreads / 32;
+    __shared__ uint32_t s_cnt[64], s_run[64], s_w[kWarps][64];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rows = (n_tiles + kScanThreads - 1) / kScanThreads;
+    const int per = (rows + (int)gridDim.x - 1) / (int)gridDim.x * kScanThreads;  // tiles of a part
+    const int part = next_part(counter);
+    const int64_t beg = (int64_t)part * per, end = min((int64_t)n_tiles, beg + per);
+    uint32_t unused;
+    const uint32_t first = block_exclusive_scan(tid < 64 ? hist[tid] : 0u, unused);
+    if (tid < 64) s_cnt[tid] = 0;
+    __syncthreads();
+    for (int64_t i = beg + tid; i < end; i += kScanThreads) atomicAdd(&s_cnt[length_bucket(ranges[i])], 1u);
+    __syncthreads();
+    if (tid < 64) {
+        uint64_t *word = words + (size_t)part * 64 + tid;
+        store_word(word, (part == 0 ? kPrefix : kAggregate) | s_cnt[tid]);
+        uint32_t before = 0;
+        if (part > 0) {
+            before = look_back(words + tid, 64, part, status);
+            store_word(word, kPrefix | (uint64_t)(before + s_cnt[tid]));
+        }
+        s_run[tid] = first + before;
+    }
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    for (int64_t base = beg; base < end; base += kScanThreads) {
+        s_w[warp][lane] = s_w[warp][lane + 32] = 0;
+        __syncwarp();
+        const int64_t i = base + tid;
+        const uint32_t d = i < end ? length_bucket(ranges[i]) : 64u;
+        const uint32_t peers = __match_any_sync(SG_FULL_MASK, d);
+        const uint32_t below = __popc(peers & lt_mask);
+        if (d < 64u && below == 0) s_w[warp][d] = __popc(peers);
+        __syncthreads();
+        if (tid < 64) {  // the warps' first positions in this row of 256 tiles
+            uint32_t run = s_run[tid];
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) {
+                const uint32_t c = s_w[w][tid];
+                s_w[w][tid] = run;
+                run += c;
+            }
+            s_run[tid] = run;
+        }
+        __syncthreads();
+        if (d < 64u) {
+            const uint32_t pos = s_w[warp][d] + below;
+            if (pos < (uint32_t)n_tiles) order[pos] = (int)i;  // (beyond only after a timeout)
+        }
+        __syncthreads();
     }
 }
 
@@ -781,14 +954,22 @@ __global__ void ranges_kernel(const uint32_t *__restrict__ tile, const int *__re
 // Workspace layout
 // ---------------------------------------------------------------------------------------
 
+// Chained-scan part counters (one per kernel of a list build).
+enum { kCtrCompact = 0, kCtrDepth = 1, kCtrSlots = 5, kCtrCull = 6, kCtrTile = 7, kCtrOrder = 11, kCtrs = 12 };
+
 struct TileWorkspace {
     uint32_t *dkey_in, *dval_in, *dkey_out, *dval_out, *dkey_tmp, *dval_tmp;
     uint32_t *slot0;      // first (record, tile row) slot of each depth-sorted record
-    uint32_t *first_rec;  // record owning the first slot of each block of the slot partition
-    uint32_t *kbsum;      // kept instances per block of the slot partition, then their offsets
+    uint32_t *first_rec;  // record owning the first slot of each 256-slot chunk
     uint32_t *tkey_in, *tval_in, *tkey_tmp, *tval_tmp;
-    uint32_t *bsum, *hist, *totals;
-    int *counts;  // [0] visible records M, [1] K clamped
+    // cleared by a memset at the start of every list build, [zero, zero + zero_bytes):
+    char *zero;
+    size_t zero_bytes;
+    int *counts;    // [0] visible records M, [1] slots S
+    int *counters;  // kCtrs part counters
+    uint32_t *dhist, *thist, *ohist;                      // 4 x 256, 4 x 256, 64
+    uint64_t *cwords, *swords, *kwords, *owords;  // chained-scan words: compaction, slots, culling, order
+    uint64_t *sweep[2];  // radix passes: [0] is cleared for the depth sort's parts
 };
 
 static int sort_grid() {
@@ -804,6 +985,8 @@ static int sort_grid() {
 }
 
 static size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
+
+static int64_t sweep_parts(int64_t n) { return (n + kSweepPart - 1) / kSweepPart; }
 
 static size_t tile_ws_layout(int64_t R, int32_t cap, int G, TileWorkspace *ws, char *base) {
     size_t off = 0;
@@ -821,17 +1004,27 @@ static size_t tile_ws_layout(int64_t R, int32_t cap, int G, TileWorkspace *ws, c
     w.dkey_tmp = (uint32_t *)take(r4);
     w.dval_tmp = (uint32_t *)take(r4);
     w.slot0 = (uint32_t *)take(r4);
-    w.first_rec = (uint32_t *)take((size_t)4 * G * 4);  // the slot partition has 4 G blocks
-    w.kbsum = (uint32_t *)take((size_t)4 * G * 4);
-
+    w.first_rec = (uint32_t *)take((size_t)kMaxChunks * 4);
     w.tkey_in = (uint32_t *)take(c4);
     w.tval_in = (uint32_t *)take(c4);
     w.tkey_tmp = (uint32_t *)take(c4);
     w.tval_tmp = (uint32_t *)take(c4);
-    w.bsum = (uint32_t *)take((size_t)4 * G * 4);  // up to 4 G blocks (the emission grid)
-    w.hist = (uint32_t *)take((size_t)G * 512 * 4);
-    w.totals = (uint32_t *)take(512 * 4);
+    const size_t z0 = off;
+    const size_t rparts = (size_t)((R + kCompactPart - 1) / kCompactPart);
+    w.zero = take(0);
     w.counts = (int *)take(4 * sizeof(int));
+    w.counters = (int *)take(kCtrs * sizeof(int));
+    w.dhist = (uint32_t *)take(4 * 256 * 4);
+    w.thist = (uint32_t *)take(4 * 256 * 4);
+    w.ohist = (uint32_t *)take(64 * 4);
+    w.cwords = (uint64_t *)take(rparts * 8);
+    w.swords = (uint64_t *)take(rparts * 8);
+    w.kwords = (uint64_t *)take((size_t)kMaxChunks * 8);
+    w.owords = (uint64_t *)take((size_t)G * 64 * 8);
+    const size_t sweep_bytes = (size_t)std::max(sweep_parts(R), sweep_parts(cap)) * 256 * 8;
+    w.zero_bytes = off - z0 + (size_t)sweep_parts(R) * 256 * 8;
+    w.sweep[0] = (uint64_t *)take(sweep_bytes);
+    w.sweep[1] = (uint64_t *)take(sweep_bytes);
     if (ws) *ws = w;
     return off;
 }
@@ -854,58 +1047,42 @@ sg_status launch_build_tile_lists(const sg_projected *proj, int N, int n_views,
     }
     const uint2 *rect = reinterpret_cast<const uint2 *>(proj->rect);
     const float4 *geo = reinterpret_cast<const float4 *>(proj->geo);
-    // 1. compaction of visible records (count -> counts[0])
-    launch_pdl(scan_reduce_kernel<VisibleCount>, G, kScanThreads, 0, st, VisibleCount{rect}, nullptr, (int)R, w.bsum, G);
-    launch_pdl(scan_blocks_kernel, 1, kScanThreads, 0, st, w.bsum, G, w.counts + 0);
-    launch_pdl(compact_apply_kernel, G, kScanThreads, 0, st, rect, geo, (int)R, w.bsum, G, w.dkey_in, w.dval_in);
-    // 2. depth sort (32 bits).  Its input (the visible records) is a small fraction of R, so it
-    // runs on a grid of about 2048 elements per block for R / 4, between G / 4 and G.
-    const int Gd = (int)std::min<int64_t>(G, std::max<int64_t>(G / 4, R / (4 * 2048)));
-    radix_sort(w.dkey_in, w.dval_in, w.dkey_out, w.dval_out, w.dkey_tmp, w.dval_tmp, w.counts + 0,
-               (int)R, 32, w.hist, w.totals, Gd, st, 8);
-    // 3. emission in depth order (K -> lists->count)
-    // The emission runs on a finer grid for large inputs (up to 4 G blocks, about one per 2048
-    // records): its blocks own ranges of depth-sorted records, and the near (large) ones,
-    // which emit most of the instances, come first.
-    const int Ge = (int)std::min<int64_t>(4 * G, std::max<int64_t>(G, R / 2048));
-    // slots: the rectangle tile rows of the records in depth order
     const float2 *ext = reinterpret_cast<const float2 *>(proj->ext);
-    launch_pdl(scan_reduce_kernel<SortedRowCount>, Ge, kScanThreads, 0, st, SortedRowCount{rect, w.dval_out},
-               w.counts + 0, 0, w.bsum, Ge);
-    launch_pdl(scan_blocks_kernel, 1, kScanThreads, 0, st, w.bsum, Ge, w.counts + 2);
-    const int Gc = 4 * G;  // blocks of the slot partition (each walks a few 256-slot chunks)
-    const bool halves = lists->half_masks != 0;  // records carry half masks
-    launch_pdl(slot_prefix_kernel, Ge, kScanThreads, 0, st, rect, w.dval_out, w.counts + 0, w.bsum, Ge,
-               w.counts + 2, Gc, w.slot0, w.first_rec);
-    // culling, evenly over the slots: kept counts, their offsets, emission (the tile sort's
-    // ping-pong buffers and the output tile ids, all free until the sort, hold the slot cache)
-    const auto count_pass = halves ? cull_pass_kernel<false, true> : cull_pass_kernel<false, false>;
-    const auto emit_pass = halves ? cull_pass_kernel<true, true> : cull_pass_kernel<true, false>;
-    launch_pdl(count_pass, Gc, kScanThreads, 0, st, rect, geo, ext, w.dval_out, w.counts + 0, w.counts + 2, w.slot0,
-               w.first_rec, Gc, N, views, n_views, tile_w, tile_h, w.kbsum, (uint32_t *)nullptr,
-               (uint32_t *)nullptr, w.tkey_tmp, w.tval_tmp, lists->tile, lists->capacity, status);
-    launch_pdl(scan_blocks_kernel, 1, kScanThreads, 0, st, w.kbsum, Gc, lists->count);
-    launch_pdl(emit_pass, Gc, kScanThreads, 0, st, rect, geo, ext, w.dval_out, w.counts + 0, w.counts + 2, w.slot0,
-               w.first_rec, Gc, N, views, n_views, tile_w, tile_h, w.kbsum, w.tkey_in, w.tval_in, w.tkey_tmp,
-               w.tval_tmp, lists->tile, lists->capacity, status);
-    // 4. stable sort by tile id
+    auto grid = [G](int64_t parts) { return (int)std::max<int64_t>(1, std::min<int64_t>(G, parts)); };
+    cudaMemsetAsync(w.zero, 0, w.zero_bytes, st);
+    // 1. compaction of the visible records (count -> counts[0])
+    const int cgrid = grid((R + kCompactPart - 1) / kCompactPart);
+    launch_pdl(compact_kernel, cgrid, kScanThreads, 0, st, rect, geo, (int)R, w.cwords, w.counters + kCtrCompact,
+               w.dkey_in, w.dval_in, w.counts, w.dhist, lists->count, status);
+    // 2. depth sort (32 bits)
+    radix_sort(w.dkey_in, w.dval_in, w.dkey_out, w.dval_out, w.dkey_tmp, w.dval_tmp, w.counts, (int)R,
+               split_digits(32, 8), w.dhist, w.sweep, w.counters + kCtrDepth, grid(sweep_parts(R)), status, st);
+    // 3. slots: the rectangle tile rows of the records in depth order (their number ->
+    // counts[1]); culling and emission (K -> lists->count)
+    launch_pdl(slot_prefix_kernel, cgrid, kScanThreads, 0, st, rect, w.dval_out, w.counts, w.swords,
+               w.counters + kCtrSlots, w.slot0, w.first_rec, w.counts + 1, status);
     int bits = 1;
     while ((1ll << bits) < (long long)n_tiles) ++bits;
-    radix_sort(w.tkey_in, w.tval_in, lists->tile, lists->record, w.tkey_tmp, w.tval_tmp,
-               lists->count, lists->capacity, bits, w.hist, w.totals, G, st, kTileDigitBits);
-    // 5. tile ranges
-    launch_pdl(clamp_count_kernel, 1, 1, 0, st, lists->count, lists->capacity, w.counts + 1);
-    launch_pdl(ranges_kernel, (n_tiles + kScanThreads - 1) / kScanThreads, kScanThreads, 0, st, lists->tile,
-               w.counts + 1, n_tiles, reinterpret_cast<int2 *>(lists->ranges));
-    count_launches(3 + 6 + 2);  // compaction, slots + culling + emission, clamp + ranges
-    // 6. work order: one stable counting pass over the 6-bit length keys
+    const Digits dg = split_digits(bits, kTileDigitBits);
+    const bool halves = lists->half_masks != 0;  // records carry half masks
+    launch_pdl(halves ? cull_kernel<true> : cull_kernel<false>, G + G / 2, kScanThreads, 0, st, rect, geo, ext, w.dval_out,
+               w.counts, w.counts + 1, w.slot0, w.first_rec, w.kwords, w.counters + kCtrCull, N, views, n_views, tile_w,
+               tile_h, w.tkey_in, w.tval_in, lists->capacity, lists->count, dg, w.thist, w.sweep[0], kSweepPart, w.tkey_tmp, w.tval_tmp,
+               lists->tile, status);
+    // 4. stable sort by tile id
+    radix_sort(w.tkey_in, w.tval_in, lists->tile, lists->record, w.tkey_tmp, w.tval_tmp, lists->count,
+               lists->capacity, dg, w.thist, w.sweep, w.counters + kCtrTile, grid(sweep_parts(lists->capacity)), status,
+               st);
+    // 5. tile ranges; 6. work order
+    int2 *ranges = reinterpret_cast<int2 *>(lists->ranges);
+    const int tblocks = (int)(((int64_t)n_tiles + kScanThreads - 1) / kScanThreads);
+    launch_pdl(ranges_kernel, tblocks, kScanThreads, 0, st, lists->tile, lists->count, lists->capacity, n_tiles, ranges,
+               lists->order ? w.ohist : (uint32_t *)nullptr);
+    count_launches(4);  // compaction, slots, culling, ranges
     if (lists->order) {
-        const TileLengthKeys src{reinterpret_cast<const int2 *>(lists->ranges)};
-        launch_pdl(rs_hist_kernel<TileLengthKeys, 256>, G, kScanThreads, 0, st, src, nullptr, n_tiles, 0, 63u, w.hist, G);
-        launch_pdl(rs_digit_scan_kernel, 256, kScanThreads, 0, st, w.hist, w.totals, G);
-        launch_pdl(rs_scatter_kernel<TileLengthKeys, 256>, G, kScanThreads, 0, st, src, nullptr, reinterpret_cast<uint32_t *>(lists->order),
-                                                      nullptr, n_tiles, 0, 63u, w.hist, w.totals, G);
-        count_launches(3);
+        launch_pdl(order_kernel, std::min(G, tblocks), kScanThreads, 0, st, ranges, n_tiles, w.ohist,
+                   w.owords, w.counters + kCtrOrder, lists->order, status);
+        count_launches(1);
     }
     return check_launch("build_tile_lists");
 }
