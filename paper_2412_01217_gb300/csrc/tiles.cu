@@ -139,22 +139,43 @@ __device__ __forceinline__ uint32_t block_look_back(uint64_t *words, int part, u
     return sum;
 }
 
-// The same for one thread whose sum has been published in words[part * stride] (a digit of a
-// radix pass): four predecessors' words are requested at a time.
-__device__ __forceinline__ uint32_t look_back(const uint64_t *words, int stride, int part, uint32_t *status) {
+// The same for the threads of a warp, each with its own words (digits of a radix pass): a
+// thread's sum has been published in words[part * stride]; four predecessors' words are
+// requested at a time.  Called by whole warps, and the warp stays together: the waits and the
+// loop end for all lanes at once (inactive lanes sum nothing), so that no lane runs ahead to the
+// caller's block barrier while others still look back.
+__device__ __forceinline__ uint32_t look_back(const uint64_t *words, int stride, int part, bool active,
+                                              uint32_t *status) {
     uint32_t sum = 0;
-    for (int p = part - 1; p >= 0; p -= 4) {
-        uint64_t w[4];
+    bool done = !active;
+    for (int p = part - 1; p >= 0 && !__all_sync(SG_FULL_MASK, done); p -= 4) {
+        uint64_t w[4];  // (before the first part: an empty prefix)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) w[i] = p - i >= 0 ? load_word(words + (size_t)(p - i) * stride) : kPrefix;
+        for (int i = 0; i < 4; ++i) w[i] = !done && p - i >= 0 ? load_word(words + (size_t)(p - i) * stride) : kPrefix;
+        for (uint32_t polls = 0;; ++polls) {
+            bool missing = false;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (p - i < 0) return sum;
-            const uint64_t v = wait_word(words + (size_t)(p - i) * stride, w[i], status);
-            sum += (uint32_t)v;
-            if (v & kPrefix) return sum;
+            for (int i = 0; i < 4; ++i) missing |= !(w[i] >> 32);
+            if (!__any_sync(SG_FULL_MASK, missing)) break;
+            if (polls >= kSpinLimit) {  // (warp-uniform)
+                if (missing) atomicOr(status, SG_STATUS_TIMEOUT);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (!(w[i] >> 32)) w[i] = kPrefix;
+                break;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (!(w[i] >> 32)) w[i] = load_word(words + (size_t)(p - i) * stride);
         }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (!done) {
+                sum += (uint32_t)w[i];
+                done = (w[i] & kPrefix) != 0;
+            }
     }
+    __syncwarp();
     return sum;
 }
 
@@ -771,9 +792,10 @@ __global__ void __launch_bounds__(kScanThreads, 4) sweep_kernel(
             }
         }
         uint32_t before = 0;
-        if (part > 0 && digit) {
-            before = look_back(words + tid, 256, part, status);
-            store_word(word, kPrefix | (uint64_t)(before + cnt));
+        if (part > 0 && (tid & ~31) <= (int)mask) {  // (warp-uniform)
+            before = look_back(words + tid, 256, part, digit, status);
+            if (digit) store_word(word, kPrefix | (uint64_t)(before + cnt));
+            __syncwarp();
         }
         to[tid] = first + before - slot0;
         if (clear) clear[(size_t)part * 256 + tid] = 0;
@@ -916,7 +938,7 @@ __global__ void __launch_bounds__(kScanThreads) order_kernel(const int2 *__restr
         store_word(word, (part == 0 ? kPrefix : kAggregate) | s_cnt[tid]);
         uint32_t before = 0;
         if (part > 0) {
-            before = look_back(words + tid, 64, part, status);
+            before = look_back(words + tid, 64, part, true, status);
             store_word(word, kPrefix | (uint64_t)(before + s_cnt[tid]));
         }
         s_run[tid] = first + before;

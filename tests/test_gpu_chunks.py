@@ -1,0 +1,89 @@
+"""Edges of the list build's radix passes and of the compositing kernels' 16-entry chunks.
+
+* Lists of every digit width of the tile sort's last pass (one tile to 825 tiles), with enough
+  instances for many parts of the chained scan, built repeatedly: always the same lists, in
+  (tile, depth bits, record) order, with the ranges and the work order they imply.
+* One small image behind stacks of 1 to 65 Gaussians (chunks of 16 with every kind of
+  remainder): every pixel and all gradients against the oracle, with the parity tolerances.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synthetic
+from helpers import AMBIGUOUS_GRAD, FWD_ABS, FWD_REL, check_close, check_grads, ref_render
+from test_gpu_parity import KEYS, _check_ranges_and_order, _gpu_lists, f32_camera, make, view_images
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("W, H, levels, tile, half", [
+    (16, 16, 1, (16, 16), False),    # 1 tile: one 1-bit pass
+    (64, 48, 1, (16, 16), False),    # 12 tiles: 4 bits
+    (160, 120, 1, (16, 16), False),  # 80 tiles: 7 bits
+    (320, 180, 3, (16, 16), False),  # 315 tiles: passes of 5 and 4 bits
+    (256, 128, 1, (8, 8), True),     # 512 tiles: 5 and 4 bits, half masks
+    (520, 400, 1, (16, 16), False),  # 825 tiles: 5 and 5 bits
+])
+def test_lists_are_sorted_and_repeatable_for_every_digit_width(W, H, levels, tile, half):
+    N = 20_000
+    g = synthetic.cloud_scene(N, 4, seed=W + H)
+    cam = f32_camera(synthetic.make_camera(W, H, 0.9 * W, 0.9 * W, W / 2 - 0.5, H / 2 - 0.5))
+    r, p = make(g, [cam], levels=levels, tile_w=tile[0], tile_h=tile[1], half_masks=half)
+    r.project(p)
+    first = None
+    for _ in range(25):
+        r.build_lists()
+        K, tiles, recs, ranges = _gpu_lists(r)
+        if first is None:
+            first = (tiles, recs)
+            _check_ranges_and_order(r, tiles, ranges)
+            depth = r.geo.view(-1, 8)[:, 2].contiguous().view(torch.int32).cpu().numpy()[recs]
+            assert np.array_equal(np.lexsort((recs, depth, tiles)), np.arange(K))
+            assert K >= 10_000 and len(np.unique(np.stack([tiles, recs]), axis=1)[0]) == K
+            local = recs // N  # the tile's view is the record's
+            off = np.array([v.tile_offset for v in r.views_host])
+            assert np.array_equal(np.searchsorted(off, tiles, "right") - 1, local)
+        assert np.array_equal(tiles, first[0]) and np.array_equal(recs, first[1])
+
+
+def _stack(n, C, seed):
+    """n Gaussians in front of a 16 x 8 camera, each reaching much of the image, faint enough
+    that all of them contribute."""
+    rng = np.random.default_rng(seed)
+    z = rng.uniform(1.0, 3.0, n)
+    mean = np.stack([rng.uniform(-0.35, 0.35, n) * z, rng.uniform(-0.15, 0.15, n) * z, z], 1)
+    q = rng.normal(size=(n, 4))
+    f = lambda a: np.ascontiguousarray(a, dtype=np.float32)
+    return dict(mean=f(mean), log_scale=f(rng.uniform(np.log(0.1), np.log(0.5), (n, 3))),
+                quat=f(q / np.linalg.norm(q, axis=1, keepdims=True)), opacity_logit=f(rng.normal(-2.5, 0.5, n)),
+                rgb=f(rng.uniform(0, 1, (n, 3))), sem=f(rng.normal(size=(n, C))))
+
+
+@pytest.mark.parametrize("C, cfg", [
+    (4, dict(tile_w=16, tile_h=8, pixels_per_thread=1, pixels_per_thread_bwd=1)),
+    (8, dict(tile_w=8, tile_h=8, pixels_per_thread=2, pixels_per_thread_bwd=2, batch=16)),
+    (16, dict(tile_w=16, tile_h=16, pixels_per_thread=4, pixels_per_thread_bwd=4, batch=32)),
+    (32, dict(tile_w=8, tile_h=8, pixels_per_thread=1, pixels_per_thread_bwd=1, half_masks=True)),
+    (40, dict(tile_w=8, tile_h=8, pixels_per_thread=1, pixels_per_thread_bwd=1, half_masks=True, half_tile_fwd=True)),
+])
+@pytest.mark.parametrize("n", [1, 4, 15, 16, 17, 31, 33, 48, 65])
+def test_stacks_around_the_chunk_size_match_oracle(n, C, cfg):
+    W, H = 15, 7  # ragged in every tile shape
+    g = _stack(n, C, seed=100 * n + C)
+    cam = f32_camera(synthetic.make_camera(W, H, 16.0, 16.0, 7.0, 3.0))
+    r, p = make(g, [cam], **cfg)
+    r.forward(p)
+    got = view_images(r, 0, C)
+    ref = ref_render(g, cam)
+    ok = (ref["flags"] & AMBIGUOUS_GRAD) == 0
+    assert ok.mean() > 0.9
+    for k in ("rgb", "depth", "sem", "T"):
+        check_close(k, got[k], ref[k], FWD_REL, FWD_ABS, mask=ok)
+    rng = np.random.default_rng(n)
+    up = [(rng.normal(size=s) * ok).astype(np.float32) for s in ((3, H, W), (H, W), (C, H, W))]
+    grads = {k: torch.zeros_like(v) for k, v in p.items()}
+    r.backward(p, grads, dL=tuple(torch.tensor(u.reshape(-1), device="cuda") for u in up))
+    want = oracle.render_backward(g, cam, *[u.astype(np.float64) for u in up])
+    check_grads({k: v.cpu().numpy() for k, v in grads.items()}, want, KEYS)
