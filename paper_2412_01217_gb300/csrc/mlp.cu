@@ -73,7 +73,7 @@ static sg_status launch_gemm_kernel(const tc::GemmParams &p, int splits, const C
         attr = true;
     }
     const dim3 grid((p.M + 127) / 128, (p.N + BN - 1) / BN, splits);
-    tc::gemm_kernel<BN, STAGES, TMA><<<grid, 128, smem, st>>>(p, ma, mb);
+    launch_pdl(tc::gemm_kernel<BN, STAGES, TMA>, grid, dim3(128), smem, st, p, ma, mb);
     count_launches(1);
     return check_launch("tcgen05 gemm");
 }
@@ -118,12 +118,16 @@ sg_status launch_gemm(tc::GemmParams p, cudaStream_t st, int max_splits = 64) {
         set_error("gemm: bias with split-K is not supported");
         return SG_ERR_INVALID_ARG;
     }
+    p.vec_mask = p.mask && p.ldmask % 8 == 0 && (uintptr_t)p.mask % 16 == 0;
+    p.vec_bf16 = p.out_bf16 && p.ld_bf16 % 8 == 0 && (uintptr_t)p.out_bf16 % 16 == 0;
+    p.vec_f32 = p.out_f32 && p.ld_f32 % 4 == 0 && (uintptr_t)p.out_f32 % 16 == 0;
     switch (BN) {
         case 32: return launch_gemm_t<32, 4>(p, splits, st);
-        // 3 stages of 32 KiB: two CTAs per SM keep twice the operand bytes in flight
-        // (layer 1 at 65536 rows: 133 -> 107 us against 4 stages and one CTA)
-        case 128: return launch_gemm_t<128, 3>(p, splits, st);
-        default: return launch_gemm_t<256, 3>(p, splits, st);
+        // with more tiles than SMs, 3 stages of 32 KiB: two CTAs per SM keep twice the operand
+        // bytes in flight (layer 1 at 65536 rows: 133 -> 107 us against 4 stages and one CTA);
+        // with fewer, one CTA per SM that keeps five chunks in flight
+        case 128: return tiles * splits > sms ? launch_gemm_t<128, 3>(p, splits, st) : launch_gemm_t<128, 6>(p, splits, st);
+        default: return launch_gemm_t<256, 4>(p, splits, st);
     }
 }
 
@@ -141,51 +145,105 @@ static tc::GemmParams gemm_params(const bf16 *A, long long lda, const bf16 *B, l
 // small CUDA-core kernels of the MLP
 // ---------------------------------------------------------------------------------------
 
-// fp32 [rows][cols] -> bf16 [rows][cols] and bf16 [cols][ld_t] transposed (zero columns of
-// the transposed copy beyond rows are left untouched: the caller zeroes them once)
-__global__ void pack_weight_kernel(const float *__restrict__ W, int rows, int cols, bf16 *__restrict__ Wb,
-                                   bf16 *__restrict__ Wt, int ld_t) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows * cols) return;
-    const int r = i / cols, c = i % cols;
-    const bf16 v = __float2bfloat16_rn(W[i]);
-    if (Wb) Wb[i] = v;
-    if (Wt) Wt[(long long)c * ld_t + r] = v;
+// The bf16 operand copies of the three weight matrices in one launch: fp32 [rows][cols] -> bf16
+// [rows][cols], and for W2, W3 also transposed, [cols][ld_t] (columns of the transposed copy
+// beyond rows are left untouched: the caller zeroes them once).
+__global__ void __launch_bounds__(256) pack_weights_kernel(const float *__restrict__ W1, const float *__restrict__ W2,
+                                                           const float *__restrict__ W3, bf16 *__restrict__ W1b,
+                                                           bf16 *__restrict__ W2b, bf16 *__restrict__ W3b,
+                                                           bf16 *__restrict__ W2t, bf16 *__restrict__ W3t) {
+    pdl_begin();
+    constexpr int H = SG_MLP_HIDDEN, n1 = H * SG_MLP_IN, n2 = H * H, n3 = SG_MLP_OUT * H;
+    int i = blockIdx.x * 256 + threadIdx.x;
+    if (i < n1) {
+        W1b[i] = __float2bfloat16_rn(W1[i]);
+        return;
+    }
+    i -= n1;
+    if (i < n2) {
+        const bf16 v = __float2bfloat16_rn(W2[i]);
+        W2b[i] = v;
+        W2t[(i % H) * H + i / H] = v;
+        return;
+    }
+    i -= n2;
+    if (i < n3) {
+        const bf16 v = __float2bfloat16_rn(W3[i]);
+        W3b[i] = v;
+        W3t[(i % H) * 64 + i / H] = v;
+    }
 }
 
-// dY = 2 w_o (Y - T) / B (bf16, [B][64] with columns >= 32 zero, and [32][B]); loss += sum
-__global__ void mse_head_kernel(const float *__restrict__ Y, const float *__restrict__ T,
-                                const float *__restrict__ w, int B, bf16 *__restrict__ dY,
-                                bf16 *__restrict__ dYt, float *__restrict__ loss) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;  // over B * 64
+// dY = 2 w_o (Y - T) / B (bf16, [B][64] with columns >= 32 zero, and [32][B]); loss += sum.
+// A block takes 64 rows, a thread four outputs of two rows at a time (16-byte loads, 8-byte
+// stores); the transposed copy goes through shared memory so that its rows are written 128
+// bytes at a time (16384 rows: 27 -> 4 us against one 2-byte store per element).
+__global__ void __launch_bounds__(256) mse_head_kernel(const float *__restrict__ Y, const float *__restrict__ T,
+                                                       const float *__restrict__ w, int B, bf16 *__restrict__ dY,
+                                                       bf16 *__restrict__ dYt, float *__restrict__ loss, bool vec) {
+    pdl_begin();
+    __shared__ uint16_t s_t[32][64 + 2];
+    const int b0 = blockIdx.x * 64;
     float l = 0.f;
-    if (i < B * 64) {
-        const int b = i / 64, o = i % 64;
-        float g = 0.f;
-        if (o < 32) {
-            const float d = Y[(long long)b * 32 + o] - T[(long long)b * 32 + o];
-            l = w[o] * d * d / (float)B;
-            g = 2.f * w[o] * d / (float)B;
-            dYt[(long long)o * B + b] = __float2bfloat16_rn(g);
+    for (int i = threadIdx.x; i < 64 * 8; i += 256) {
+        const int r = i >> 3, o = (i & 7) * 4, b = b0 + r;  // (B is a multiple of 128)
+        const float *yp = Y + (long long)b * 32 + o, *tp = T + (long long)b * 32 + o;
+        float d[4];
+        if (vec) {
+            const float4 y = *reinterpret_cast<const float4 *>(yp), t = *reinterpret_cast<const float4 *>(tp);
+            d[0] = y.x - t.x; d[1] = y.y - t.y; d[2] = y.z - t.z; d[3] = y.w - t.w;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) d[k] = yp[k] - tp[k];
         }
-        dY[(long long)b * 64 + o] = __float2bfloat16_rn(g);
+        uint16_t h[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            l += w[o + k] * d[k] * d[k] / (float)B;
+            h[k] = __bfloat16_as_ushort(__float2bfloat16_rn(2.f * w[o + k] * d[k] / (float)B));
+            s_t[o + k][r] = h[k];
+        }
+        uint2 *row = reinterpret_cast<uint2 *>(dY + (long long)b * 64 + o);
+        row[0] = make_uint2(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16));
+        row[8] = make_uint2(0u, 0u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 32 * 32; i += 256) {
+        const int o = i >> 5, r = (i & 31) * 2;
+        *reinterpret_cast<uint32_t *>(dYt + (long long)o * B + b0 + r) = s_t[o][r] | ((uint32_t)s_t[o][r + 1] << 16);
     }
     for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(SG_FULL_MASK, l, off);
     if ((threadIdx.x & 31) == 0 && l != 0.f) atomicAdd(loss, l);
 }
 
-// out[r] += sum_c M[r][c] for a bf16 [rows][cols] matrix (one CTA per row)
-__global__ void row_sum_kernel(const bf16 *__restrict__ M, int cols, float *__restrict__ out) {
-    const int r = blockIdx.x;
+// Bias gradients: out[r] += sum_c M[r][c] for the rows of three bf16 [rows][cols] matrices (one
+// CTA per row, 16-byte loads; cols is a multiple of 128).
+struct RowSums {
+    const bf16 *M[3];
+    float *out[3];
+    int rows[3];
+};
+__global__ void __launch_bounds__(256) row_sum_kernel(RowSums a, int cols) {
+    pdl_begin();
+    const int b1 = a.rows[0], b2 = b1 + a.rows[1], i = blockIdx.x;
+    const bf16 *M = i < b1 ? a.M[0] : i < b2 ? a.M[1] : a.M[2];
+    float *out = i < b1 ? a.out[0] : i < b2 ? a.out[1] : a.out[2];
+    const int r = i < b1 ? i : i < b2 ? i - b1 : i - b2;
+    const uint4 *row = reinterpret_cast<const uint4 *>(M + (long long)r * cols);
     float s = 0.f;
-    for (int c = threadIdx.x; c < cols; c += blockDim.x) s += __bfloat162float(M[(long long)r * cols + c]);
+    for (int c = threadIdx.x; c < cols / 8; c += 256) {
+        const uint4 q = row[c];
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s += __uint_as_float(w[i] << 16) + __uint_as_float(w[i] & 0xffff0000u);
+    }
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(SG_FULL_MASK, s, off);
-    __shared__ float sw[32];
+    __shared__ float sw[8];
     if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
         float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sw[w];
+        for (int w = 0; w < 8; ++w) t += sw[w];
         out[r] += t;
     }
 }
@@ -242,13 +300,10 @@ sg_status sg_mlp_pack_weights(const float *W1, const float *W2, const float *W3,
                               uint16_t *W3b, uint16_t *W2t, uint16_t *W3t, sg_stream_t stream) {
     MLP_REQUIRE(W1 && W2 && W3 && W1b && W2b && W3b && W2t && W3t, "pack_weights: NULL argument");
     cudaStream_t st = (cudaStream_t)stream;
-    pack_weight_kernel<<<(SG_MLP_HIDDEN * SG_MLP_IN + 255) / 256, 256, 0, st>>>(W1, SG_MLP_HIDDEN, SG_MLP_IN,
-                                                                                 (bf16 *)W1b, nullptr, 0);
-    pack_weight_kernel<<<(SG_MLP_HIDDEN * SG_MLP_HIDDEN + 255) / 256, 256, 0, st>>>(
-        W2, SG_MLP_HIDDEN, SG_MLP_HIDDEN, (bf16 *)W2b, (bf16 *)W2t, SG_MLP_HIDDEN);
-    pack_weight_kernel<<<(SG_MLP_OUT * SG_MLP_HIDDEN + 255) / 256, 256, 0, st>>>(
-        W3, SG_MLP_OUT, SG_MLP_HIDDEN, (bf16 *)W3b, (bf16 *)W3t, 64);
-    count_launches(3);
+    const int n = SG_MLP_HIDDEN * (SG_MLP_IN + SG_MLP_HIDDEN + SG_MLP_OUT);
+    launch_pdl(pack_weights_kernel, (n + 255) / 256, 256, 0, st, W1, W2, W3, (bf16 *)W1b, (bf16 *)W2b, (bf16 *)W3b,
+               (bf16 *)W2t, (bf16 *)W3t);
+    count_launches(1);
     return check_launch("mlp_pack_weights");
 }
 
@@ -286,8 +341,8 @@ sg_status sg_mlp_backward(const sg_mlp *net, const uint16_t *Xt, const float *ta
     MLP_REQUIRE(B > 0 && B % 128 == 0, "mlp_backward: B = %d must be a positive multiple of 128", B);
     cudaStream_t st = (cudaStream_t)stream;
     const int H = SG_MLP_HIDDEN, O = SG_MLP_OUT;
-    mse_head_kernel<<<(B * 64 + 255) / 256, 256, 0, st>>>(acts->Y, target, out_weight, B, (bf16 *)acts->dY,
-                                                          (bf16 *)acts->dYt, loss);
+    launch_pdl(mse_head_kernel, B / 64, 256, 0, st, acts->Y, target, out_weight, B, (bf16 *)acts->dY, (bf16 *)acts->dYt,
+               loss, (((uintptr_t)acts->Y | (uintptr_t)target) & 15) == 0);
     count_launches(1);
     // dW3 [32][128] += (H2^T dY)^T
     tc::GemmParams p = gemm_params((const bf16 *)acts->H2t, B, (const bf16 *)acts->dYt, B, H, O, B, status);
@@ -313,10 +368,11 @@ sg_status sg_mlp_backward(const sg_mlp *net, const uint16_t *Xt, const float *ta
     p.out_f32 = grads->W1; p.ld_f32 = SG_MLP_IN; p.f32_atomic = 1;
     MLP_TRY(launch_gemm(p, st));
     // bias gradients: row sums of the transposed copies
-    row_sum_kernel<<<O, 256, 0, st>>>((const bf16 *)acts->dYt, B, grads->b3);
-    row_sum_kernel<<<H, 256, 0, st>>>((const bf16 *)acts->dH2t, B, grads->b2);
-    row_sum_kernel<<<H, 256, 0, st>>>((const bf16 *)acts->dH1t, B, grads->b1);
-    count_launches(3);
+    const RowSums rs{{(const bf16 *)acts->dYt, (const bf16 *)acts->dH2t, (const bf16 *)acts->dH1t},
+                     {grads->b3, grads->b2, grads->b1},
+                     {O, H, H}};
+    launch_pdl(row_sum_kernel, O + 2 * H, 256, 0, st, rs, B);
+    count_launches(1);
     return check_launch("mlp_backward");
 }
 

@@ -188,6 +188,12 @@ __device__ __forceinline__ void red_add_v2(float *addr, float a, float b) {
     asm volatile("red.global.add.v2.f32 [%0], {%1, %2};\n" ::"l"(addr), "f"(a), "f"(b) : "memory");
 }
 
+// Four float additions to consecutive, 16-byte aligned addresses in one vector reduction.
+__device__ __forceinline__ void red_add_v4(float *addr, float a, float b, float c, float d) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d)
+                 : "memory");
+}
+
 // ----------------------------------------------------------------------------------------
 // Programmatic dependent launch.  The kernels of one iteration are launched with
 // launch_pdl() (programmatic stream serialisation), and every kernel starts with

@@ -87,3 +87,44 @@ def test_stacks_around_the_chunk_size_match_oracle(n, C, cfg):
     r.backward(p, grads, dL=tuple(torch.tensor(u.reshape(-1), device="cuda") for u in up))
     want = oracle.render_backward(g, cam, *[u.astype(np.float64) for u in up])
     check_grads({k: v.cpu().numpy() for k, v in grads.items()}, want, KEYS)
+
+
+@pytest.mark.parametrize("M, N, K, pad", [(130, 72, 128, 0), (130, 72, 128, 1), (128, 160, 4096, 4), (64, 288, 192, 3),
+                                          (300, 32, 64, 2)])
+@pytest.mark.parametrize("accumulate", [0, 1])
+def test_gemm_epilogue_edges_and_unaligned_rows(M, N, K, pad, accumulate):
+    """32-column blocks that end inside or at the matrix, output rows with and without 16-byte
+    alignment, stored and accumulated (4-wide reductions): the tolerance of the GEMM tests, and
+    nothing written beyond the N columns of a row."""
+    import ctypes
+    from paper_2412_01217_gb300._lib import call
+    torch.manual_seed(M + N + pad)
+    A = torch.randn(M, K, device="cuda").to(torch.bfloat16)
+    B = torch.randn(N, K, device="cuda").to(torch.bfloat16)
+    D = torch.full((M, N + pad), 0.5, device="cuda")
+    ptr = lambda t: ctypes.c_void_p(t.data_ptr())
+    call("sg_gemm_bf16", ptr(A), K, ptr(B), K, M, N, K, ptr(D), N + pad, accumulate, None,
+         ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    torch.cuda.synchronize()
+    ref = A.double() @ B.double().T + (0.5 if accumulate else 0.0)
+    assert (D[:, :N].double() - ref).abs().max().item() <= 1e-5 * ref.abs().max().item() + 1e-3
+    assert bool((D[:, N:] == 0.5).all())
+
+
+def test_mlp_backward_takes_unaligned_targets():
+    """The loss head reads Y and the targets 16 bytes at a time only when both are aligned: the
+    same batch with targets one float off gives the same bf16 output gradients."""
+    from paper_2412_01217_gb300.learned_init import MLPInit
+    B = 256
+    torch.manual_seed(1)
+    X = torch.randn(B, 2048, device="cuda").to(torch.bfloat16)
+    buf = torch.randn(B * 32 + 1, device="cuda")
+    shifted = buf[1:].view(B, 32)
+    out = []
+    for T in (shifted, shifted.clone()):
+        net = MLPInit(seed=3)
+        net.train_step(X, X.T.contiguous(), T, B, torch.zeros(1, device="cuda"))
+        a, _ = net.acts(B)
+        out.append({k: a[k].clone() for k in ("dY", "dYt", "dH2", "dH1t")})
+    for k in out[0]:
+        assert torch.equal(out[0][k], out[1][k]), k
