@@ -26,51 +26,89 @@ struct Frame {
     float fx, fy, cx, cy;
 };
 
-__device__ __forceinline__ float patch_feature(const Frame &fr, int x0, int y0, int f) {
-    if (f >= kPatchFeat) return 0.f;
-    const int pix = f / kPatchCh, ch = f % kPatchCh;
-    const int x = x0 + pix % kPatch - kPatch / 2, y = y0 + pix / kPatch - kPatch / 2;
-    if (x < 0 || y < 0 || x >= fr.W || y >= fr.H) return 0.f;
-    const size_t p = (size_t)y * fr.W + x, HW = (size_t)fr.W * fr.H;
-    if (ch < 3) return fr.rgb[ch * HW + p];
-    const float d = fr.depth[p];
-    if (ch == 3) return d > 0.f ? d : 0.f;
-    if (ch < 36) return fr.label && fr.label[p] == ch - 4 ? 1.f : 0.f;
-    if (ch < 39) {
-        const float rx = (x - fr.cx) / fr.fx, ry = (y - fr.cy) / fr.fy;
-        const float inv = rsqrtf(rx * rx + ry * ry + 1.f);
-        return ch == 36 ? rx * inv : (ch == 37 ? ry * inv : inv);
+// Patch features of ROWS pixels per block, into X [B_pad][2048] and/or Xt [2048][B_pad]
+// (rows from B on are zero).  The 49 x 9 values of each pixel's patch (label channels aside) are
+// formed once and kept in shared memory as bf16 next to the labels; features are then written
+// 8 at a time (X: one 16-byte store per thread, a row per pass of the block; Xt: 16 rows of the
+// batch, 32 bytes, per half warp).  One thread per element formed every feature from the images
+// again, with two integer divisions each (5120 rows into X: 50 us).  X alone takes 4 rows per
+// block, so that the gathers of 1280 blocks overlap (16 rows per block: 19 us).
+constexpr int kPatchVals = 9;  // rgb, depth, ray, valid, 1/fx
+template <int ROWS>
+__global__ void __launch_bounds__(256) patch_kernel(Frame fr, const int2 *__restrict__ pix, int B, int B_pad,
+                                                    uint16_t *__restrict__ X, uint16_t *__restrict__ Xt, bool vec) {
+    pdl_begin();
+    constexpr int NP = kPatch * kPatch;
+    __shared__ uint16_t s_v[ROWS][NP][kPatchVals];
+    __shared__ int s_lab[ROWS][NP];
+    const int b0 = blockIdx.x * ROWS;
+    const size_t HW = (size_t)fr.W * fr.H;
+    auto bits = [](float v) { return __bfloat16_as_ushort(__float2bfloat16_rn(v)); };
+    for (int i = threadIdx.x; i < ROWS * NP; i += 256) {
+        const int r = i / NP, k = i % NP, b = b0 + r;
+        float v[kPatchVals];
+#pragma unroll
+        for (int c = 0; c < kPatchVals; ++c) v[c] = 0.f;
+        int lab = -1;
+        if (b < B) {
+            const int2 q = pix[b];
+            const int x = q.x + k % kPatch - kPatch / 2, y = q.y + k / kPatch - kPatch / 2;
+            if (!(x < 0 || y < 0 || x >= fr.W || y >= fr.H)) {
+                const size_t p = (size_t)y * fr.W + x;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) v[c] = fr.rgb[c * HW + p];
+                const float d = fr.depth[p];
+                v[3] = d > 0.f ? d : 0.f;
+                if (fr.label) lab = fr.label[p];
+                const float rx = (x - fr.cx) / fr.fx, ry = (y - fr.cy) / fr.fy;
+                const float inv = rsqrtf(rx * rx + ry * ry + 1.f);
+                v[4] = rx * inv;
+                v[5] = ry * inv;
+                v[6] = inv;
+                v[7] = d > 0.f ? 1.f : 0.f;
+                v[8] = 1.f / fr.fx;
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < kPatchVals; ++c) s_v[r][k][c] = bits(v[c]);
+        s_lab[r][k] = lab;
     }
-    if (ch == 39) return d > 0.f ? 1.f : 0.f;
-    return 1.f / fr.fx;
-}
-
-// X [B_pad][2048] row-major (coalesced over features)
-__global__ void patch_rows_kernel(Frame fr, const int2 *__restrict__ pix, int B, int B_pad,
-                                  __nv_bfloat16 *__restrict__ X) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)B_pad * SG_MLP_IN) return;
-    const int b = (int)(i / SG_MLP_IN), f = (int)(i % SG_MLP_IN);
-    float v = 0.f;
-    if (b < B) {
-        const int2 q = pix[b];
-        v = patch_feature(fr, q.x, q.y, f);
+    __syncthreads();
+    const uint16_t one = bits(1.f);
+    // channel f % 41: rgb, depth, 32 label channels, ray, valid, 1/fx; features from 2009 on are 0
+    auto feature = [&](int r, int k, int ch) -> uint32_t {
+        if (ch < 4) return s_v[r][k][ch];
+        if (ch < 36) return s_lab[r][k] == ch - 4 ? one : 0;
+        return s_v[r][k][ch - 32];
+    };
+    if (X) {
+        const int f0 = threadIdx.x * 8;  // 256 x 8 = 2048 features
+        for (int r = 0; r < ROWS; ++r) {
+            int k = f0 / kPatchCh, ch = f0 % kPatchCh;
+            uint32_t h[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                h[j] = f0 + j < kPatchFeat ? feature(r, k, ch) : 0u;
+                if (++ch == kPatchCh) {
+                    ch = 0;
+                    ++k;
+                }
+            }
+            uint16_t *o = X + (size_t)(b0 + r) * SG_MLP_IN + f0;
+            if (vec) {
+                *reinterpret_cast<uint4 *>(o) =
+                    make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) o[j] = (uint16_t)h[j];
+            }
+        }
     }
-    X[i] = __float2bfloat16_rn(v);
-}
-
-// Xt [2048][B_pad] (coalesced over rows of the batch)
-__global__ void patch_cols_kernel(Frame fr, const int2 *__restrict__ pix, int B, int B_pad,
-                                  __nv_bfloat16 *__restrict__ Xt) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)B_pad * SG_MLP_IN) return;
-    const int f = (int)(i / B_pad), b = (int)(i % B_pad);
-    float v = 0.f;
-    if (b < B) {
-        const int2 q = pix[b];
-        v = patch_feature(fr, q.x, q.y, f);
+    if (Xt) {
+        const int r = threadIdx.x % ROWS;
+        for (int f = threadIdx.x / ROWS; f < SG_MLP_IN; f += 256 / ROWS)
+            Xt[(size_t)f * B_pad + b0 + r] = f < kPatchFeat ? (uint16_t)feature(r, f / kPatchCh, f % kPatchCh) : 0;
     }
-    Xt[i] = __float2bfloat16_rn(v);
 }
 
 struct InitOut {
@@ -79,6 +117,7 @@ struct InitOut {
 
 __global__ void heuristic_init_kernel(Frame fr, sg_camera cam, const int2 *__restrict__ pix, int B, int C,
                                       const float *__restrict__ code, int n_classes, float kappa, InitOut o) {
+    pdl_begin();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
     const int2 q = pix[b];
@@ -111,6 +150,7 @@ __global__ void heuristic_init_kernel(Frame fr, sg_camera cam, const int2 *__res
 __global__ void apply_mlp_kernel(const float *__restrict__ Y, int B, int C, const float *__restrict__ mu,
                                  const float *__restrict__ sd, float *__restrict__ log_scale,
                                  float *__restrict__ opacity_logit, float *__restrict__ sem) {
+    pdl_begin();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
     const float *y = Y + (size_t)b * SG_MLP_OUT;
@@ -134,17 +174,10 @@ sg_status sg_extract_patches(const float *rgb, const float *depth, const int32_t
     }
     Frame fr{rgb, depth, label, cam->W, cam->H, cam->fx, cam->fy, cam->cx, cam->cy};
     cudaStream_t st = (cudaStream_t)stream;
-    const long long n = (long long)B_pad * SG_MLP_IN;
-    const int blocks = (int)((n + 255) / 256);
-    if (blocks > 0) {
-        if (X) {
-            patch_rows_kernel<<<blocks, 256, 0, st>>>(fr, (const int2 *)pixels, B, B_pad, (__nv_bfloat16 *)X);
-            count_launches(1);
-        }
-        if (Xt) {
-            patch_cols_kernel<<<blocks, 256, 0, st>>>(fr, (const int2 *)pixels, B, B_pad, (__nv_bfloat16 *)Xt);
-            count_launches(1);
-        }
+    if (B_pad > 0) {
+        launch_pdl(Xt ? patch_kernel<16> : patch_kernel<4>, B_pad / (Xt ? 16 : 4), 256, 0, st, fr, (const int2 *)pixels, B,
+                   B_pad, X, Xt, ((uintptr_t)X & 15) == 0);
+        count_launches(1);
     }
     return check_launch("extract_patches");
 }
@@ -160,8 +193,8 @@ sg_status sg_init_gaussians(const float *rgb, const float *depth, const int32_t 
     if (B == 0) return SG_OK;
     Frame fr{rgb, depth, label, cam->W, cam->H, cam->fx, cam->fy, cam->cx, cam->cy};
     InitOut o{out->mean, out->log_scale, out->quat, out->opacity_logit, out->rgb, out->sem};
-    heuristic_init_kernel<<<(B + 127) / 128, 128, 0, (cudaStream_t)stream>>>(fr, *cam, (const int2 *)pixels, B,
-                                                                             out->C, sem_code, n_classes, kappa, o);
+    launch_pdl(heuristic_init_kernel, (B + 127) / 128, 128, 0, (cudaStream_t)stream, fr, *cam, (const int2 *)pixels, B,
+               out->C, sem_code, n_classes, kappa, o);
     count_launches(1);
     return check_launch("init_gaussians");
 }
@@ -173,8 +206,8 @@ sg_status sg_apply_mlp_init(const float *Y, int32_t B, const float *y_mean, cons
         return SG_ERR_INVALID_ARG;
     }
     if (B == 0) return SG_OK;
-    apply_mlp_kernel<<<(B + 127) / 128, 128, 0, (cudaStream_t)stream>>>(Y, B, out->C, y_mean, y_std, out->log_scale,
-                                                                        out->opacity_logit, out->sem);
+    launch_pdl(apply_mlp_kernel, (B + 127) / 128, 128, 0, (cudaStream_t)stream, Y, B, out->C, y_mean, y_std,
+               out->log_scale, out->opacity_logit, out->sem);
     count_launches(1);
     return check_launch("apply_mlp_init");
 }
