@@ -8,6 +8,8 @@ from __future__ import annotations
 import ctypes as C
 import os
 
+import torch
+
 from . import _build
 
 c_f = C.c_float
@@ -139,6 +141,13 @@ SIGNATURES = {
 }
 
 _lib = None
+
+
+def stream_ptr():
+    """The current device's current stream, as the C ABI takes it.  Read straight from the
+    runtime's per-thread state: torch.cuda.current_stream() builds a Stream object behind three
+    Python layers, 19 us on the target's host cores, five times in a forward and backward."""
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
 
 
 class SgError(RuntimeError):

@@ -16,7 +16,7 @@ import math
 import torch
 
 from . import _lib
-from ._lib import SgAdamGroup, SgMlp, SgMlpActs, SgMlpGrads, call
+from ._lib import SgAdamGroup, SgMlp, SgMlpActs, SgMlpGrads, call, stream_ptr
 
 IN, HID, OUT = 2048, 128, 32
 USED_OUT = 20  # log-scale 3, opacity logit 1, semantic feature 16
@@ -24,10 +24,6 @@ USED_OUT = 20  # log-scale 3, opacity logit 1, semantic feature 16
 
 def _p(t):
     return C.c_void_p(t.data_ptr()) if t is not None else C.c_void_p(0)
-
-
-def _s():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
 
 
 class MLPInit:
@@ -63,7 +59,7 @@ class MLPInit:
 
     def pack(self):
         call("sg_mlp_pack_weights", _p(self.W1), _p(self.W2), _p(self.W3), _p(self.W1b), _p(self.W2b),
-             _p(self.W3b), _p(self.W2t), _p(self.W3t), _s())
+             _p(self.W3b), _p(self.W2t), _p(self.W3t), stream_ptr())
 
     def net(self):
         return SgMlp(*[t.data_ptr() for t in (self.W1b, self.W2b, self.W3b, self.W2t, self.W3t, self.b1,
@@ -90,7 +86,7 @@ class MLPInit:
     def forward(self, X, B):
         a, s = self.acts(B)
         net = self.net()
-        call("sg_mlp_forward", C.byref(net), _p(X), B, C.byref(s), _p(self.status), _s())
+        call("sg_mlp_forward", C.byref(net), _p(X), B, C.byref(s), _p(self.status), stream_ptr())
         return a["Y"]
 
     def train_step(self, X, Xt, T_std, B, loss_acc):
@@ -98,14 +94,14 @@ class MLPInit:
         a, s = self.acts(B)
         net = self.net()
         G = SgMlpGrads(*[t.data_ptr() for t in self.grads])
-        call("sg_mlp_forward", C.byref(net), _p(X), B, C.byref(s), _p(self.status), _s())
+        call("sg_mlp_forward", C.byref(net), _p(X), B, C.byref(s), _p(self.status), stream_ptr())
         call("sg_mlp_backward", C.byref(net), _p(Xt), _p(T_std), _p(self.out_w), B, C.byref(s), C.byref(G),
-             _p(loss_acc), _p(self.status), _s())
+             _p(loss_acc), _p(self.status), stream_ptr())
         self.step_count += 1
         groups = (SgAdamGroup * 6)(*[SgAdamGroup(p.data_ptr(), g.data_ptr(), m.data_ptr(), v.data_ptr(),
                                                   p.numel(), self.lr)
                                      for p, g, m, v in zip(self.params, self.grads, self.m, self.v)])
-        call("sg_adam_multi", groups, 6, 0.9, 0.999, 1e-8, self.step_count, 1, None, _s())
+        call("sg_adam_multi", groups, 6, 0.9, 0.999, 1e-8, self.step_count, 1, None, stream_ptr())
         self.W1[:, 2009:] = 0  # padding features stay inert
         self.pack()
 

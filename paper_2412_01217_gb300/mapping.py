@@ -17,17 +17,13 @@ import numpy as np
 import torch
 
 from . import _lib
-from ._lib import call
+from ._lib import call, stream_ptr
 from .splat import (LossConfig, MappingStep, PyramidRasterizer, RenderConfig, build_pyramid,
                     camera_struct, gaussians_struct)
 
 
 def _p(t):
     return C.c_void_p(t.data_ptr()) if t is not None else C.c_void_p(0)
-
-
-def _s():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
 
 
 class Mapper:
@@ -107,16 +103,16 @@ class Mapper:
         cam = camera_struct(self.cams[k])
         out = gaussians_struct({kk: v[self.N:self.N + B] for kk, v in self.P.items()})
         call("sg_init_gaussians", _p(rgb), _p(depth), _p(label), C.byref(cam), _p(pix_d), B, _p(self.decoder),
-             self.n_classes, kappa, C.byref(out), _s())
+             self.n_classes, kappa, C.byref(out), stream_ptr())
         if init == "learned":
             Bp = ((B + 127) // 128) * 128
             X = torch.empty(Bp, 2048, dtype=torch.bfloat16, device=self.dev)
             t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             t0.record()
             call("sg_extract_patches", _p(rgb), _p(depth), _p(label), C.byref(cam), _p(pix_d), B, Bp, _p(X), None,
-                 _s())
+                 stream_ptr())
             Y = mlp.forward(X, Bp)
-            call("sg_apply_mlp_init", _p(Y), B, _p(mlp.y_mean), _p(mlp.y_std), C.byref(out), _s())
+            call("sg_apply_mlp_init", _p(Y), B, _p(mlp.y_mean), _p(mlp.y_std), C.byref(out), stream_ptr())
             t1.record()
             t1.synchronize()
             self.mlp_seconds += t0.elapsed_time(t1) / 1e3

@@ -13,7 +13,7 @@ import torch
 
 from . import _lib
 from ._lib import (SgCamera, SgConfig, SgGaussians, SgImages, SgLossConfig, SgProjected, SgSaved,
-                   SgTargets, SgTileLists, SgView, call)
+                   SgTargets, SgTileLists, SgView, call, stream_ptr)
 
 PARAM_KEYS = ("mean", "log_scale", "quat", "opacity_logit", "rgb", "sem")
 
@@ -46,8 +46,7 @@ def _ptr(t):
     return C.c_void_p(t.data_ptr()) if t is not None else C.c_void_p(0)
 
 
-def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+_stream = stream_ptr
 
 
 def require_cuda():
@@ -149,11 +148,12 @@ def views_to_device(views, device):
 
 
 def gaussians_struct(g, N=None, C_=None):
-    s = SgGaussians()
-    s.mean, s.log_scale, s.quat = g["mean"].data_ptr(), g["log_scale"].data_ptr(), g["quat"].data_ptr()
-    s.opacity_logit, s.rgb, s.sem = g["opacity_logit"].data_ptr(), g["rgb"].data_ptr(), g["sem"].data_ptr()
-    s.N = g["mean"].shape[0] if N is None else N
-    s.C = g["sem"].shape[1] if C_ is None else C_
+    mean, sem = g["mean"], g["sem"]
+    s = SgGaussians(mean.data_ptr(), g["log_scale"].data_ptr(), g["quat"].data_ptr(), g["opacity_logit"].data_ptr(),
+                    g["rgb"].data_ptr(), sem.data_ptr(), mean.shape[0] if N is None else N,
+                    sem.shape[1] if C_ is None else C_)
+    if g.get("sh") is None and g.get("sem_sh") is None:
+        return s
     D = sh_degree(g)
     if D:
         s.sh_degree = D
@@ -254,6 +254,8 @@ class PyramidRasterizer:
                                   device=self.device)
 
     def _check_colour(self, g):
+        if g.get("sh") is None and g.get("sem_sh") is None:
+            return
         keys = param_keys(g)
         need = [("sh" in keys and self.rec_rgb is None, self._alloc_record_colour),
                 ("sem_sh" in keys and self.rec_sem is None, self._alloc_record_semantics)]
@@ -426,7 +428,9 @@ class PyramidSplat(torch.autograd.Function):
     def backward(ctx, d_rgb, d_depth, d_sem):
         rast = ctx.rast
         params = dict(zip(ctx.keys, ctx.saved_tensors))
-        grads = {k: torch.zeros_like(v) for k, v in params.items()}
+        # separate tensors, zeroed by one launch
+        grads = {k: torch.empty_like(v) for k, v in params.items()}
+        torch._foreach_zero_(list(grads.values()))
         z = lambda t, n: t.contiguous() if t is not None else torch.zeros(n, dtype=torch.float32, device=rast.device)
         rast.backward(params, grads, dL=(z(d_rgb, 3 * rast.P), z(d_depth, rast.P), z(d_sem, rast.C * rast.P)))
         return (None, *[grads[k] for k in PARAM_KEYS], grads.get("sh"), grads.get("sem_sh"))
