@@ -217,7 +217,8 @@ __global__ void __launch_bounds__(256) mse_head_kernel(const float *__restrict__
 }
 
 // Bias gradients: out[r] += sum_c M[r][c] for the rows of three bf16 [rows][cols] matrices (one
-// CTA per row, 16-byte loads; cols is a multiple of 128).
+// CTA per row; cols is a multiple of 128).  2048 columns at a time through shared memory: 16-byte
+// loads, while thread t sums columns t, t + 256, ... in order.
 struct RowSums {
     const bf16 *M[3];
     float *out[3];
@@ -230,12 +231,20 @@ __global__ void __launch_bounds__(256) row_sum_kernel(RowSums a, int cols) {
     float *out = i < b1 ? a.out[0] : i < b2 ? a.out[1] : a.out[2];
     const int r = i < b1 ? i : i < b2 ? i - b1 : i - b2;
     const uint4 *row = reinterpret_cast<const uint4 *>(M + (long long)r * cols);
+    __shared__ uint4 s_q[256];
+    const uint16_t *s_c = reinterpret_cast<const uint16_t *>(s_q);
+    const int n8 = cols / 8, tid = threadIdx.x;
     float s = 0.f;
-    for (int c = threadIdx.x; c < cols / 8; c += 256) {
-        const uint4 q = row[c];
-        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+    uint4 next = tid < n8 ? row[tid] : make_uint4(0u, 0u, 0u, 0u);
+    for (int q0 = 0; q0 < n8; q0 += 256) {
+        s_q[tid] = next;
+        __syncthreads();
+        const int q = q0 + 256 + tid;
+        next = q < n8 ? row[q] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) s += __uint_as_float(w[i] << 16) + __uint_as_float(w[i] & 0xffff0000u);
+        for (int i = 0; i < 8; ++i)
+            if (8 * q0 + 256 * i + tid < cols) s += __uint_as_float((uint32_t)s_c[256 * i + tid] << 16);
+        __syncthreads();
     }
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(SG_FULL_MASK, s, off);
     __shared__ float sw[8];
