@@ -12,6 +12,7 @@
 // Depth term (Eq. 11): mean |D - D_gt| over pixels with D_gt > 0.
 // Semantic term, cross-entropy mode: mean CE(softmax(decoder * S), label) over label >= 0.
 // Sums are per-CTA partials reduced in a fixed order (deterministic).
+#include <algorithm>
 #include <cstdio>
 
 #include "sg_common.cuh"
@@ -59,38 +60,88 @@ __device__ __forceinline__ float block_sum(float v, float *s_red) {
     return t;  // valid in thread 0
 }
 
-struct SsimArgs {
-    const float *x, *y;  // planar images (rendered, target), nch planes per view
+// One term's images: nch planes per view.
+struct SsimPlanes {
+    const float *x, *y;  // planar images (rendered, target)
     float *grad;         // dL/dx
     int nch;
     float l1_coef_num;   // (1 - lambda) * weight  (divided by n = nch*W*H per view)
     float ssim_coef_num; // lambda * weight
+    float lambda;
+};
+// The planes are split over kSsimGroups groups of CTAs (blockIdx.y), a group's planes one after
+// the other: the first rgb_groups groups take the colour planes, the others the semantic
+// ones.  Each plane in a CTA of its own fills the chip three times as well on small image
+// sets (320x180 x 3 levels: 80 tiles on 152 SMs); the number of groups is what the workspace's
+// four floats per tile hold.
+constexpr int kSsimGroups = 4;
+struct SsimArgs {
+    SsimPlanes rgb, sem;
+    int rgb_groups, sem_groups;
     const sg_view *views;
     LossViews lv;
-    float *partials;     // per CTA: (sum |x - y|, sum ssim)
+    float *partials;     // per (group, tile): (1 - lambda) sum |x - y| - lambda sum ssim
     // valid-pixel counts (counts[2v]: target depth > 0, counts[2v+1]: label >= 0) gathered
-    // on the side, or null
+    // on the side by the first group; label may be null
     const float *gt_depth;
     const int *label;
     int *counts;
 };
 
+// A pair of floats multiplied and added by one instruction (fma.rn.f32x2; each half rounds as
+// fmaf does).
+struct F2 {
+    uint64_t v;
+};
+__device__ __forceinline__ F2 f2(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};\n" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack(F2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;\n" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+    return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+
 // Sliding-window separable passes: each thread produces a run of consecutive outputs of one
-// row (horizontal) or column (vertical) from a register window of input values.
+// row (horizontal) or column (vertical), adding each input to every output whose window
+// holds it.  The kernel is bound by instruction issue, so the window sums run two quantities
+// to an instruction: the planes are staged as (x, y) pairs, the four moments (x, y),
+// (x^2 + y^2, xy) -- SSIM takes the two variances only by their sum -- as 16-byte entries, and
+// two of the three partials as pairs, which also makes every shared-memory access of a pass
+// one 8- or 16-byte word.  1200x680 x 3 levels: 66 us against 101 with one quantity per
+// instruction, five moments and a tile's planes in one CTA (loss with a 32-class decoder
+// 233 -> 198 us; colour and four semantic planes at 637x477 x 3 levels 113 -> 81 us).
 __global__ void __launch_bounds__(kLossThreads, 3) ssim_l1_kernel(SsimArgs a) {
     pdl_begin();
     extern __shared__ __align__(16) float sm[];
-    float *X = sm;                   // kXH x kXP
-    float *Y = X + kXH * kXP;        // kXH x kXP
-    float *Hm = Y + kXH * kXP;       // 5 x kXH x kMP (later: 3 x kMH x kMP)
-    float *Mp = X;                   // 3 x kMH x kMP: reuses the staged planes once the
-                                     // horizontal pass has consumed them
+    float4 *Hm = reinterpret_cast<float4 *>(sm);                // kXH x kMP moments
+    float2 *XY = reinterpret_cast<float2 *>(Hm + kXH * kMP);    // kXH x kXP staged planes
+    // the partials reuse the staged planes once the horizontal pass has consumed them, and
+    // their horizontal sums the moments
+    float2 *PQ = XY;                                            // kMH x kMP
+    float *Rp = reinterpret_cast<float *>(PQ + kMH * kMP);      // kMH x kMP
+    constexpr int kHP = kLTW + 1;
+    float2 *HPQ = reinterpret_cast<float2 *>(Hm);               // kMH x kHP
+    float *HR = reinterpret_cast<float *>(HPQ + kMH * kHP);     // kMH x kHP
     static_assert(3 * kMH * kMP <= 2 * kXH * kXP, "partials must fit the staged planes");
+    static_assert(3 * kMH * kHP <= 4 * kXH * kMP, "their row sums must fit the moments");
+    static_assert(kLossThreads == 256 && kXW <= 64 && kLTH * kLTW == 4 * kLossThreads, "work split");
     __shared__ int s_cnt[2];
     __shared__ float w[11];
     __shared__ float s_red[kLossThreads / 32];
     if (threadIdx.x == 0) gauss_window(w);
-    const int item = blockIdx.x;
+    const int item = blockIdx.x, group = blockIdx.y;
+    const bool is_rgb = group < a.rgb_groups;
+    const SsimPlanes &pl = is_rgb ? a.rgb : a.sem;
+    const int sub = is_rgb ? group : group - a.rgb_groups, subs = is_rgb ? a.rgb_groups : a.sem_groups;
+    const int nch = pl.nch, ch0 = nch * sub / subs, ch1 = nch * (sub + 1) / subs;
     const int v = find_prefix(a.lv.tile_off, a.lv.n, item);
     const sg_view &vw = a.views[v];
     const int W = vw.W, H = vw.H;
@@ -99,60 +150,61 @@ __global__ void __launch_bounds__(kLossThreads, 3) ssim_l1_kernel(SsimArgs a) {
     const int bx = local % tiles_x, by = local / tiles_x;
     const int ox = bx * kLTW - 10, oy = by * kLTH - 10;
     const size_t HW = (size_t)W * H;
-    const float n = (float)a.nch * (float)HW;
-    const float l1c = a.l1_coef_num / n, sc = -a.ssim_coef_num / n;
+    const float n = (float)nch * (float)HW;
+    const float l1c = pl.l1_coef_num / n, sc = -pl.ssim_coef_num / n;
     const float C1 = 0.01f * 0.01f, C2 = 0.03f * 0.03f;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float l1_sum = 0.f, ssim_sum = 0.f;
-    int n_depth = 0, n_label = 0;
     if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
     __syncthreads();
-    float wr[11];
+    F2 wr[11];  // (weight, weight); the window is symmetric
 #pragma unroll
-    for (int i = 0; i < 11; ++i) wr[i] = w[i];
-    for (int ch = 0; ch < a.nch; ++ch) {
-        const float *xs = a.x + (size_t)a.nch * vw.pixel_offset + ch * HW;
-        const float *ys = a.y + (size_t)a.nch * vw.pixel_offset + ch * HW;
-        // stage x, y with a 10-pixel halo (zero outside the image)
-        for (int i = threadIdx.x; i < kXH * kXW; i += kLossThreads) {
-            const int r = i / kXW, c = i - r * kXW;
-            const int gy = oy + r, gx = ox + c;
-            const bool in = gx >= 0 && gx < W && gy >= 0 && gy < H;
-            X[r * kXP + c] = in ? xs[(size_t)gy * W + gx] : 0.f;
-            Y[r * kXP + c] = in ? ys[(size_t)gy * W + gx] : 0.f;
+    for (int i = 0; i < 6; ++i) wr[i] = wr[10 - i] = f2(w[i], w[i]);
+    auto w1 = [&](int j) { return unpack(wr[j]).x; };
+    for (int ch = ch0; ch < ch1; ++ch) {
+        const float *xs = pl.x + (size_t)nch * vw.pixel_offset + ch * HW;
+        const float *ys = pl.y + (size_t)nch * vw.pixel_offset + ch * HW;
+        // stage x, y with a 10-pixel halo (zero outside the image): a warp per row
+#pragma unroll
+        for (int cs = 0; cs < 2; ++cs) {
+            const int c = lane + 32 * cs, gx = ox + c;
+            const bool in_x = c < kXW && gx >= 0 && gx < W;
+#pragma unroll
+            for (int k = 0; k < (kXH + 7) / 8; ++k) {
+                const int r = warp + 8 * k, gy = oy + r;
+                const bool in = in_x && gy >= 0 && gy < H;
+                const size_t q = (size_t)gy * W + gx;
+                const float xv = in ? xs[q] : 0.f, yv = in ? ys[q] : 0.f;
+                if (c < kXW && r < kXH) XY[r * kXP + c] = make_float2(xv, yv);
+            }
         }
         __syncthreads();
-        // Run lengths are chosen so that every phase's work items fill whole rounds of the
-        // block's 256 threads (728, 252, 504 and 256 items).
-        // horizontal window sums of x, y, x^2, y^2, xy: rows kXH, outputs kMW in runs of 3
+        // Run lengths are chosen so that the passes' work items fill whole rounds of the
+        // block's 256 threads (728, 252, 168 and 256 items).
+        // horizontal window sums of the moments: rows kXH, outputs kMW in runs of 3
         {
             constexpr int RUN = 3, SEGS = kMW / RUN;  // 42 = 14 * 3
             for (int it = threadIdx.x; it < SEGS * kXH; it += kLossThreads) {
                 const int seg = it / kXH, r = it - seg * kXH;
                 const int c0 = seg * RUN;
-                float xv[RUN + 10], yv[RUN + 10];
+                F2 s[RUN][2];
+#pragma unroll
+                for (int o = 0; o < RUN; ++o) s[o][0] = s[o][1] = f2(0.f, 0.f);
 #pragma unroll
                 for (int i = 0; i < RUN + 10; ++i) {
-                    xv[i] = X[r * kXP + c0 + i];
-                    yv[i] = Y[r * kXP + c0 + i];
+                    const float2 q = XY[r * kXP + c0 + i];
+                    const F2 xy = f2(q.x, q.y), mom = f2(fmaf(q.y, q.y, q.x * q.x), q.x * q.y);
+#pragma unroll
+                    for (int o = 0; o < RUN; ++o)
+                        if (i - o >= 0 && i - o < 11) {
+                            s[o][0] = fma2(wr[i - o], xy, s[o][0]);
+                            s[o][1] = fma2(wr[i - o], mom, s[o][1]);
+                        }
                 }
 #pragma unroll
                 for (int o = 0; o < RUN; ++o) {
-                    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f, s4 = 0.f;
-#pragma unroll
-                    for (int j = 0; j < 11; ++j) {
-                        const float x = xv[o + j], y = yv[o + j];
-                        s0 = fmaf(wr[j], x, s0);
-                        s1 = fmaf(wr[j], y, s1);
-                        s2 = fmaf(wr[j], x * x, s2);
-                        s3 = fmaf(wr[j], y * y, s3);
-                        s4 = fmaf(wr[j], x * y, s4);
-                    }
-                    const int idx = r * kMP + c0 + o;
-                    Hm[0 * kXH * kMP + idx] = s0;
-                    Hm[1 * kXH * kMP + idx] = s1;
-                    Hm[2 * kXH * kMP + idx] = s2;
-                    Hm[3 * kXH * kMP + idx] = s3;
-                    Hm[4 * kXH * kMP + idx] = s4;
+                    const float2 p = unpack(s[o][0]), q = unpack(s[o][1]);
+                    Hm[r * kMP + c0 + o] = make_float4(p.x, p.y, q.x, q.y);
                 }
             }
         }
@@ -164,19 +216,19 @@ __global__ void __launch_bounds__(kLossThreads, 3) ssim_l1_kernel(SsimArgs a) {
             for (int it = threadIdx.x; it < SEGS * kMW; it += kLossThreads) {
                 const int seg = it / kMW, c = it - seg * kMW;
                 const int r0 = seg * RUN;
-                float m[5][RUN];
+                F2 m[RUN][2];
 #pragma unroll
-                for (int k = 0; k < 5; ++k) {
-                    float col[RUN + 10];
+                for (int o = 0; o < RUN; ++o) m[o][0] = m[o][1] = f2(0.f, 0.f);
 #pragma unroll
-                    for (int i = 0; i < RUN + 10; ++i) col[i] = Hm[k * kXH * kMP + (r0 + i) * kMP + c];
+                for (int i = 0; i < RUN + 10; ++i) {
+                    const float4 q = Hm[(r0 + i) * kMP + c];
+                    const F2 xy = f2(q.x, q.y), mom = f2(q.z, q.w);
 #pragma unroll
-                    for (int o = 0; o < RUN; ++o) {
-                        float acc = 0.f;
-#pragma unroll
-                        for (int j = 0; j < 11; ++j) acc = fmaf(wr[j], col[o + j], acc);
-                        m[k][o] = acc;
-                    }
+                    for (int o = 0; o < RUN; ++o)
+                        if (i - o >= 0 && i - o < 11) {
+                            m[o][0] = fma2(wr[i - o], xy, m[o][0]);
+                            m[o][1] = fma2(wr[i - o], mom, m[o][1]);
+                        }
                 }
 #pragma unroll
                 for (int o = 0; o < RUN; ++o) {
@@ -184,95 +236,120 @@ __global__ void __launch_bounds__(kLossThreads, 3) ssim_l1_kernel(SsimArgs a) {
                     const int gy = by * kLTH - 5 + r, gx = bx * kLTW - 5 + c;
                     float P = 0.f, Q = 0.f, R = 0.f;
                     if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
-                        const float mx = m[0][o], my = m[1][o];
-                        const float sxx = m[2][o] - mx * mx, syy = m[3][o] - my * my, sxy = m[4][o] - mx * my;
-                        const float A1 = 2.f * mx * my + C1, A2 = 2.f * sxy + C2;
-                        const float B1 = mx * mx + my * my + C1, B2 = sxx + syy + C2;
+                        const float2 mu = unpack(m[o][0]), e2 = unpack(m[o][1]);
+                        const float mx = mu.x, my = mu.y;
+                        const float A1 = 2.f * mx * my + C1, A2 = 2.f * (e2.y - mx * my) + C2;
+                        const float B1 = fmaf(mx, mx, my * my) + C1;
+                        const float B2 = fmaf(-my, my, fmaf(-mx, mx, e2.x)) + C2;
                         const float inv = 1.f / (B1 * B2);
                         const float s = A1 * A2 * inv;
                         if (r >= 5 && r < kLTH + 5 && c >= 5 && c < kLTW + 5) ssim_sum += s;
-                        const float d_mx = 2.f * my * A2 * inv - s * 2.f * mx / B1;
-                        const float d_sxx = -s / B2;
+                        const float d_mx = 2.f * my * A2 * inv - s * 2.f * mx * (B2 * inv);
+                        const float d_sxx = -s * (B1 * inv);
                         const float d_sxy = 2.f * A1 * inv;
                         P = sc * (d_mx - 2.f * mx * d_sxx - my * d_sxy);
                         Q = sc * d_sxx;
                         R = sc * d_sxy;
                     }
-                    Mp[0 * kMH * kMP + r * kMP + c] = P;
-                    Mp[1 * kMH * kMP + r * kMP + c] = Q;
-                    Mp[2 * kMH * kMP + r * kMP + c] = R;
+                    PQ[r * kMP + c] = make_float2(P, Q);
+                    Rp[r * kMP + c] = R;
                 }
             }
         }
         __syncthreads();
-        float *Hp = Hm;  // 3 x kMH x kMP, reuses the moment buffer
-        // horizontal sums of the partials: (partial, row, run of 8 outputs) per item
+        // horizontal sums of the partials: rows kMH, outputs kLTW in runs of 8
         {
             constexpr int RUN = 8, SEGS = kLTW / RUN;
-            for (int it = threadIdx.x; it < 3 * SEGS * kMH; it += kLossThreads) {
-                const int k = it / (SEGS * kMH), rem = it - k * (SEGS * kMH);
-                const int seg = rem / kMH, r = rem - seg * kMH;
+            if (threadIdx.x < SEGS * kMH) {
+                const int seg = threadIdx.x / kMH, r = threadIdx.x - seg * kMH;
                 const int c0 = seg * RUN;
-                {
-                    float row[RUN + 10];
+                F2 s[RUN];
+                float t[RUN];
 #pragma unroll
-                    for (int i = 0; i < RUN + 10; ++i) row[i] = Mp[k * kMH * kMP + r * kMP + c0 + i];
-#pragma unroll
-                    for (int o = 0; o < RUN; ++o) {
-                        float acc = 0.f;
-#pragma unroll
-                        for (int j = 0; j < 11; ++j) acc = fmaf(wr[j], row[o + j], acc);
-                        Hp[k * kMH * kMP + r * kMP + c0 + o] = acc;
-                    }
+                for (int o = 0; o < RUN; ++o) {
+                    s[o] = f2(0.f, 0.f);
+                    t[o] = 0.f;
                 }
-            }
-        }
-        __syncthreads();
-        // vertical sums of the partials -> dL/dx on the tile: columns kLTW, rows in runs of 4
-        float *gs = a.grad + (size_t)a.nch * vw.pixel_offset + ch * HW;
-        {
-            constexpr int RUN = 4, SEGS = kLTH / RUN;
-            for (int it = threadIdx.x; it < SEGS * kLTW; it += kLossThreads) {
-                const int seg = it / kLTW, c = it - seg * kLTW;
-                const int r0 = seg * RUN;
-                float cv[3][RUN];
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    float col[RUN + 10];
+                for (int i = 0; i < RUN + 10; ++i) {
+                    const float2 q = PQ[r * kMP + c0 + i];
+                    const F2 pq = f2(q.x, q.y);
+                    const float rr = Rp[r * kMP + c0 + i];
 #pragma unroll
-                    for (int i = 0; i < RUN + 10; ++i) col[i] = Hp[k * kMH * kMP + (r0 + i) * kMP + c];
-#pragma unroll
-                    for (int o = 0; o < RUN; ++o) {
-                        float acc = 0.f;
-#pragma unroll
-                        for (int j = 0; j < 11; ++j) acc = fmaf(wr[j], col[o + j], acc);
-                        cv[k][o] = acc;
-                    }
+                    for (int o = 0; o < RUN; ++o)
+                        if (i - o >= 0 && i - o < 11) {
+                            s[o] = fma2(wr[i - o], pq, s[o]);
+                            t[o] = fmaf(w1(i - o), rr, t[o]);
+                        }
                 }
 #pragma unroll
                 for (int o = 0; o < RUN; ++o) {
-                    const int r = r0 + o;
-                    const int gy = by * kLTH + r, gx = bx * kLTW + c;
-                    if (gx >= W || gy >= H) continue;
-                    const size_t gp = (size_t)gy * W + gx;
-                    const float xv = xs[gp], yv = ys[gp];  // the staged planes now hold partials
-                    if (ch == 0 && a.counts) {
-                        n_depth += a.gt_depth[(size_t)vw.pixel_offset + gp] > 0.f;
-                        if (a.label) n_label += a.label[(size_t)vw.pixel_offset + gp] >= 0;
-                    }
-                    const float d = xv - yv;
-                    l1_sum += fabsf(d);
-                    const float sg = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
-                    gs[(size_t)gy * W + gx] = l1c * sg + cv[0][o] + 2.f * xv * cv[1][o] + yv * cv[2][o];
+                    HPQ[r * kHP + c0 + o] = unpack(s[o]);
+                    HR[r * kHP + c0 + o] = t[o];
                 }
+            }
+        }
+        __syncthreads();
+        // vertical sums of the partials -> dL/dx on the tile: a column and 4 rows per thread
+        float *gs = pl.grad + (size_t)nch * vw.pixel_offset + ch * HW;
+        {
+            constexpr int RUN = 4;
+            const int c = lane, r0 = warp * RUN;
+            const int gx = bx * kLTW + c;
+            float xv[RUN], yv[RUN];  // (the staged planes now hold partials)
+#pragma unroll
+            for (int o = 0; o < RUN; ++o) {
+                const int gy = by * kLTH + r0 + o;
+                const bool in = gx < W && gy < H;
+                const size_t gp = (size_t)gy * W + gx;
+                xv[o] = in ? xs[gp] : 0.f;
+                yv[o] = in ? ys[gp] : 0.f;
+            }
+            F2 s[RUN];
+            float t[RUN];
+#pragma unroll
+            for (int o = 0; o < RUN; ++o) {
+                s[o] = f2(0.f, 0.f);
+                t[o] = 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < RUN + 10; ++i) {
+                const float2 q = HPQ[(r0 + i) * kHP + c];
+                const F2 pq = f2(q.x, q.y);
+                const float rr = HR[(r0 + i) * kHP + c];
+#pragma unroll
+                for (int o = 0; o < RUN; ++o)
+                    if (i - o >= 0 && i - o < 11) {
+                        s[o] = fma2(wr[i - o], pq, s[o]);
+                        t[o] = fmaf(w1(i - o), rr, t[o]);
+                    }
+            }
+#pragma unroll
+            for (int o = 0; o < RUN; ++o) {
+                const int gy = by * kLTH + r0 + o;
+                if (gx >= W || gy >= H) continue;
+                const float2 pq = unpack(s[o]);
+                const float d = xv[o] - yv[o];
+                l1_sum += fabsf(d);
+                const float sg = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
+                gs[(size_t)gy * W + gx] = l1c * sg + pq.x + 2.f * xv[o] * pq.y + yv[o] * t[o];
             }
         }
         __syncthreads();
     }
-    if (a.counts) {
+    if (group == 0) {  // the tile's valid pixels
+        int n_depth = 0, n_label = 0;
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            const int gx = bx * kLTW + lane, gy = by * kLTH + 4 * warp + o;
+            if (gx >= W || gy >= H) continue;
+            const size_t gp = (size_t)vw.pixel_offset + (size_t)gy * W + gx;
+            n_depth += a.gt_depth[gp] > 0.f;
+            if (a.label) n_label += a.label[gp] >= 0;
+        }
         n_depth = __reduce_add_sync(SG_FULL_MASK, n_depth);
         n_label = __reduce_add_sync(SG_FULL_MASK, n_label);
-        if ((threadIdx.x & 31) == 0) {
+        if (lane == 0) {
             atomicAdd(&s_cnt[0], n_depth);
             atomicAdd(&s_cnt[1], n_label);
         }
@@ -280,11 +357,10 @@ __global__ void __launch_bounds__(kLossThreads, 3) ssim_l1_kernel(SsimArgs a) {
     const float t1 = block_sum(l1_sum, s_red);  // (its barriers also order the counts above)
     const float t2 = block_sum(ssim_sum, s_red);
     if (threadIdx.x == 0) {
-        a.partials[2 * item] = t1;
-        a.partials[2 * item + 1] = t2;
+        a.partials[(size_t)group * gridDim.x + item] = (1.f - pl.lambda) * t1 - pl.lambda * t2;
         // integer atomics: the totals do not depend on the order
-        if (a.counts && s_cnt[0]) atomicAdd(a.counts + 2 * v, s_cnt[0]);
-        if (a.counts && s_cnt[1]) atomicAdd(a.counts + 2 * v + 1, s_cnt[1]);
+        if (group == 0 && s_cnt[0]) atomicAdd(a.counts + 2 * v, s_cnt[0]);
+        if (group == 0 && s_cnt[1]) atomicAdd(a.counts + 2 * v + 1, s_cnt[1]);
     }
 }
 
@@ -817,7 +893,8 @@ static int launch_ce_mma(PixelArgs &pa, int blocks, cudaStream_t st) {
 }
 
 struct FinalArgs {
-    const float *ssim_rgb, *ssim_sem, *pix;  // partial arrays
+    const float *ssim, *pix;  // partial arrays
+    int rgb_groups, sem_groups, n_tiles;
     const int *counts;
     const sg_view *views;
     LossViews lv;
@@ -846,15 +923,11 @@ __global__ void loss_finalize_kernel(FinalArgs a) {
     const sg_view &vw = a.views[v];
     const double HW = (double)vw.W * vw.H;
     __shared__ double s_w[kLossThreads / 32];
-    double acc[4] = {0, 0, 0, 0};
-    for (int i = a.lv.tile_off[v] + threadIdx.x; i < a.lv.tile_off[v + 1]; i += kLossThreads) {
-        acc[0] += a.ssim_rgb[2 * i];
-        acc[1] += a.ssim_rgb[2 * i + 1];
-        if (a.ssim_sem) {
-            acc[2] += a.ssim_sem[2 * i];
-            acc[3] += a.ssim_sem[2 * i + 1];
-        }
-    }
+    double acc[2] = {0, 0};  // colour, semantics
+    for (int i = a.lv.tile_off[v] + threadIdx.x; i < a.lv.tile_off[v + 1]; i += kLossThreads)
+#pragma unroll
+        for (int g = 0; g < kSsimGroups; ++g)
+            if (g < a.rgb_groups + a.sem_groups) acc[g >= a.rgb_groups] += a.ssim[(size_t)g * a.n_tiles + i];
     // the per-unit (depth L1, CE) sums: two units per 16-byte load, four loads in flight per
     // thread, summed in a fixed order (a latency-bound chain of dependent adds otherwise)
     double b[2] = {0, 0};
@@ -881,22 +954,23 @@ __global__ void loss_finalize_kernel(FinalArgs a) {
         b[0] = (c[0][0] + c[1][0]) + (c[2][0] + c[3][0]);
         b[1] = (c[0][1] + c[1][1]) + (c[2][1] + c[3][1]);
     }
-    double r[4];
-    for (int k = 0; k < 4; ++k) r[k] = block_sum_d(acc[k], s_w);
+    const double r_rgb = block_sum_d(acc[0], s_w);
+    const double r_sem = block_sum_d(acc[1], s_w);
     const double l1d_sum = block_sum_d(b[0], s_w);
     const double ce_sum = block_sum_d(b[1], s_w);
     if (threadIdx.x == 0) {
         const double l1d = l1d_sum, ce = ce_sum;
         const int nd = a.counts[2 * v], nl = a.counts[2 * v + 1];
         const double n_rgb = 3.0 * HW;
-        const double L_r = (1.0 - a.lambda_r) * r[0] / n_rgb + a.lambda_r * (1.0 - r[1] / n_rgb);
+        // (1 - lambda) L1 + lambda (1 - SSIM)
+        const double L_r = r_rgb / n_rgb + a.lambda_r;
         const double L_d = nd > 0 ? a.w_depth * l1d / nd : 0.0;
         double L_s;
         if (a.sem_mode == 0) {
             L_s = nl > 0 ? a.w_sem * ce / nl : 0.0;
         } else {
             const double n_s = (double)a.C * HW;
-            L_s = a.w_sem * ((1.0 - a.lambda_s) * r[2] / n_s + a.lambda_s * (1.0 - r[3] / n_s));
+            L_s = a.w_sem * (r_sem / n_s + a.lambda_s);
         }
         a.terms[4 * v + 0] = (float)L_r;
         a.terms[4 * v + 1] = (float)L_d;
@@ -908,7 +982,7 @@ __global__ void loss_finalize_kernel(FinalArgs a) {
 
 // ---------------------------------------------------------------------------------------
 
-static size_t ssim_smem() { return sizeof(float) * (2 * kXH * kXP + 5 * kXH * kMP); }
+static size_t ssim_smem() { return sizeof(float) * (2 * kXH * kXP + 4 * kXH * kMP); }
 
 static void make_loss_views(const sg_view *vh, int n_views, LossViews &lv) {
     lv.n = n_views;
@@ -923,7 +997,7 @@ static void make_loss_views(const sg_view *vh, int n_views, LossViews &lv) {
 
 static size_t loss_ws_bytes(int n_views, int n_tiles, int n_blocks, int KC) {
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    return al(sizeof(int) * 2 * n_views) + 2 * al(sizeof(float) * 2 * n_tiles) +
+    return al(sizeof(int) * 2 * n_views) + 2 * al(sizeof(float) * (kSsimGroups / 2) * n_tiles) +
            al(sizeof(float) * 2 * kPixSlots * n_blocks) + al(sizeof(float) * (size_t)n_blocks * KC) +
            al(sizeof(float) * (size_t)kDecChunks * KC);
 }
@@ -986,8 +1060,8 @@ sg_status launch_loss(const sg_images *r, const sg_targets *gt, const sg_view *v
     size_t off = 0;
     auto take = [&](size_t bytes) { char *p = base + off; off += (bytes + 255) & ~(size_t)255; return p; };
     int *counts = (int *)take(sizeof(int) * 2 * n_views);
-    float *p_rgb = (float *)take(sizeof(float) * 2 * n_tiles);
-    float *p_sem = (float *)take(sizeof(float) * 2 * n_tiles);
+    float *p_ssim = (float *)take(sizeof(float) * (kSsimGroups / 2) * n_tiles);
+    take(sizeof(float) * (kSsimGroups / 2) * n_tiles);  // (its second half)
     float *p_pix = (float *)take(sizeof(float) * 2 * kPixSlots * n_blocks);
     const int ce = lc->sem_mode == 0;
     const int K = ce ? lc->n_classes : C;
@@ -1005,14 +1079,14 @@ sg_status launch_loss(const sg_images *r, const sg_targets *gt, const sg_view *v
         cudaFuncSetAttribute(ssim_l1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssim_smem());
         attr = true;
     }
-    SsimArgs sa{r->rgb, gt->rgb, dL->rgb, 3, 1.f - lc->lambda_r, lc->lambda_r, views, lv, p_rgb,
-                gt->depth, ce ? gt->label : nullptr, counts};
-    launch_pdl(ssim_l1_kernel, n_tiles, kLossThreads, ssim_smem(), st, sa);
-    if (!ce) {
-        SsimArgs ss{r->sem, gt->sem, dL->sem, C, lc->w_sem * (1.f - lc->lambda_s), lc->w_sem * lc->lambda_s,
-                    views, lv, p_sem, nullptr, nullptr, nullptr};
-        launch_pdl(ssim_l1_kernel, n_tiles, kLossThreads, ssim_smem(), st, ss);
-    }
+    // cross-entropy: a group per colour plane; otherwise one for the colour planes and three for
+    // the semantic ones
+    const int rgb_groups = ce ? 3 : 1, sem_groups = ce ? 0 : std::min(C, kSsimGroups - rgb_groups);
+    const SsimArgs sa{{r->rgb, gt->rgb, dL->rgb, 3, 1.f - lc->lambda_r, lc->lambda_r, lc->lambda_r},
+                      {r->sem, gt->sem, dL->sem, C, lc->w_sem * (1.f - lc->lambda_s), lc->w_sem * lc->lambda_s,
+                       lc->lambda_s},
+                      rgb_groups, sem_groups, views, lv, p_ssim, gt->depth, ce ? gt->label : nullptr, counts};
+    launch_pdl(ssim_l1_kernel, dim3(n_tiles, rgb_groups + sem_groups), kLossThreads, ssim_smem(), st, sa);
     PixelArgs pa{r->depth, gt->depth, r->sem, gt->label, dL->depth, dL->sem, lc->decoder,
                  KC ? lc->decoder_grad : nullptr, C, K, ce, lc->w_depth, lc->w_sem, counts, views, lv, p_pix, p_dec};
     const int dec_rows = launch_pixel(pa, n_blocks, st);
@@ -1025,10 +1099,10 @@ sg_status launch_loss(const sg_images *r, const sg_targets *gt, const sg_view *v
         launch_pdl(decoder_reduce2_kernel, (KC + 127) / 128, 128, 0, st, p_dec2, KC, lc->decoder_grad);
         count_launches(2);
     }
-    FinalArgs fa{p_rgb, ce ? nullptr : p_sem, p_pix, counts, views, lv, C, lc->sem_mode,
+    FinalArgs fa{p_ssim, p_pix, rgb_groups, sem_groups, n_tiles, counts, views, lv, C, lc->sem_mode,
                  lc->lambda_r, lc->lambda_s, lc->w_depth, lc->w_sem, terms, status};
     launch_pdl(loss_finalize_kernel, n_views, kLossThreads, 0, st, fa);
-    count_launches(ce ? 3 : 4);
+    count_launches(3);
     return check_launch("pyramid_loss");
 }
 
