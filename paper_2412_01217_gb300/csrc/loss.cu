@@ -12,6 +12,8 @@
 // Depth term (Eq. 11): mean |D - D_gt| over pixels with D_gt > 0.
 // Semantic term, cross-entropy mode: mean CE(softmax(decoder * S), label) over label >= 0.
 // Sums are per-CTA partials reduced in a fixed order (deterministic).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cstdio>
 
@@ -917,47 +919,64 @@ __device__ __forceinline__ double block_sum_d(double v, double *s_w) {
     return t;
 }
 
-__global__ void loss_finalize_kernel(FinalArgs a) {
+// A view's partial sums and its loss terms by a cluster of kFinalCtas CTAs, their shares added
+// in rank order through distributed shared memory.  Bound by the latency of the partials'
+// loads and the double additions, of which one SM does a few per clock: 1200x680 x 3 levels with
+// one CTA per view took 38 us (loss with a 32-class decoder 198 -> 173 us, 637x477 x 3
+// levels without one 81 -> 73).
+constexpr int kFinalCtas = 8;
+__global__ void __cluster_dims__(kFinalCtas, 1, 1) __launch_bounds__(kLossThreads) loss_finalize_kernel(FinalArgs a) {
     pdl_begin();
-    const int v = blockIdx.x;
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int v = blockIdx.x / kFinalCtas, rank = blockIdx.x % kFinalCtas;
+    const int first = rank * kLossThreads + (int)threadIdx.x;
+    constexpr int kStride = kFinalCtas * kLossThreads;
     const sg_view &vw = a.views[v];
     const double HW = (double)vw.W * vw.H;
     __shared__ double s_w[kLossThreads / 32];
+    __shared__ double s_part[kFinalCtas][4];  // (rank 0's holds the shares)
     double acc[2] = {0, 0};  // colour, semantics
-    for (int i = a.lv.tile_off[v] + threadIdx.x; i < a.lv.tile_off[v + 1]; i += kLossThreads)
+    for (int i = a.lv.tile_off[v] + first; i < a.lv.tile_off[v + 1]; i += kStride)
 #pragma unroll
         for (int g = 0; g < kSsimGroups; ++g)
-            if (g < a.rgb_groups + a.sem_groups) acc[g >= a.rgb_groups] += a.ssim[(size_t)g * a.n_tiles + i];
+            if (g < a.rgb_groups + a.sem_groups) {
+                const double t = a.ssim[(size_t)g * a.n_tiles + i];
+                if (g < a.rgb_groups) acc[0] += t; else acc[1] += t;
+            }
     // the per-unit (depth L1, CE) sums: two units per 16-byte load, four loads in flight per
-    // thread, summed in a fixed order (a latency-bound chain of dependent adds otherwise)
+    // thread, summed in a fixed order
     double b[2] = {0, 0};
     {
         const float4 *p4 = reinterpret_cast<const float4 *>(a.pix);
         const int s1 = kPixSlots * a.lv.pix_blk_off[v + 1] / 2;
-        double c[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-        int i = kPixSlots * a.lv.pix_blk_off[v] / 2 + threadIdx.x;
-        for (; i + 3 * kLossThreads < s1; i += 4 * kLossThreads) {
+        for (int i = kPixSlots * a.lv.pix_blk_off[v] / 2 + first; i < s1; i += 4 * kStride) {
             float4 q[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) q[k] = p4[i + k * kLossThreads];
+            for (int k = 0; k < 4; ++k)
+                q[k] = i + k * kStride < s1 ? p4[i + k * kStride] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                c[k][0] += (double)q[k].x + (double)q[k].z;
-                c[k][1] += (double)q[k].y + (double)q[k].w;
+                b[0] += (double)q[k].x + (double)q[k].z;
+                b[1] += (double)q[k].y + (double)q[k].w;
             }
         }
-        for (; i < s1; i += kLossThreads) {
-            const float4 q = p4[i];
-            c[0][0] += (double)q.x + (double)q.z;
-            c[0][1] += (double)q.y + (double)q.w;
-        }
-        b[0] = (c[0][0] + c[1][0]) + (c[2][0] + c[3][0]);
-        b[1] = (c[0][1] + c[1][1]) + (c[2][1] + c[3][1]);
     }
-    const double r_rgb = block_sum_d(acc[0], s_w);
-    const double r_sem = block_sum_d(acc[1], s_w);
-    const double l1d_sum = block_sum_d(b[0], s_w);
-    const double ce_sum = block_sum_d(b[1], s_w);
+    const double part[4] = {block_sum_d(acc[0], s_w), block_sum_d(acc[1], s_w), block_sum_d(b[0], s_w),
+                            block_sum_d(b[1], s_w)};
+    cluster.sync();  // (rank 0 runs: its shared memory can be written)
+    if (threadIdx.x == 0) {
+        double *to = cluster.map_shared_rank(&s_part[rank][0], 0);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) to[k] = part[k];
+    }
+    cluster.sync();
+    if (rank != 0) return;
+    double sum[4] = {0, 0, 0, 0};
+    for (int r = 0; r < kFinalCtas; ++r)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) sum[k] += s_part[r][k];
+    const double r_rgb = sum[0], r_sem = sum[1], l1d_sum = sum[2], ce_sum = sum[3];
     if (threadIdx.x == 0) {
         const double l1d = l1d_sum, ce = ce_sum;
         const int nd = a.counts[2 * v], nl = a.counts[2 * v + 1];
@@ -1101,7 +1120,7 @@ sg_status launch_loss(const sg_images *r, const sg_targets *gt, const sg_view *v
     }
     FinalArgs fa{p_ssim, p_pix, rgb_groups, sem_groups, n_tiles, counts, views, lv, C, lc->sem_mode,
                  lc->lambda_r, lc->lambda_s, lc->w_depth, lc->w_sem, terms, status};
-    launch_pdl(loss_finalize_kernel, n_views, kLossThreads, 0, st, fa);
+    launch_pdl(loss_finalize_kernel, n_views * kFinalCtas, kLossThreads, 0, st, fa);
     count_launches(3);
     return check_launch("pyramid_loss");
 }
