@@ -25,7 +25,7 @@ from .splat import PyramidRasterizer, RenderConfig
 TILES = ((16, 16), (8, 8), (32, 8), (16, 8))
 BATCHES = (16, 32, 64, 128, 256)
 PPT_FWD = (1, 2)
-PPT_BWD = (1, 2, 4)
+PPT_BWD = (1,)  # (what the adjoint runs)
 CACHE = os.path.join(os.path.expanduser("~"), ".cache", "pyramid_splat_gb300_autotune.json")
 
 

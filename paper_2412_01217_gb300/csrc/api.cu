@@ -404,7 +404,6 @@ sg_status sg_render_pyramid_backward_raster(const sg_gaussians *g, const sg_proj
     // with sem_sh, per-record semantic gradients in the workspace's semantic block
     a.g_sem = sh_semantic(g) ? g2d + 12 * R : grads->sem;
     a.sem_v2 = ((uintptr_t)a.g_sem % 8) == 0 && (g->C % 2) == 0;
-    a.ppt = cfg->pixels_per_thread_bwd;
     if (cfg->batch_bwd) a.batch = cfg->batch_bwd;
     return launch_raster(a, g->C, true, st);
 }

@@ -23,9 +23,9 @@ struct RasterArgs {
     int tile_w, tile_h, batch;
     int *work_counter;
     int persistent;
-    int ppt;  // pixels per thread (1, 2 or 4)
+    int ppt;  // forward: pixels per thread (1, 2 or 4)
     int half;             // records carry half masks in bits 30-31: the adjoint of 8 x 8
-                          // tiles at one pixel per thread runs one warp per half tile
+                          // tiles runs one warp per half tile
     int half_fwd;         // ... and so does the forward (sg_config.half_tile_fwd)
     int half_pairs;       // half-tile adjoint: a work item is a whole tile, both halves in turn
     uint32_t rec_mask;    // bits of a list word that hold the record id

@@ -1,6 +1,6 @@
 // raster_impl.cuh -- tile compositing of RGB, depth and C semantic channels (Eq. 7-9) and its
-// adjoint (Sec. III-D backpropagation), templated on the semantic width C and on the
-// number of pixels each thread owns (PPT = 1, 2 or 4).
+// adjoint (Sec. III-D backpropagation), templated on the semantic width C and, in the
+// forward, on the number of pixels each thread owns (PPT = 1, 2 or 4; the adjoint has one).
 //
 // One CTA owns one screen tile of one view-level.  Every view-level of every keyframe is
 // addressed through one global tile id, so a single launch renders the whole pyramid of
@@ -8,7 +8,7 @@
 // atomic work counter.  Each warp owns an 8 x (4 PPT) pixel sub-tile: lane l has the PPT
 // pixels (l mod 8, l div 8 + 4k), k < PPT.  A whole warp skips a Gaussian whose footprint
 // misses its sub-tile (one uniform test), and with PPT > 1 every per-Gaussian cost
-// (shared-memory loads, the per-chunk contractions of the backward) is shared by PPT pixels.
+// (shared-memory loads) is shared by PPT pixels.
 //
 // Forward: the tile's depth-sorted list is walked in batches the CTA stages into shared
 // memory; each pixel composites front to back and stops when T would fall below T_min;
@@ -576,8 +576,7 @@ __global__ void __launch_bounds__(kMaxTileThreads) __maxnreg__((fwd_max_regs<C, 
 // The 2D-mean, conic and opacity gradients are linear in the moments (see moment_grads).
 constexpr int kHalfQueue = kChunk + 32;  // entries pending (< 16 + one 32-entry scan)
 
-template <int NPX>
-__host__ __device__ constexpr int chunk_pitch() { return NPX + 4; }  // 4 mod 32: conflict-free fragments
+constexpr int kChunkPitch = 32 + 4;  // 4 mod 32: conflict-free fragments
 
 template <int NF>
 __host__ __device__ constexpr int padded_features() { return (NF + 7) / 8 * 8; }
@@ -588,18 +587,22 @@ __host__ __device__ constexpr int padded_features() { return (NF + 7) / 8 * 8; }
 template <int NF>
 __host__ __device__ constexpr int g_pitch() { return (NF / 4) % 2 == 1 ? NF : NF + 4; }
 
+// The adjoint gives every thread one pixel, whatever the forward's number.  With two or four, the
+// per-chunk costs are shared by more pixels, but half or a quarter of the warps are left, each
+// with a longer serial recurrence, and shared memory holds fewer of them: at 16 x 16, 32 x 8,
+// 16 x 8 and 8 x 8 tiles, C = 4 to 40 and 100 to 4270 tiles a whole iteration took 0 to 12 %
+// longer with two (320x180 x 3 levels, C = 16: 293 against 261 us; 640x480 x 2 levels with 1M
+// Gaussians, C = 40: 1647 against 1474) and up to 58 % with four.
+//
 // shared memory of one warp (4-byte words): the chunk's rows and the queue (with records in
-// half mode), their list positions, G (NPX x g_pitch), two chunk buffers (16 x chunk_pitch) and
-// the chunk's alphas; a multiple of 16 bytes.  At one pixel per thread the second chunk buffer
-// reuses the alphas' (read into registers first): 20 instead of 17 one-warp CTAs per SM in half
-// mode (batched workload 2072 -> 2009 us); with more pixels the registers cost more than that.
-template <int PPT>
-__host__ __device__ constexpr bool bwd_overlay() { return PPT == 1; }
-template <int C, int PPT, bool HALF>
+// half mode), their list positions, G (32 x g_pitch), the first chunk buffer (16 x kChunkPitch)
+// and the chunk's alphas; a multiple of 16 bytes.  The second chunk buffer reuses the alphas'
+// (read into registers first): 20 instead of 17 one-warp CTAs per SM in half mode (batched
+// workload 2072 -> 2009 us).
+template <int C, bool HALF>
 __host__ __device__ constexpr int bwd_warp_words() {
-    static_assert(kChunk * chunk_pitch<32 * PPT>() <= 32 * PPT * kAPitch, "the second chunk buffer reuses the alphas'");
-    return 2 * kChunk + (HALF ? 2 : 1) * kHalfQueue + 32 * PPT * g_pitch<4 + C>() +
-           (bwd_overlay<PPT>() ? 1 : 2) * kChunk * chunk_pitch<32 * PPT>() + 32 * PPT * kAPitch;
+    static_assert(kChunk * kChunkPitch <= 32 * kAPitch, "the second chunk buffer reuses the alphas'");
+    return 2 * kChunk + (HALF ? 2 : 1) * kHalfQueue + 32 * g_pitch<4 + C>() + kChunk * kChunkPitch + 32 * kAPitch;
 }
 
 // Gradients of the 2D mean (u, v), the conic (a, b, c) and the opacity from the moments
@@ -628,29 +631,28 @@ __device__ __forceinline__ void moment_grads(const float (&M)[6], float U, float
     }
 }
 
-template <int C, int PPT>
-__host__ __device__ constexpr int bwd_max_regs() { return PPT == 1 ? (C <= 16 ? 96 : 128) : 255; }
+template <int C>
+__host__ __device__ constexpr int bwd_max_regs() { return C <= 16 ? 96 : 128; }
 
-template <int C, int PPT, bool HALF = false>
-__global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterArgs a) {
+template <int C, bool HALF>
+__global__ void __maxnreg__((bwd_max_regs<C>())) raster_bwd_kernel(RasterArgs a) {
     pdl_begin();
     constexpr int NF = 4 + C;                     // rgb(3) depth | sem(C)
     constexpr int NFP = padded_features<NF>();    // features padded to 8
     constexpr int NT = NFP / 8;                   // 8-feature tiles
-    constexpr int NPX = 32 * PPT;                 // pixels of one warp (pixel q = 32 k + lane)
+    constexpr int NPX = 32;                       // pixels of one warp (pixel = lane)
     constexpr int KS = NPX / 8;                   // 8-pixel steps
-    constexpr int WQ = chunk_pitch<NPX>();
+    constexpr int WQ = kChunkPitch;
     constexpr int GP = g_pitch<NF>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_item, s_max_last;
-    // Half mode (8 x 8 tiles, one pixel per thread, half masks given): a CTA is one warp that
+    // Half mode (8 x 8 tiles, half masks given): a CTA is one warp that
     // works on one half (8 x 4 pixels) of a tile at a time; it walks the tile's list back to
     // front, keeps the entries whose half mask holds its half in a queue, and stages and
     // processes them 16 at a time, so its chunks hold only its own entries; no block barrier.
     // Otherwise the CTA's warps share each batch of the list, staged between two block
     // barriers.
     constexpr bool hm = HALF;
-    static_assert(!HALF || PPT == 1, "half mode runs one pixel per thread");
     const int batch = hm ? kChunk : a.batch;
     float4 *s_geo0 = reinterpret_cast<float4 *>(smem_raw);
     float4 *s_geo1 = s_geo0 + batch;
@@ -661,23 +663,22 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
     uint32_t *s_rec = reinterpret_cast<uint32_t *>(s_feat + (size_t)batch * NF);
     // per warp: the staged row of each chunk row (shared batches), its list position, and the
     // queue of pending entries: (list position, record), or staged rows
-    const int nthreads = hm ? 32 : a.tile_w * a.tile_h / PPT;
+    const int nthreads = hm ? 32 : a.tile_w * a.tile_h;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int *s_pos = reinterpret_cast<int *>(s_rec + batch) + (size_t)warp * bwd_warp_words<C, PPT, HALF>();
+    int *s_pos = reinterpret_cast<int *>(s_rec + batch) + (size_t)warp * bwd_warp_words<C, HALF>();
     int *s_lp = s_pos + kChunk;  // list position of each chunk row (the largest int past its end)
     int *s_q = s_lp + kChunk;
     uint32_t *s_qr = reinterpret_cast<uint32_t *>(s_q + kHalfQueue);
     float *s_G = reinterpret_cast<float *>(s_qr + (hm ? kHalfQueue : 0));
     float *s_gw = s_G + NPX * GP;     // per chunk row: gf, then overwritten with w = alpha T
     float *s_A = s_gw + kChunk * WQ;  // alphas (chunk_alphas)
-    constexpr bool OVER = bwd_overlay<PPT>();
-    float *s_sg = OVER ? s_A : s_A + 32 * PPT * kAPitch;  // per chunk row: s = dL/dsigma
+    float *s_sg = s_A;                // per chunk row: s = dL/dsigma
     const int gid = lane >> 2, tig = lane & 3;
-    const WarpTile<PPT> wt(a.tile_w);
+    const WarpTile<1> wt(a.tile_w);
     const float ax = (float)(wt.lx - (lane & 7) + 4 * (lane >> 4)), ay = (float)(wt.ly - (lane >> 3));
     const float ln_amin = __logf(a.alpha_min);
     // moment polynomials at the B-fragment pixels: pixel 8 ks + tig (+ 4) has X = tig - 3.5
-    // (tig + 0.5), Y = (ks % 4) + 4 (ks / 4) - (2 PPT - 0.5); P_gid = P0 + Y (P1 + Y P2)
+    // (tig + 0.5), Y = ks - 1.5; P_gid = P0 + Y (P1 + Y P2)
     // (all values small multiples of 1/4: exact in TF32, so B needs no split)
     const float X0 = tig - 3.5f, X1 = tig + 0.5f;
     const float P0a = gid == 0 ? 1.f : gid == 1 ? X0 : gid == 3 ? X0 * X0 : 0.f;
@@ -706,19 +707,15 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
         const size_t HW = (size_t)vw.W * vw.H;
         const size_t p0 = (size_t)vw.pixel_offset;
         const uint32_t rec_base = (uint32_t)ti.v * (uint32_t)a.N;
-        float T[PPT], acc_a[PPT];
-        int my_last[PPT];
-        int thread_last = 0;
-#pragma unroll
-        for (int k = 0; k < PPT; ++k) {
-            const int py = ti.py0 + wt.ly + 4 * k;
+        float T = 1.f, acc_a;
+        int my_last = 0;
+        {
+            const int py = ti.py0 + wt.ly;
             const bool inside = px < vw.W && py < vw.H;
             const size_t p = (size_t)py * vw.W + px;
             float g[NFP];
 #pragma unroll
             for (int f = 0; f < NFP; ++f) g[f] = 0.f;
-            T[k] = 1.f;
-            my_last[k] = 0;
             if (inside) {
                 g[0] = a.dL_rgb[3 * p0 + p];
                 g[1] = a.dL_rgb[3 * p0 + HW + p];
@@ -726,22 +723,21 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
                 g[3] = a.dL_depth[p0 + p];
 #pragma unroll
                 for (int c = 0; c < C; ++c) g[4 + c] = a.dL_sem[(size_t)C * p0 + c * HW + p];
-                T[k] = a.T_final[p0 + p];
-                my_last[k] = a.last[p0 + p];
+                T = a.T_final[p0 + p];
+                my_last = a.last[p0 + p];
             }
-            acc_a[k] = g[0] * a.bg0 + g[1] * a.bg1 + g[2] * a.bg2;
-            thread_last = max(thread_last, my_last[k]);
-            float4 *row = reinterpret_cast<float4 *>(s_G + (32 * k + lane) * GP);
+            acc_a = g[0] * a.bg0 + g[1] * a.bg1 + g[2] * a.bg2;
+            float4 *row = reinterpret_cast<float4 *>(s_G + lane * GP);
 #pragma unroll
             for (int f = 0; f < NF; f += 4) row[f / 4] = make_float4(g[f], g[f + 1], g[f + 2], g[f + 3]);
         }
-        const int warp_last = __reduce_max_sync(SG_FULL_MASK, thread_last);
+        const int warp_last = __reduce_max_sync(SG_FULL_MASK, my_last);
         __syncwarp();
         // One chunk of c <= 16 list entries, back to front: chunk row r (ascending list position)
         // is staged row row_of(r) at list position s_lp[r] (>= warp_last for r >= c), and lane l
         // holds the geometry g of row l % 16 (rows >= c: opacity 0).
         auto chunk = [&](const int c, const EntryGeo &g, auto row_of) {
-                chunk_alphas<PPT>(g, ax, ay, a.alpha_max, a.alpha_min, s_A);
+                chunk_alphas<1>(g, ax, ay, a.alpha_max, a.alpha_min, s_A);
                 // ---- gf = F G^T for the chunk (M = entries, N = pixels, K = features) ----
                 // ldmatrix row addresses: lanes 0-15 rows 0-15 of the first four columns, lanes
                 // 16-31 the same rows four columns further (A); lanes 8 m + i row i of matrix m (B)
@@ -796,53 +792,35 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
                 }
                 __syncwarp();
                 // ---- back to front: the recurrence in T and a ----
-                uint32_t hits = 0;  // rows that contribute to one of the lane's pixels
-                auto recur = [&](const int rg, const float (&al)[PPT][4]) {  // rows rg .. rg + 3
-                    const int4 lp = *reinterpret_cast<const int4 *>(s_lp + rg);
+                uint32_t hits = 0;  // rows that contribute to the lane's pixel
+                float4 al[kChunk / 4];
+#pragma unroll
+                for (int q = 0; q < kChunk / 4; ++q)
+                    al[q] = *reinterpret_cast<const float4 *>(s_A + lane * kAPitch + 4 * q);
+                __syncwarp();  // (s_sg reuses s_A)
+#pragma unroll
+                for (int q = kChunk / 4 - 1; q >= 0; --q) {  // rows 4 q .. 4 q + 3
+                    if (4 * q >= c) continue;  // (warp-uniform)
+                    const int4 lp = *reinterpret_cast<const int4 *>(s_lp + 4 * q);
                     const int pos[4] = {lp.x, lp.y, lp.z, lp.w};
+                    const float a4[4] = {al[q].x, al[q].y, al[q].z, al[q].w};
                     uint32_t hb = 0;
 #pragma unroll
                     for (int i = 3; i >= 0; --i) {
-                        float *gw = s_gw + (rg + i) * WQ + lane;
-#pragma unroll
-                        for (int k = 0; k < PPT; ++k) {
-                            const float A = pos[i] < my_last[k] ? al[k][i] : 0.f, om = 1.f - A;
-                            // (a pixel without a contribution keeps T and a: A = 0, gf taken as 0)
-                            const float gf = A > 0.f ? gw[32 * k] : 0.f;
-                            if (A > 0.f) hb |= 1u << i;
-                            // transmittance before this Gaussian (only gradients depend on it)
-                            T[k] *= rcp_fast(om);
-                            const float dalpha = T[k] * (gf - acc_a[k]);
-                            acc_a[k] = fmaf(om, acc_a[k], A * gf);
-                            gw[32 * k] = A * T[k];
-                            // (alpha = alpha_max: clamped, no gradient; else alpha = o G)
-                            s_sg[(rg + i) * WQ + 32 * k + lane] = A < a.alpha_max ? -dalpha * A : 0.f;
-                        }
+                        float *gw = s_gw + (4 * q + i) * WQ + lane;
+                        const float A = pos[i] < my_last ? a4[i] : 0.f, om = 1.f - A;
+                        // (a pixel without a contribution keeps T and a: A = 0, gf taken as 0)
+                        const float gf = A > 0.f ? *gw : 0.f;
+                        if (A > 0.f) hb |= 1u << i;
+                        // transmittance before this Gaussian (only gradients depend on it)
+                        T *= rcp_fast(om);
+                        const float dalpha = T * (gf - acc_a);
+                        acc_a = fmaf(om, acc_a, A * gf);
+                        *gw = A * T;
+                        // (alpha = alpha_max: clamped, no gradient; else alpha = o G)
+                        s_sg[(4 * q + i) * WQ + lane] = A < a.alpha_max ? -dalpha * A : 0.f;
                     }
-                    hits |= hb << rg;
-                };
-                auto alphas = [&](int rg, float (&al)[PPT][4]) {
-#pragma unroll
-                    for (int k = 0; k < PPT; ++k) {
-                        const float4 t = *reinterpret_cast<const float4 *>(s_A + (32 * k + lane) * kAPitch + rg);
-                        al[k][0] = t.x; al[k][1] = t.y; al[k][2] = t.z; al[k][3] = t.w;
-                    }
-                };
-                if constexpr (OVER) {
-                    float al[kChunk / 4][PPT][4];
-#pragma unroll
-                    for (int q = 0; q < kChunk / 4; ++q) alphas(4 * q, al[q]);
-                    __syncwarp();  // (s_sg reuses s_A)
-#pragma unroll
-                    for (int q = kChunk / 4 - 1; q >= 0; --q)
-                        if (4 * q < c) recur(4 * q, al[q]);  // (warp-uniform)
-                } else {
-#pragma unroll 1
-                    for (int rg = (c - 1) & ~3; rg >= 0; rg -= 4) {
-                        float al[PPT][4];
-                        alphas(rg, al);
-                        recur(rg, al);
-                    }
+                    hits |= hb << (4 * q);
                 }
                 const uint32_t mask = __reduce_or_sync(SG_FULL_MASK, hits);
                 __syncwarp();
@@ -874,7 +852,7 @@ __global__ void __maxnreg__((bwd_max_regs<C, PPT>())) raster_bwd_kernel(RasterAr
                     ldsm_x4(sa + 8 * ks, ar);
 #pragma unroll
                     for (int i = 0; i < 4; ++i) split_tf32(__uint_as_float(ar[i]), ah[i], al[i]);
-                    const float Y = (float)((ks & 3) + 4 * (ks >> 2)) - (2.f * PPT - 0.5f);
+                    const float Y = (float)ks - 1.5f;
                     const uint32_t pb0 = __float_as_uint(fmaf(Y, fmaf(Y, P2, P1a), P0a));
                     const uint32_t pb1 = __float_as_uint(fmaf(Y, fmaf(Y, P2, P1b), P0b));
                     mma_tf32(mom, al, pb0, pb1);
@@ -1058,14 +1036,14 @@ template <int C>
 inline size_t fwd_half_smem() {
     return sizeof(float) * fwd_warp_words<C, 1, true>();
 }
-template <int C, int PPT>
+template <int C>
 inline size_t bwd_smem(int batch, int threads) {
-    return batch_smem<C>(batch) + (size_t)batch * 4 + sizeof(float) * (threads / 32) * bwd_warp_words<C, PPT, false>();
+    return batch_smem<C>(batch) + (size_t)batch * 4 + sizeof(float) * (threads / 32) * bwd_warp_words<C, false>();
 }
 // half mode: one 16-entry chunk staged without its (u, v, ex, ey) rows, one warp
 template <int C>
 inline size_t bwd_half_smem() {
-    return batch_smem<C>(kChunk) - (size_t)kChunk * 16 + (size_t)kChunk * 4 + sizeof(float) * bwd_warp_words<C, 1, true>();
+    return batch_smem<C>(kChunk) - (size_t)kChunk * 16 + (size_t)kChunk * 4 + sizeof(float) * bwd_warp_words<C, true>();
 }
 
 inline int resident_grid(const void *fn, int threads, size_t smem) {
@@ -1077,31 +1055,21 @@ inline int resident_grid(const void *fn, int threads, size_t smem) {
     return sms * per_sm;
 }
 
-template <int C, int PPT>
-sg_status launch_raster_cp(RasterArgs &a, bool backward, cudaStream_t st) {
-    // with half masks, the adjoint of 8 x 8 tiles at one pixel per thread runs one warp per
-    // half tile, and so does the forward when the config asks for it
-    const bool half = a.half && PPT == 1 && a.tile_w == 8 && a.tile_h == 8 && (backward || a.half_fwd);
-    const int threads = half ? 32 : a.tile_w * a.tile_h / PPT;
-    const size_t smem = backward ? (half ? bwd_half_smem<C>() : bwd_smem<C, PPT>(a.batch, threads))
-                                 : (half ? fwd_half_smem<C>() : fwd_smem<C, PPT>(a.batch, threads));
-    const void *fn = backward ? (half ? (const void *)raster_bwd_kernel<C, PPT, PPT == 1>
-                                      : (const void *)raster_bwd_kernel<C, PPT>)
-                              : (half ? (const void *)raster_fwd_kernel<C, PPT, PPT == 1>
-                                      : (const void *)raster_fwd_kernel<C, PPT>);
+// One launch of kernel fn (one of the instantiations below).  configured: the dynamic shared
+// memory that fn has been opted in to.
+inline sg_status launch_raster_fn(void (*fn)(RasterArgs), RasterArgs &a, bool half, bool backward, int threads, size_t smem,
+                                  size_t &configured, cudaStream_t st) {
     // opt in to the dynamic size whenever it grows: at 48 KB and just below, the kernel's
     // static shared variables alone take the total past the default limit
-    static size_t configured[4] = {0, 0, 0, 0};
-    const int which = 2 * (int)backward + (int)half;
-    if (configured[which] < smem) {
+    if (configured < smem) {
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
             return check_launch("raster smem attribute");
-        configured[which] = smem;
+        configured = smem;
     }
     // the half-tile adjoint takes whole tiles as work items when there are at least 16 tiles
     // per resident CTA (measured: batched workload, 29 per CTA, -1.4 %); with fewer, twice as
     // long items leave the persistent grid's tail unbalanced
-    const int resident = a.persistent ? resident_grid(fn, threads, smem) : 0;
+    const int resident = a.persistent ? resident_grid((const void *)fn, threads, smem) : 0;
     a.half_pairs = backward && half && a.persistent && (int64_t)a.n_tiles >= 16 * (int64_t)resident;
     const int n_items = half && !a.half_pairs ? 2 * a.n_tiles : a.n_tiles;
     int grid = n_items;
@@ -1110,24 +1078,41 @@ sg_status launch_raster_cp(RasterArgs &a, bool backward, cudaStream_t st) {
         if (grid > n_items) grid = n_items;
     }
     if (grid <= 0) return SG_OK;
-    if (backward && half)
-        launch_pdl(raster_bwd_kernel<C, PPT, PPT == 1>, grid, threads, smem, st, a);
-    else if (backward)
-        launch_pdl(raster_bwd_kernel<C, PPT>, grid, threads, smem, st, a);
-    else if (half)
-        launch_pdl(raster_fwd_kernel<C, PPT, PPT == 1>, grid, threads, smem, st, a);
-    else
-        launch_pdl(raster_fwd_kernel<C, PPT>, grid, threads, smem, st, a);
+    launch_pdl(fn, grid, threads, smem, st, a);
     count_launches(1);
     return check_launch(backward ? "raster_bwd" : "raster_fwd");
 }
 
+// Lists with half masks (8 x 8 tiles): the adjoint runs one warp per half tile, and so does the
+// forward at one pixel per thread when the config asks for it.
+template <int C, int PPT>
+sg_status launch_raster_fwd(RasterArgs &a, cudaStream_t st) {
+    static size_t configured[2] = {0, 0};
+    const bool half = a.half && PPT == 1 && a.tile_w == 8 && a.tile_h == 8 && a.half_fwd;
+    const int threads = half ? 32 : a.tile_w * a.tile_h / PPT;
+    return half ? launch_raster_fn(raster_fwd_kernel<C, PPT, PPT == 1>, a, true, false, threads, fwd_half_smem<C>(),
+                                   configured[1], st)
+                : launch_raster_fn(raster_fwd_kernel<C, PPT>, a, false, false, threads, fwd_smem<C, PPT>(a.batch, threads),
+                                   configured[0], st);
+}
+
+template <int C>
+sg_status launch_raster_bwd(RasterArgs &a, cudaStream_t st) {
+    static size_t configured[2] = {0, 0};
+    const bool half = a.half && a.tile_w == 8 && a.tile_h == 8;
+    const int threads = half ? 32 : a.tile_w * a.tile_h;
+    return half ? launch_raster_fn(raster_bwd_kernel<C, true>, a, true, true, threads, bwd_half_smem<C>(), configured[1], st)
+                : launch_raster_fn(raster_bwd_kernel<C, false>, a, false, true, threads, bwd_smem<C>(a.batch, threads),
+                                   configured[0], st);
+}
+
 template <int C>
 sg_status launch_raster_c(RasterArgs &a, bool backward, cudaStream_t st) {
+    if (backward) return launch_raster_bwd<C>(a, st);
     switch (a.ppt) {
-        case 1: return launch_raster_cp<C, 1>(a, backward, st);
-        case 2: return launch_raster_cp<C, 2>(a, backward, st);
-        default: return launch_raster_cp<C, 4>(a, backward, st);
+        case 1: return launch_raster_fwd<C, 1>(a, st);
+        case 2: return launch_raster_fwd<C, 2>(a, st);
+        default: return launch_raster_fwd<C, 4>(a, st);
     }
 }
 

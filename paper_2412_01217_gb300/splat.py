@@ -69,12 +69,12 @@ class RenderConfig:
     batch: int = 256
     persistent: bool = True
     pixels_per_thread: int = 1
-    pixels_per_thread_bwd: int = 2
+    pixels_per_thread_bwd: int = 2  # an upper bound: the adjoint runs one pixel per thread
     batch_bwd: int = 0  # 0: same as batch
     isotropic: bool = False  # Eq. 2 projection (radius f r / d) instead of EWA
     check_numeric: bool = False  # flag non-finite Gaussian parameters in the status word
-    # per-instance half masks in the tile lists: the adjoint of 8x8 tiles at one pixel per
-    # thread then runs one warp per half tile (faster on long lists, lists slower to build)
+    # per-instance half masks in the tile lists: the adjoint of 8x8 tiles then runs one warp
+    # per half tile (faster on long lists, lists slower to build)
     half_masks: bool = False
     # with half masks: the forward also one warp per half tile (faster on long lists)
     half_tile_fwd: bool = False
