@@ -659,13 +659,21 @@ __global__ void __launch_bounds__(kLossThreads, 2) ce_decoder_mma_kernel(PixelAr
         cp_async4(s_gd + lane, a.gt_depth + q, ok);
         cp_async_commit_group();
     };
+    // (the unit found for the prefetch is the next iteration's: the search and the division of
+    // the weight by the view's pixel count once a unit instead of twice and four times a lane:
+    // batched workload 402 -> 383 us)
     int u = (int)blockIdx.x * kPixSlots + warp;
-    if (u < n_units) prefetch(unit_of(u));
+    Unit next{};
+    if (u < n_units) {
+        next = unit_of(u);
+        prefetch(next);
+    }
     for (; u < n_units; u += n_warps) {
-        const Unit x = unit_of(u);
+        const Unit x = next;
         const int v = x.v, HW = x.HW, pw = x.pw;
         const size_t p0 = x.p0;
         const int nd = a.counts[2 * v], nl = a.counts[2 * v + 1];
+        const float scale = a.w_sem / (float)nl;
         cp_async_wait_groups<0>();
         __syncwarp();
         float l1d = 0.f, ce = 0.f;
@@ -758,7 +766,7 @@ __global__ void __launch_bounds__(kLossThreads, 2) ce_decoder_mma_kernel(PixelAr
                 se += __shfl_xor_sync(SG_FULL_MASK, se, 2);
                 const bool valid = lab >= 0;
                 if (valid && has_lab) ce += logf(se) - zl;
-                const float sc = valid ? a.w_sem / (float)nl : 0.f;
+                const float sc = valid ? scale : 0.f;
                 const float inv = 1.f / se;
 #pragma unroll
                 for (int nt = 0; nt < NK; ++nt)
@@ -813,7 +821,10 @@ __global__ void __launch_bounds__(kLossThreads, 2) ce_decoder_mma_kernel(PixelAr
         }
         // the stage's last read is done: request the next unit (it arrives during dS)
         __syncwarp();
-        if (u + n_warps < n_units) prefetch(unit_of(u + n_warps));
+        if (u + n_warps < n_units) {
+            next = unit_of(u + n_warps);
+            prefetch(next);
+        }
         // ---- dS = dZ W: M = pixels, N = features, K = classes (permuted within each 8-class step) ----
         {
             float ds[2][NC][4];
