@@ -581,11 +581,23 @@ constexpr int kChunkPitch = 32 + 4;  // 4 mod 32: conflict-free fragments
 template <int NF>
 __host__ __device__ constexpr int padded_features() { return (NF + 7) / 8 * 8; }
 
-// Row pitch of the per-warp copy of dL/dimage: the least odd multiple of 4 that holds the NF
-// features (conflict-free fragment loads).  Features NF .. padded_features - 1 of the last
-// 8-feature tile are not stored: their fragment loads are predicated to zero.
+// Row pitch of the per-warp copy G of dL/dimage (a row per pixel).  It is read by ldmatrix (8
+// rows of 16 bytes) and by words, lane (gid, tig) row tig and column gid of a tile.  Where the
+// features padded to 8 are 8 mod 16 (C = 4, 16, 32) that is the pitch, with the 4-column groups of
+// rows 4 .. 7 of every 8 swapped (g_swap): both reads are then free of bank conflicts (at the
+// least odd multiple of 4 the word reads took two passes, 24 of some 330 shared-memory passes of
+// a chunk; batched workload 2030 -> 2006 us, 1200x680 x 3 levels 276 -> 272).  Otherwise the least odd multiple of 4 that holds the features: padding to 8 mod 16
+// would cost a CTA per SM.  Features NF .. padded_features - 1 are not stored: their fragment
+// loads are predicated to zero.
 template <int NF>
-__host__ __device__ constexpr int g_pitch() { return (NF / 4) % 2 == 1 ? NF : NF + 4; }
+__host__ __device__ constexpr bool g_swapped() { return padded_features<NF>() % 16 == 8; }
+template <int NF>
+__host__ __device__ constexpr int g_pitch() {
+    return g_swapped<NF>() ? padded_features<NF>() : (NF / 4) % 2 == 1 ? NF : NF + 4;
+}
+// what to exclusive-or a 4-column group's index with in G's row p
+template <int NF>
+__device__ __forceinline__ int g_swap(int p) { return g_swapped<NF>() ? (p >> 2) & 1 : 0; }
 
 // The adjoint gives every thread one pixel, whatever the forward's number.  With two or four, the
 // per-chunk costs are shared by more pixels, but half or a quarter of the warps are left, each
@@ -729,7 +741,7 @@ __global__ void __maxnreg__((bwd_max_regs<C>())) raster_bwd_kernel(RasterArgs a)
             acc_a = g[0] * a.bg0 + g[1] * a.bg1 + g[2] * a.bg2;
             float4 *row = reinterpret_cast<float4 *>(s_G + lane * GP);
 #pragma unroll
-            for (int f = 0; f < NF; f += 4) row[f / 4] = make_float4(g[f], g[f + 1], g[f + 2], g[f + 3]);
+            for (int f = 0; f < NF; f += 4) row[(f / 4) ^ g_swap<NF>(lane)] = make_float4(g[f], g[f + 1], g[f + 2], g[f + 3]);
         }
         const int warp_last = __reduce_max_sync(SG_FULL_MASK, my_last);
         __syncwarp();
@@ -743,7 +755,8 @@ __global__ void __maxnreg__((bwd_max_regs<C>())) raster_bwd_kernel(RasterArgs a)
                 // 16-31 the same rows four columns further (A); lanes 8 m + i row i of matrix m (B)
                 {
                     const float *fa = s_feat + (size_t)row_of(lane & 15) * NF + 4 * (lane >> 4);
-                    const float *ga = s_G + ((lane & 7) + 8 * (lane >> 4)) * GP + 4 * ((lane >> 3) & 1);
+                    const float *ga =
+                        s_G + ((lane & 7) + 8 * (lane >> 4)) * GP + 4 * (((lane >> 3) & 1) ^ g_swap<NF>(lane & 7));
                     float d[KS][4];
 #pragma unroll
                     for (int nt = 0; nt < KS; ++nt) d[nt][0] = d[nt][1] = d[nt][2] = d[nt][3] = 0.f;
@@ -773,7 +786,7 @@ __global__ void __maxnreg__((bwd_max_regs<C>())) raster_bwd_kernel(RasterArgs a)
 #pragma unroll
                         for (int n4 = 0; n4 < KS / 4; ++n4) {
                             uint32_t br[4];
-                            ldsm_x4(s_G + (32 * n4 + lane) * GP + 8 * (NF / 8), br);
+                            ldsm_x4(s_G + (32 * n4 + lane) * GP + 8 * (NF / 8) + 4 * g_swap<NF>(lane), br);
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
                                 uint32_t bh, bl;
@@ -842,11 +855,11 @@ __global__ void __maxnreg__((bwd_max_regs<C>())) raster_bwd_kernel(RasterArgs a)
 #pragma unroll
                     for (int nt = 0; nt < NT; ++nt) {
                         // B (8 x 8): b0 (tig, gid), b1 (tig + 4, gid) = G[pixel][feature]
-                        const float *gp = s_G + (8 * ks + tig) * GP + 8 * nt + gid;
+                        const float *gp = s_G + (8 * ks + tig) * GP + 8 * nt;
                         const bool stored = 8 * nt + 8 <= NF || 8 * nt + gid < NF;
                         uint32_t bh0, bl0, bh1, bl1;
-                        split_tf32(stored ? gp[0] : 0.f, bh0, bl0);
-                        split_tf32(stored ? gp[4 * GP] : 0.f, bh1, bl1);
+                        split_tf32(stored ? gp[gid] : 0.f, bh0, bl0);
+                        split_tf32(stored ? gp[4 * GP + (gid ^ (g_swapped<NF>() ? 4 : 0))] : 0.f, bh1, bl1);
                         mma_tf32x3(df[nt], ah, al, bh0, bh1, bl0, bl1);
                     }
                     ldsm_x4(sa + 8 * ks, ar);

@@ -89,6 +89,13 @@ def test_stacks_around_the_chunk_size_match_oracle(n, C, cfg):
     check_grads({k: v.cpu().numpy() for k, v in grads.items()}, want, KEYS)
 
 
+@pytest.mark.parametrize("C", [4, 16])
+def test_half_mask_lists_with_a_larger_bound_on_the_adjoint_s_pixels(C):
+    """Lists with half masks take the half-tile adjoint whatever pixels_per_thread_bwd bounds."""
+    test_stacks_around_the_chunk_size_match_oracle(
+        17, C, dict(tile_w=8, tile_h=8, pixels_per_thread=1, pixels_per_thread_bwd=2, half_masks=True))
+
+
 @pytest.mark.parametrize("M, N, K, pad", [(130, 72, 128, 0), (130, 72, 128, 1), (128, 160, 4096, 4), (64, 288, 192, 3),
                                           (300, 32, 64, 2)])
 @pytest.mark.parametrize("accumulate", [0, 1])
