@@ -390,9 +390,30 @@ struct PixelArgs {
 // block sum and zeroes the others).
 constexpr int kPixSlots = kLossThreads / 32;
 
-// Two-level, fixed-order reduction of the per-CTA decoder-gradient shares:
+// Fixed-order reduction of the per-CTA decoder-gradient shares.  Up to kDecRows rows (what the
+// persistent kernel's resident grid writes) are summed by one kernel: a CTA takes 32 outputs, warp
+// w rows w, w + 32, ..., the warps in a fixed tree (304 rows of 512: 7.4 us for the two
+// kernels below, most of it latency).  More rows go in two levels:
 // level 1: chunk c of kDecChunks sums CTAs [c n / kDecChunks, (c+1) n / kDecChunks);
 // level 2: decoder_grad[o] += sum over chunks.
+constexpr int kDecRows = 1024;
+__global__ void __launch_bounds__(1024) decoder_reduce_kernel(const float *__restrict__ part, int rows, int KC,
+                                                              float *__restrict__ out) {
+    pdl_begin();
+    __shared__ float s_sum[32][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, o = blockIdx.x * 32 + lane;
+    float s = 0.f;
+    if (o < KC)
+#pragma unroll 8
+        for (int b = warp; b < rows; b += 32) s += part[(size_t)b * KC + o];
+    s_sum[lane][warp] = s;
+    __syncthreads();
+    // warp w adds output w's 32 sums
+    float t = s_sum[warp][lane];
+#pragma unroll
+    for (int i = 16; i > 0; i >>= 1) t += __shfl_xor_sync(SG_FULL_MASK, t, i);
+    if (lane == 0 && blockIdx.x * 32 + warp < KC) out[blockIdx.x * 32 + warp] += t;
+}
 constexpr int kDecChunks = 128;
 __global__ void decoder_reduce1_kernel(const float *__restrict__ part, int n_blocks, int KC,
                                        float *__restrict__ chunk_sums) {
@@ -917,22 +938,26 @@ struct FinalArgs {
     uint32_t *status;  // non-NULL: flag non-finite loss terms (SG_STATUS_NUMERIC)
 };
 
-// Sum of v over the block in double, in a fixed order (warp butterflies, then the warps in
-// order); the result is valid in thread 0.
-__device__ __forceinline__ double block_sum_d(double v, double *s_w) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(SG_FULL_MASK, v, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < kLossThreads / 32; ++w) t += s_w[w];
-    return t;
-}
+// A sum of floats with the rounding errors kept beside it (about 48 bits).
+struct PairSum {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const DF s = two_sum(hi, x);
+        hi = s.hi;
+        lo += s.lo;
+    }
+    __device__ __forceinline__ void add(float h, float l) {
+        add(h);
+        lo += l;
+    }
+    // (an infinite sum has no error term)
+    __device__ __forceinline__ double value() const { return isinf(hi) ? (double)hi : (double)hi + (double)lo; }
+};
 
 // A view's partial sums and its loss terms by a cluster of kFinalCtas CTAs, their shares added
 // in rank order through distributed shared memory.  Bound by the latency of the partials'
-// loads and the double additions, of which one SM does a few per clock: 1200x680 x 3 levels with
+// loads; the sums over a CTA are pairs of floats, because an SM does only a few double additions
+// per clock (12.7 us with doubles, 637x477 x 3 levels 9.7 -> 7.2): 1200x680 x 3 levels with
 // one CTA per view took 38 us (loss with a 32-class decoder 198 -> 173 us, 637x477 x 3
 // levels without one 81 -> 73).
 constexpr int kFinalCtas = 8;
@@ -945,19 +970,18 @@ __global__ void __cluster_dims__(kFinalCtas, 1, 1) __launch_bounds__(kLossThread
     constexpr int kStride = kFinalCtas * kLossThreads;
     const sg_view &vw = a.views[v];
     const double HW = (double)vw.W * vw.H;
-    __shared__ double s_w[kLossThreads / 32];
+    __shared__ PairSum s_w[kLossThreads / 32][4];
     __shared__ double s_part[kFinalCtas][4];  // (rank 0's holds the shares)
-    double acc[2] = {0, 0};  // colour, semantics
+    PairSum part[4];  // colour, semantics, depth L1, CE
     for (int i = a.lv.tile_off[v] + first; i < a.lv.tile_off[v + 1]; i += kStride)
 #pragma unroll
         for (int g = 0; g < kSsimGroups; ++g)
             if (g < a.rgb_groups + a.sem_groups) {
-                const double t = a.ssim[(size_t)g * a.n_tiles + i];
-                if (g < a.rgb_groups) acc[0] += t; else acc[1] += t;
+                const float t = a.ssim[(size_t)g * a.n_tiles + i];
+                if (g < a.rgb_groups) part[0].add(t); else part[1].add(t);
             }
     // the per-unit (depth L1, CE) sums: two units per 16-byte load, four loads in flight per
     // thread, summed in a fixed order
-    double b[2] = {0, 0};
     {
         const float4 *p4 = reinterpret_cast<const float4 *>(a.pix);
         const int s1 = kPixSlots * a.lv.pix_blk_off[v + 1] / 2;
@@ -968,40 +992,49 @@ __global__ void __cluster_dims__(kFinalCtas, 1, 1) __launch_bounds__(kLossThread
                 q[k] = i + k * kStride < s1 ? p4[i + k * kStride] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                b[0] += (double)q[k].x + (double)q[k].z;
-                b[1] += (double)q[k].y + (double)q[k].w;
+                part[2].add(q[k].x);
+                part[2].add(q[k].z);
+                part[3].add(q[k].y);
+                part[3].add(q[k].w);
             }
         }
     }
-    const double part[4] = {block_sum_d(acc[0], s_w), block_sum_d(acc[1], s_w), block_sum_d(b[0], s_w),
-                            block_sum_d(b[1], s_w)};
-    cluster.sync();  // (rank 0 runs: its shared memory can be written)
-    if (threadIdx.x == 0) {
-        double *to = cluster.map_shared_rank(&s_part[rank][0], 0);
+    // the four sums side by side: warp trees, then one thread each over the warps and the CTAs, in
+    // order and in double
 #pragma unroll
-        for (int k = 0; k < 4; ++k) to[k] = part[k];
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            part[k].add(__shfl_down_sync(SG_FULL_MASK, part[k].hi, o), __shfl_down_sync(SG_FULL_MASK, part[k].lo, o));
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s_w[threadIdx.x >> 5][k] = part[k];
+    cluster.sync();  // (rank 0 runs: its shared memory can be written)
+    const int k = threadIdx.x;
+    if (k < 4) {
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < kLossThreads / 32; ++w) t += s_w[w][k].value();
+        *cluster.map_shared_rank(&s_part[rank][k], 0) = t;
     }
     cluster.sync();
-    if (rank != 0) return;
-    double sum[4] = {0, 0, 0, 0};
-    for (int r = 0; r < kFinalCtas; ++r)
+    if (rank != 0 || threadIdx.x >= 32) return;
+    double t = 0.0;
+    if (k < 4)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) sum[k] += s_part[r][k];
-    const double r_rgb = sum[0], r_sem = sum[1], l1d_sum = sum[2], ce_sum = sum[3];
-    if (threadIdx.x == 0) {
-        const double l1d = l1d_sum, ce = ce_sum;
-        const int nd = a.counts[2 * v], nl = a.counts[2 * v + 1];
-        const double n_rgb = 3.0 * HW;
-        // (1 - lambda) L1 + lambda (1 - SSIM)
-        const double L_r = r_rgb / n_rgb + a.lambda_r;
-        const double L_d = nd > 0 ? a.w_depth * l1d / nd : 0.0;
-        double L_s;
-        if (a.sem_mode == 0) {
-            L_s = nl > 0 ? a.w_sem * ce / nl : 0.0;
-        } else {
-            const double n_s = (double)a.C * HW;
-            L_s = a.w_sem * (r_sem / n_s + a.lambda_s);
-        }
+        for (int r = 0; r < kFinalCtas; ++r) t += s_part[r][k];
+    // thread k's term: colour, semantic images, depth, cross-entropy
+    const int nd = a.counts[2 * v], nl = a.counts[2 * v + 1];
+    const double n = k == 0 ? 3.0 * HW : k == 1 ? (double)a.C * HW : (double)(k == 2 ? nd : nl);
+    double L = n > 0.0 ? t / n : 0.0;
+    // (1 - lambda) L1 + lambda (1 - SSIM)
+    if (k == 0) L += a.lambda_r;
+    if (k == 1) L = a.w_sem * (L + a.lambda_s);
+    if (k == 2) L *= a.w_depth;
+    if (k == 3) L *= a.w_sem;
+    const double L_r = __shfl_sync(SG_FULL_MASK, L, 0), L_d = __shfl_sync(SG_FULL_MASK, L, 2);
+    const double L_s = __shfl_sync(SG_FULL_MASK, L, a.sem_mode == 0 ? 3 : 1);
+    if (k == 0) {
         a.terms[4 * v + 0] = (float)L_r;
         a.terms[4 * v + 1] = (float)L_d;
         a.terms[4 * v + 2] = (float)L_s;
@@ -1125,9 +1158,14 @@ sg_status launch_loss(const sg_images *r, const sg_targets *gt, const sg_view *v
         return SG_ERR_INVALID_ARG;
     }
     if (ce && lc->decoder_grad) {
-        launch_pdl(decoder_reduce1_kernel, dim3((KC + 127) / 128, kDecChunks), 128, 0, st, p_dec, dec_rows, KC, p_dec2);
-        launch_pdl(decoder_reduce2_kernel, (KC + 127) / 128, 128, 0, st, p_dec2, KC, lc->decoder_grad);
-        count_launches(2);
+        if (dec_rows <= kDecRows) {
+            launch_pdl(decoder_reduce_kernel, (KC + 31) / 32, 1024, 0, st, p_dec, dec_rows, KC, lc->decoder_grad);
+            count_launches(1);
+        } else {
+            launch_pdl(decoder_reduce1_kernel, dim3((KC + 127) / 128, kDecChunks), 128, 0, st, p_dec, dec_rows, KC, p_dec2);
+            launch_pdl(decoder_reduce2_kernel, (KC + 127) / 128, 128, 0, st, p_dec2, KC, lc->decoder_grad);
+            count_launches(2);
+        }
     }
     FinalArgs fa{p_ssim, p_pix, rgb_groups, sem_groups, n_tiles, counts, views, lv, C, lc->sem_mode,
                  lc->lambda_r, lc->lambda_s, lc->w_depth, lc->w_sem, terms, status};
