@@ -121,6 +121,13 @@ sg_status launch_gemm(tc::GemmParams p, cudaStream_t st, int max_splits = 64) {
     p.vec_mask = p.mask && p.ldmask % 8 == 0 && (uintptr_t)p.mask % 16 == 0;
     p.vec_bf16 = p.out_bf16 && p.ld_bf16 % 8 == 0 && (uintptr_t)p.out_bf16 % 16 == 0;
     p.vec_f32 = p.out_f32 && p.ld_f32 % 4 == 0 && (uintptr_t)p.out_f32 % 16 == 0;
+    // fewer tiles than half the SMs: narrower ones, each with the same K order, so that more SMs
+    // stream the operands; the A rows they read again come from L2.  An SM then takes in 640 or
+    // 768 KiB of a 2048-deep layer instead of 1 MiB, in parallel with more of the others (network
+    // forward at up to 4864 rows 32.8 -> 26.7 us, at 5120 to 8192 28.7; training step at 2048
+    // rows 76 -> 66; the same from 77 tiles on)
+    if (BN == 128 && splits == 1 && 2 * tiles <= sms)
+        return tiles * ((p.N + 31) / 32) <= sms ? launch_gemm_t<32, 8>(p, splits, st) : launch_gemm_t<64, 6>(p, splits, st);
     switch (BN) {
         case 32: return launch_gemm_t<32, 4>(p, splits, st);
         // with more tiles than SMs, 3 stages of 32 KiB: two CTAs per SM keep twice the operand

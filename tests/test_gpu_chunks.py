@@ -118,6 +118,29 @@ def test_gemm_epilogue_edges_and_unaligned_rows(M, N, K, pad, accumulate):
     assert bool((D[:, N:] == 0.5).all())
 
 
+@pytest.mark.parametrize("M, N", [(4865, 128), (4865, 100), (9728, 65)])
+def test_gemm_with_few_tiles_takes_narrower_ones(M, N):
+    """64-column tiles (39 to 76 tiles of 128 columns), with ragged rows and columns: the result
+    of each row block computed alone (32-column tiles, the same K order), bit for bit."""
+    import ctypes
+    from paper_2412_01217_gb300._lib import call
+    torch.manual_seed(M + N)
+    K = 192
+    A = torch.randn(M, K, device="cuda").to(torch.bfloat16)
+    B = torch.randn(N, K, device="cuda").to(torch.bfloat16)
+    st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    ptr = lambda t: ctypes.c_void_p(t.data_ptr())
+    D, E = torch.full((M, N), 0.5, device="cuda"), torch.full((M, N), 0.5, device="cuda")
+    call("sg_gemm_bf16", ptr(A), K, ptr(B), K, M, N, K, ptr(D), N, 0, None, st)
+    for m in range(0, M, 1024):
+        a, e = A[m:m + 1024], E[m:m + 1024]
+        call("sg_gemm_bf16", ptr(a), K, ptr(B), K, a.shape[0], N, K, ptr(e), N, 0, None, st)
+    torch.cuda.synchronize()
+    ref = A.double() @ B.double().T
+    assert (D.double() - ref).abs().max().item() <= 1e-5 * ref.abs().max().item() + 1e-3
+    assert torch.equal(D, E)
+
+
 def test_mlp_backward_takes_unaligned_targets():
     """The loss head reads Y and the targets 16 bytes at a time only when both are aligned: the
     same batch with targets one float off gives the same bf16 output gradients."""
