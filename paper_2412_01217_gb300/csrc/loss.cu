@@ -114,17 +114,19 @@ __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
 // Sliding-window separable passes: each thread produces a run of consecutive outputs of one
 // row (horizontal) or column (vertical), adding each input to every output whose window
 // holds it.  The kernel is bound by instruction issue, so the window sums run two quantities
-// to an instruction: the planes are staged as (x, y) pairs, the four moments (x, y),
-// (x^2 + y^2, xy) -- SSIM takes the two variances only by their sum -- as 16-byte entries, and
-// two of the three partials as pairs, which also makes every shared-memory access of a pass
-// one 8- or 16-byte word.  1200x680 x 3 levels: 66 us against 101 with one quantity per
-// instruction, five moments and a tile's planes in one CTA (loss with a 32-class decoder
-// 233 -> 198 us; colour and four semantic planes at 637x477 x 3 levels 113 -> 81 us).
+// to an instruction: the planes are staged as (x, y) pairs, the five moments as (x, y), (x^2, y^2)
+// and xy, and two of the three partials as pairs, which also makes most shared-memory accesses
+// one 8- or 16-byte word.  Every sum keeps its order, so the gradients are bit for bit those of
+// one quantity per instruction, with which 1200x680 x 3 levels took 101 us against about 77 (loss
+// with a 32-class decoder 233 -> 174 us, colour and four semantic planes at 637x477 x 3 levels
+// 112 -> 79, with the loss's other kernels).  One moment of x^2 + y^2 in place of two took 66 us,
+// but its rounding put the gradients of flat regions up to 1.46 times as far from 64 bits.
 __global__ void __launch_bounds__(kLossThreads, 3) ssim_l1_kernel(SsimArgs a) {
     pdl_begin();
     extern __shared__ __align__(16) float sm[];
     float4 *Hm = reinterpret_cast<float4 *>(sm);                // kXH x kMP moments
-    float2 *XY = reinterpret_cast<float2 *>(Hm + kXH * kMP);    // kXH x kXP staged planes
+    float *Hxy = reinterpret_cast<float *>(Hm + kXH * kMP);      // kXH x kMP: the moment of xy
+    float2 *XY = reinterpret_cast<float2 *>(Hxy + kXH * kMP);   // kXH x kXP staged planes
     // the partials reuse the staged planes once the horizontal pass has consumed them, and
     // their horizontal sums the moments
     float2 *PQ = XY;                                            // kMH x kMP
@@ -190,23 +192,30 @@ __global__ void __launch_bounds__(kLossThreads, 3) ssim_l1_kernel(SsimArgs a) {
                 const int seg = it / kXH, r = it - seg * kXH;
                 const int c0 = seg * RUN;
                 F2 s[RUN][2];
+                float sxy[RUN];
 #pragma unroll
-                for (int o = 0; o < RUN; ++o) s[o][0] = s[o][1] = f2(0.f, 0.f);
+                for (int o = 0; o < RUN; ++o) {
+                    s[o][0] = s[o][1] = f2(0.f, 0.f);
+                    sxy[o] = 0.f;
+                }
 #pragma unroll
                 for (int i = 0; i < RUN + 10; ++i) {
                     const float2 q = XY[r * kXP + c0 + i];
-                    const F2 xy = f2(q.x, q.y), mom = f2(fmaf(q.y, q.y, q.x * q.x), q.x * q.y);
+                    const F2 xy = f2(q.x, q.y), sq = f2(q.x * q.x, q.y * q.y);
+                    const float pr = q.x * q.y;
 #pragma unroll
                     for (int o = 0; o < RUN; ++o)
                         if (i - o >= 0 && i - o < 11) {
                             s[o][0] = fma2(wr[i - o], xy, s[o][0]);
-                            s[o][1] = fma2(wr[i - o], mom, s[o][1]);
+                            s[o][1] = fma2(wr[i - o], sq, s[o][1]);
+                            sxy[o] = fmaf(w1(i - o), pr, sxy[o]);
                         }
                 }
 #pragma unroll
                 for (int o = 0; o < RUN; ++o) {
                     const float2 p = unpack(s[o][0]), q = unpack(s[o][1]);
                     Hm[r * kMP + c0 + o] = make_float4(p.x, p.y, q.x, q.y);
+                    Hxy[r * kMP + c0 + o] = sxy[o];
                 }
             }
         }
@@ -219,17 +228,23 @@ __global__ void __launch_bounds__(kLossThreads, 3) ssim_l1_kernel(SsimArgs a) {
                 const int seg = it / kMW, c = it - seg * kMW;
                 const int r0 = seg * RUN;
                 F2 m[RUN][2];
+                float mxy[RUN];
 #pragma unroll
-                for (int o = 0; o < RUN; ++o) m[o][0] = m[o][1] = f2(0.f, 0.f);
+                for (int o = 0; o < RUN; ++o) {
+                    m[o][0] = m[o][1] = f2(0.f, 0.f);
+                    mxy[o] = 0.f;
+                }
 #pragma unroll
                 for (int i = 0; i < RUN + 10; ++i) {
                     const float4 q = Hm[(r0 + i) * kMP + c];
-                    const F2 xy = f2(q.x, q.y), mom = f2(q.z, q.w);
+                    const F2 xy = f2(q.x, q.y), sq = f2(q.z, q.w);
+                    const float pr = Hxy[(r0 + i) * kMP + c];
 #pragma unroll
                     for (int o = 0; o < RUN; ++o)
                         if (i - o >= 0 && i - o < 11) {
                             m[o][0] = fma2(wr[i - o], xy, m[o][0]);
-                            m[o][1] = fma2(wr[i - o], mom, m[o][1]);
+                            m[o][1] = fma2(wr[i - o], sq, m[o][1]);
+                            mxy[o] = fmaf(w1(i - o), pr, mxy[o]);
                         }
                 }
 #pragma unroll
@@ -240,14 +255,14 @@ __global__ void __launch_bounds__(kLossThreads, 3) ssim_l1_kernel(SsimArgs a) {
                     if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
                         const float2 mu = unpack(m[o][0]), e2 = unpack(m[o][1]);
                         const float mx = mu.x, my = mu.y;
-                        const float A1 = 2.f * mx * my + C1, A2 = 2.f * (e2.y - mx * my) + C2;
-                        const float B1 = fmaf(mx, mx, my * my) + C1;
-                        const float B2 = fmaf(-my, my, fmaf(-mx, mx, e2.x)) + C2;
+                        const float sxx = e2.x - mx * mx, syy = e2.y - my * my, sxy = mxy[o] - mx * my;
+                        const float A1 = 2.f * mx * my + C1, A2 = 2.f * sxy + C2;
+                        const float B1 = mx * mx + my * my + C1, B2 = sxx + syy + C2;
                         const float inv = 1.f / (B1 * B2);
                         const float s = A1 * A2 * inv;
                         if (r >= 5 && r < kLTH + 5 && c >= 5 && c < kLTW + 5) ssim_sum += s;
-                        const float d_mx = 2.f * my * A2 * inv - s * 2.f * mx * (B2 * inv);
-                        const float d_sxx = -s * (B1 * inv);
+                        const float d_mx = 2.f * my * A2 * inv - s * 2.f * mx / B1;
+                        const float d_sxx = -s / B2;
                         const float d_sxy = 2.f * A1 * inv;
                         P = sc * (d_mx - 2.f * mx * d_sxx - my * d_sxy);
                         Q = sc * d_sxx;
@@ -958,8 +973,7 @@ struct PairSum {
 // in rank order through distributed shared memory.  Bound by the latency of the partials'
 // loads; the sums over a CTA are pairs of floats, because an SM does only a few double additions
 // per clock (12.7 us with doubles, 637x477 x 3 levels 9.7 -> 7.2): 1200x680 x 3 levels with
-// one CTA per view took 38 us (loss with a 32-class decoder 198 -> 173 us, 637x477 x 3
-// levels without one 81 -> 73).
+// one CTA per view took 38 us (25 us less of the loss with a 32-class decoder).
 constexpr int kFinalCtas = 8;
 __global__ void __cluster_dims__(kFinalCtas, 1, 1) __launch_bounds__(kLossThreads) loss_finalize_kernel(FinalArgs a) {
     pdl_begin();
@@ -1045,7 +1059,7 @@ __global__ void __cluster_dims__(kFinalCtas, 1, 1) __launch_bounds__(kLossThread
 
 // ---------------------------------------------------------------------------------------
 
-static size_t ssim_smem() { return sizeof(float) * (2 * kXH * kXP + 4 * kXH * kMP); }
+static size_t ssim_smem() { return sizeof(float) * (2 * kXH * kXP + 5 * kXH * kMP); }
 
 static void make_loss_views(const sg_view *vh, int n_views, LossViews &lv) {
     lv.n = n_views;
