@@ -485,6 +485,16 @@ sg_status sg_mlp_backward(const sg_mlp *net, const uint16_t *Xt, const float *ta
                           const float *out_weight, int32_t B, sg_mlp_acts *acts,
                           sg_mlp_grads *grads, float *loss, uint32_t *status, sg_stream_t stream);
 
+/* The same with a workspace of sg_mlp_backward_workspace_size(B) bytes for the current device
+ * (16-byte aligned; its contents do not matter): the parts of the K-split weight gradients and of
+ * the loss are added in a fixed order, so the same inputs give the same bits, where
+ * sg_mlp_backward adds them atomically in any order.  SG_ERR_CAPACITY: workspace too small. */
+size_t sg_mlp_backward_workspace_size(int32_t B);
+sg_status sg_mlp_backward_ordered(const sg_mlp *net, const uint16_t *Xt, const float *target,
+                                  const float *out_weight, int32_t B, sg_mlp_acts *acts,
+                                  sg_mlp_grads *grads, float *loss, void *workspace,
+                                  size_t workspace_bytes, uint32_t *status, sg_stream_t stream);
+
 /* Sec. III-A (the mapping thread converts keyframe data into Gaussian primitives): for B
  * pixels (x, y) of a level-0 frame (planar rgb 3 x H x W, depth H x W, label H x W or NULL)
  * with valid depth, writes B new Gaussians into out (device arrays with room for B; out->C

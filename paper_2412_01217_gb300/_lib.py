@@ -135,6 +135,9 @@ SIGNATURES = {
     "sg_mlp_pack_weights": (c_i, [c_p] * 8 + [c_p]),
     "sg_mlp_forward": (c_i, [P(SgMlp), c_p, c_i, P(SgMlpActs), c_p, c_p]),
     "sg_mlp_backward": (c_i, [P(SgMlp), c_p, c_p, c_p, c_i, P(SgMlpActs), P(SgMlpGrads), c_p, c_p, c_p]),
+    "sg_mlp_backward_workspace_size": (C.c_size_t, [c_i]),
+    "sg_mlp_backward_ordered": (c_i, [P(SgMlp), c_p, c_p, c_p, c_i, P(SgMlpActs), P(SgMlpGrads), c_p, c_p,
+                                      C.c_size_t, c_p, c_p]),
     "sg_extract_patches": (c_i, [c_p, c_p, c_p, P(SgCamera), c_p, c_i, c_i, c_p, c_p, c_p]),
     "sg_init_gaussians": (c_i, [c_p, c_p, c_p, P(SgCamera), c_p, c_i, c_p, c_i, c_f, P(SgGaussians), c_p]),
     "sg_apply_mlp_init": (c_i, [c_p, c_i, c_p, c_p, P(SgGaussians), c_p]),

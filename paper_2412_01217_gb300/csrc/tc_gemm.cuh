@@ -181,6 +181,9 @@ struct GemmParams {
     long long ld_f32;
     int f32_transposed;
     int f32_atomic;  // 1: atomicAdd (split-K / accumulation), 0: store
+    // split-K without atomics (f32_atomic 0): split z stores its product at
+    // out_f32 + z * split_stride, zeros if it timed out; the caller adds the splits.  0: no split
+    long long split_stride;
     // 16-byte accesses to a row of the mask, out_bf16, out_f32 (bases and leading dimensions
     // aligned; set by the launch)
     int vec_mask, vec_bf16, vec_f32;
@@ -352,14 +355,18 @@ __global__ void __launch_bounds__(128, 2) gemm_kernel(const GemmParams p, const 
     tc_fence_after();
     __syncthreads();
     const bool write = done && !s_timeout;
+    if (!write) issued = 0;
     const int row = warp * 32 + lane;
     const int gm = m0 + row;
-    if (write) {
+    float *const out_f32 = p.out_f32 ? p.out_f32 + (long long)blockIdx.z * p.split_stride : nullptr;
+    if (write || p.split_stride) {
 #pragma unroll 1
         for (int c0 = 0; c0 < BN; c0 += 32) {
             uint32_t r[32];
-            tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, r);
-            tmem_ld_wait();
+            if (write) {
+                tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, r);
+                tmem_ld_wait();
+            }
             if (gm >= p.M) continue;
             const int nc = n0 + c0;
             if (nc + 32 <= p.N && (!p.mask || p.vec_mask) && (!p.out_bf16 || p.vec_bf16) &&
@@ -410,14 +417,14 @@ __global__ void __launch_bounds__(128, 2) gemm_kernel(const GemmParams p, const 
                 }
                 if (p.out_f32 && (issued > 0 || !p.f32_atomic)) {
                     if (p.f32_transposed) {
-                        float *o = p.out_f32 + (long long)nc * p.ld_f32 + gm;
+                        float *o = out_f32 + (long long)nc * p.ld_f32 + gm;
 #pragma unroll
                         for (int j = 0; j < 32; ++j) {
                             if (p.f32_atomic) atomicAdd(o + (long long)j * p.ld_f32, v[j]);
                             else o[(long long)j * p.ld_f32] = v[j];
                         }
                     } else {
-                        float *o = p.out_f32 + (long long)gm * p.ld_f32 + nc;
+                        float *o = out_f32 + (long long)gm * p.ld_f32 + nc;
 #pragma unroll
                         for (int q = 0; q < 8; ++q) {
                             if (p.f32_atomic) red_add_v4(o + 4 * q, v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
@@ -439,8 +446,8 @@ __global__ void __launch_bounds__(128, 2) gemm_kernel(const GemmParams p, const 
                 if (p.out_bf16) p.out_bf16[(long long)gm * p.ld_bf16 + gn] = __float2bfloat16_rn(v);
                 if (p.out_bf16_t) p.out_bf16_t[(long long)gn * p.ld_bf16_t + gm] = __float2bfloat16_rn(v);
                 if (p.out_f32) {
-                    float *dst = p.f32_transposed ? p.out_f32 + (long long)gn * p.ld_f32 + gm
-                                                  : p.out_f32 + (long long)gm * p.ld_f32 + gn;
+                    float *dst = p.f32_transposed ? out_f32 + (long long)gn * p.ld_f32 + gm
+                                                  : out_f32 + (long long)gm * p.ld_f32 + gn;
                     if (p.f32_atomic) {
                         if (issued > 0) atomicAdd(dst, v);
                     } else {

@@ -55,6 +55,7 @@ class MLPInit:
         self.status = torch.zeros(1, dtype=torch.int32, device=dev)
         self.device = dev
         self._acts = {}
+        self._work = {}
         self.pack()
 
     def pack(self):
@@ -76,6 +77,13 @@ class MLPInit:
             self._acts[B] = (a, s)
         return self._acts[B]
 
+    def work(self, B):
+        """Workspace of the backward at batch B (the parts of the K-split weight gradients)."""
+        if B not in self._work:
+            n = _lib.load().sg_mlp_backward_workspace_size(B)
+            self._work[B] = torch.empty(n, dtype=torch.uint8, device=self.device)
+        return self._work[B]
+
     def set_standardisation(self, T):
         """Per-output mean/std of the (un-standardised) training targets T [n][32]."""
         self.y_mean = T.mean(0)
@@ -90,13 +98,15 @@ class MLPInit:
         return a["Y"]
 
     def train_step(self, X, Xt, T_std, B, loss_acc):
-        """One Adam step on a batch: X [B][2048], Xt [2048][B] bf16, standardised targets."""
+        """One Adam step on a batch: X [B][2048], Xt [2048][B] bf16, standardised targets.  The
+        same inputs give the same bits."""
         a, s = self.acts(B)
         net = self.net()
         G = SgMlpGrads(*[t.data_ptr() for t in self.grads])
         call("sg_mlp_forward", C.byref(net), _p(X), B, C.byref(s), _p(self.status), stream_ptr())
-        call("sg_mlp_backward", C.byref(net), _p(Xt), _p(T_std), _p(self.out_w), B, C.byref(s), C.byref(G),
-             _p(loss_acc), _p(self.status), stream_ptr())
+        work = self.work(B)
+        call("sg_mlp_backward_ordered", C.byref(net), _p(Xt), _p(T_std), _p(self.out_w), B, C.byref(s), C.byref(G),
+             _p(loss_acc), _p(work), work.numel(), _p(self.status), stream_ptr())
         self.step_count += 1
         groups = (SgAdamGroup * 6)(*[SgAdamGroup(p.data_ptr(), g.data_ptr(), m.data_ptr(), v.data_ptr(),
                                                   p.numel(), self.lr)

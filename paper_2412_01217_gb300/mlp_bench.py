@@ -40,15 +40,16 @@ def time_batch(B, reps=20, seed=0):
     st = lambda: C.c_void_p(torch.cuda.current_stream().cuda_stream)
     grads = SgMlpGrads(*[t.data_ptr() for t in mlp.grads])
     loss = torch.zeros(1, device="cuda")
+    work = mlp.work(B)
 
     def fwd():
         call("sg_mlp_forward", C.byref(net), C.c_void_p(X.data_ptr()), B, C.byref(s), C.c_void_p(mlp.status.data_ptr()),
              st())
 
     def bwd():
-        call("sg_mlp_backward", C.byref(net), C.c_void_p(Xt.data_ptr()), C.c_void_p(T.data_ptr()),
+        call("sg_mlp_backward_ordered", C.byref(net), C.c_void_p(Xt.data_ptr()), C.c_void_p(T.data_ptr()),
              C.c_void_p(mlp.out_w.data_ptr()), B, C.byref(s), C.byref(grads), C.c_void_p(loss.data_ptr()),
-             C.c_void_p(mlp.status.data_ptr()), st())
+             C.c_void_p(work.data_ptr()), work.numel(), C.c_void_p(mlp.status.data_ptr()), st())
 
     # layer 1's GEMM alone: X W1^T into fp32 (the forward adds the bias / ReLU / bf16 epilogue)
     def layer1():
