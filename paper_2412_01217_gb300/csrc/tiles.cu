@@ -624,8 +624,13 @@ __global__ void __launch_bounds__(kScanThreads, 6) cull_kernel(
                 }
             }
         }
-        // the next chunk starts in the record that owns this chunk's last slot
-        if (threadIdx.x == kScanThreads - 1) s_next = ic + k;
+        // the next chunk starts in the record that owns this chunk's last slot, or in the one after
+        // if that ends here (its prefix is not staged when the 256 slots have 256 owners)
+        if (threadIdx.x == kScanThreads - 1) {
+            const int e = ic + k + 1;
+            const uint32_t after = k + 1 < kScanThreads ? s_P[k + 1] : e < n ? P[e] : 0xffffffffu;
+            s_next = after <= c0 + kScanThreads ? e : e - 1;
+        }
         return cnt;
     };
     // the chunk's instances [run, run + tot)
