@@ -822,16 +822,19 @@ __global__ void __maxnreg__((bwd_max_regs<C>())) raster_bwd_kernel(RasterArgs a)
                     for (int i = 3; i >= 0; --i) {
                         float *gw = s_gw + (4 * q + i) * WQ + lane;
                         const float A = pos[i] < my_last ? a4[i] : 0.f, om = 1.f - A;
-                        // (a pixel without a contribution keeps T and a: A = 0, gf taken as 0)
-                        const float gf = A > 0.f ? *gw : 0.f;
-                        if (A > 0.f) hb |= 1u << i;
+                        // (a pixel without a contribution keeps T and a: A = 0, gf taken as 0;
+                        // w and s are 0 there even if T or a is not finite, which would reach every
+                        // row's sums over the warp's pixels)
+                        const bool on = A > 0.f;
+                        const float gf = on ? *gw : 0.f;
+                        if (on) hb |= 1u << i;
                         // transmittance before this Gaussian (only gradients depend on it)
                         T *= rcp_fast(om);
                         const float dalpha = T * (gf - acc_a);
                         acc_a = fmaf(om, acc_a, A * gf);
-                        *gw = A * T;
+                        *gw = on ? A * T : 0.f;
                         // (alpha = alpha_max: clamped, no gradient; else alpha = o G)
-                        s_sg[(4 * q + i) * WQ + lane] = A < a.alpha_max ? -dalpha * A : 0.f;
+                        s_sg[(4 * q + i) * WQ + lane] = on && A < a.alpha_max ? -dalpha * A : 0.f;
                     }
                     hits |= hb << (4 * q);
                 }
