@@ -51,7 +51,8 @@ typedef enum {
 #define SG_STATUS_CAPACITY 1u /* more tile instances than sg_tile_lists.capacity  */
 #define SG_STATUS_NUMERIC 2u  /* non-finite value met (checks on: sg_config /
                                  sg_loss_config check_numeric, sg_adam_multi status) */
-#define SG_STATUS_TIMEOUT 4u  /* a bounded wait inside a tensor-core kernel gave up */
+#define SG_STATUS_TIMEOUT 4u  /* a bounded wait inside a tensor-core kernel or the list
+                                 build gave up */
 
 #define SG_MAX_VIEWS 64
 
@@ -284,11 +285,23 @@ size_t sg_tile_lists_workspace_size(int64_t n_records, int32_t capacity);
  * deterministic radix sort), plus each tile's [start, end) and (with lists->half_masks)
  * each instance's half mask.  n_tiles: total tiles of the views (sg_make_views); with half
  * masks N * n_views must be below 2^30.  If more than capacity instances arise, the surplus
- * is dropped, *count holds the required number and SG_STATUS_CAPACITY is set in *status. */
+ * is dropped, *count holds the required number and SG_STATUS_CAPACITY is set in *status.  The
+ * kernels' blocks wait for one another's counts, each wait bounded (some seconds): should one give
+ * up, SG_STATUS_TIMEOUT is set, *count is 0 and every tile's list is empty. */
 sg_status sg_build_tile_lists(const sg_projected *proj, int32_t N, int32_t n_views,
                               const sg_view *views, int32_t n_tiles, const sg_config *cfg,
                               sg_tile_lists *lists, void *workspace, size_t workspace_bytes,
                               uint32_t *status, sg_stream_t stream);
+
+/* Self-test of that failure detection: sg_build_tile_lists with at most `polls` polls (1..2^20) per
+ * wait, in which the first part of step `step` publishes nothing, so that the waits of its other
+ * parts run out.  Steps: 0 compaction, 1..4 depth passes, 5 slots, 6 culling, 7..10 tile passes,
+ * 11 work order (whose parts then count for themselves: only the status shows it). */
+sg_status sg_tile_lists_timeout_probe(const sg_projected *proj, int32_t N, int32_t n_views,
+                                      const sg_view *views, int32_t n_tiles, const sg_config *cfg,
+                                      sg_tile_lists *lists, void *workspace, size_t workspace_bytes,
+                                      int32_t step, uint32_t polls, uint32_t *status,
+                                      sg_stream_t stream);
 
 /* Eq. 7-9 for every view-level in one launch: per tile, front-to-back compositing of RGB,
  * depth and C semantic channels.  work_counter: 2 int32 of device scratch for the persistent

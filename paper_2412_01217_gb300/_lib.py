@@ -110,6 +110,8 @@ SIGNATURES = {
     "sg_tile_lists_workspace_size": (C.c_size_t, [C.c_int64, c_i]),
     "sg_build_tile_lists": (c_i, [P(SgProjected), c_i, c_i, c_p, c_i, P(SgConfig), P(SgTileLists),
                                   c_p, C.c_size_t, c_p, c_p]),
+    "sg_tile_lists_timeout_probe": (c_i, [P(SgProjected), c_i, c_i, c_p, c_i, P(SgConfig), P(SgTileLists),
+                                          c_p, C.c_size_t, c_i, C.c_uint32, c_p, c_p]),
     "sg_render_pyramid": (c_i, [P(SgGaussians), P(SgProjected), P(SgTileLists), c_p, c_i, c_i,
                                 P(SgConfig), P(SgImages), P(SgSaved), c_p, c_p]),
     "sg_loss_workspace_size": (C.c_size_t, [P(SgView), c_i, c_i, c_i]),

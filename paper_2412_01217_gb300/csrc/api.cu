@@ -36,7 +36,8 @@ sg_status launch_project_bwd(const sg_gaussians *, const sg_view *, int, const s
                              const sg_projected *, float *, sg_gaussian_grads *, cudaStream_t);
 size_t tile_lists_workspace_size(int64_t R, int32_t cap);
 sg_status launch_build_tile_lists(const sg_projected *, int, int, const sg_view *, int, int, int,
-                                  sg_tile_lists *, void *, size_t, uint32_t *, cudaStream_t);
+                                  sg_tile_lists *, void *, size_t, uint32_t *, cudaStream_t,
+                                  int withheld_step = -1, uint32_t polls = 0);
 size_t loss_workspace_size(const sg_view *vh, int n_views, int C, int n_classes);
 sg_status launch_loss(const sg_images *, const sg_targets *, const sg_view *, const sg_view *, int,
                       int, const sg_loss_config *, float *, sg_images *, void *, size_t, uint32_t *,
@@ -281,10 +282,9 @@ size_t sg_tile_lists_workspace_size(int64_t n_records, int32_t capacity) {
     return tile_lists_workspace_size(n_records, capacity);
 }
 
-sg_status sg_build_tile_lists(const sg_projected *proj, int32_t N, int32_t n_views,
-                              const sg_view *views, int32_t n_tiles, const sg_config *cfg,
-                              sg_tile_lists *lists, void *workspace, size_t workspace_bytes,
-                              uint32_t *status, sg_stream_t stream) {
+static sg_status check_tile_lists(const sg_projected *proj, int32_t N, int32_t n_views, const sg_view *views,
+                                  int32_t n_tiles, const sg_config *cfg, const sg_tile_lists *lists,
+                                  const void *workspace, const uint32_t *status) {
     SG_REQUIRE(proj && proj->geo && proj->rect && proj->ext, "projected buffers are NULL");
     SG_TRY(check_cfg(cfg));
     SG_TRY(check_views(views, n_views));
@@ -295,9 +295,28 @@ sg_status sg_build_tile_lists(const sg_projected *proj, int32_t N, int32_t n_vie
     SG_REQUIRE(lists->capacity >= 1, "capacity must be >= 1");
     SG_REQUIRE(workspace && status, "workspace/status is NULL");
     SG_REQUIRE(aligned16(workspace), "workspace must be 16-byte aligned");
+    return SG_OK;
+}
+
+sg_status sg_build_tile_lists(const sg_projected *proj, int32_t N, int32_t n_views,
+                              const sg_view *views, int32_t n_tiles, const sg_config *cfg,
+                              sg_tile_lists *lists, void *workspace, size_t workspace_bytes,
+                              uint32_t *status, sg_stream_t stream) {
+    SG_TRY(check_tile_lists(proj, N, n_views, views, n_tiles, cfg, lists, workspace, status));
     return launch_build_tile_lists(proj, N, n_views, views, n_tiles, cfg->tile_w, cfg->tile_h, lists, workspace,
                                    workspace_bytes,
                                    status, (cudaStream_t)stream);
+}
+
+sg_status sg_tile_lists_timeout_probe(const sg_projected *proj, int32_t N, int32_t n_views,
+                                      const sg_view *views, int32_t n_tiles, const sg_config *cfg,
+                                      sg_tile_lists *lists, void *workspace, size_t workspace_bytes,
+                                      int32_t step, uint32_t polls, uint32_t *status, sg_stream_t stream) {
+    SG_TRY(check_tile_lists(proj, N, n_views, views, n_tiles, cfg, lists, workspace, status));
+    SG_REQUIRE(step >= 0 && step < 12, "timeout probe: step %d not in 0..11", step);
+    SG_REQUIRE(polls >= 1 && polls <= (1u << 20), "timeout probe: polls must be in [1, 2^20]");
+    return launch_build_tile_lists(proj, N, n_views, views, n_tiles, cfg->tile_w, cfg->tile_h, lists, workspace,
+                                   workspace_bytes, status, (cudaStream_t)stream, step, polls);
 }
 
 sg_status sg_render_pyramid(const sg_gaussians *g, const sg_projected *proj,

@@ -24,7 +24,9 @@
 // number from a counter, publishes the part's aggregate, sums its predecessors' published
 // words back to the nearest one that already holds an inclusive prefix, and publishes its own.
 // Parts are drawn in order, so the predecessors of a part are held by blocks that already run;
-// every wait is bounded all the same (SG_STATUS_TIMEOUT).  The steps were three kernels each
+// every wait is bounded all the same (SG_STATUS_TIMEOUT), and a step whose predecessor gave up
+// takes its input as empty: what the failed step left behind (places never written) is not read,
+// and the lists come out empty.  The steps were three kernels each
 // before (count, scan of the counts, apply): 33 launches per list build, now 12 or 13 and one
 // memset, and the keys and footprints are read once instead of twice.  What that gives is
 // the launches and their latencies (320x180 x 3 levels with 30k Gaussians: 110 -> 70 us of
@@ -85,6 +87,27 @@ constexpr uint64_t kAggregate = 1ull << 32;  // value: the part's own sum
 constexpr uint64_t kPrefix = 1ull << 33;     // value: inclusive prefix through the part
 constexpr uint32_t kSpinLimit = 1u << 22;
 
+// A step's bounded waits.  polls: limit of each; before, own: flags of the step before (null for
+// the first) and of this one, set once a wait has given up.  withhold (self-test): part 0
+// publishes nothing, so that every wait for it runs out.
+struct StepWaits {
+    uint32_t *status;
+    const int *before;
+    int *own;
+    uint32_t polls;
+    int withhold;
+    __device__ __forceinline__ void gave_up() const {
+        atomicOr(status, SG_STATUS_TIMEOUT);
+        *own = 1;
+    }
+    // Whether an earlier step gave up (uniform over the grid: their kernels are done).
+    __device__ __forceinline__ bool broken() const {
+        if (!before || !*before) return false;
+        *own = 1;
+        return true;
+    }
+};
+
 __device__ __forceinline__ uint64_t load_word(const uint64_t *p) {
     uint64_t v;
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];\n" : "=l"(v) : "l"(p) : "memory");
@@ -94,11 +117,11 @@ __device__ __forceinline__ void store_word(uint64_t *p, uint64_t v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;\n" ::"l"(p), "l"(v) : "memory");
 }
 
-// The word of an earlier part, once published; on a timeout (status flagged) an empty prefix.
-__device__ __forceinline__ uint64_t wait_word(const uint64_t *p, uint64_t w, uint32_t *status) {
+// The word of an earlier part, once published; on a timeout an empty prefix.
+__device__ __forceinline__ uint64_t wait_word(const uint64_t *p, uint64_t w, const StepWaits &sw) {
     for (uint32_t polls = 0; !(w >> 32); ++polls) {
-        if (polls >= kSpinLimit) {
-            atomicOr(status, SG_STATUS_TIMEOUT);
+        if (polls >= sw.polls) {
+            sw.gave_up();
             return kPrefix;
         }
         w = load_word(p);
@@ -109,17 +132,17 @@ __device__ __forceinline__ uint64_t wait_word(const uint64_t *p, uint64_t w, uin
 // Exclusive prefix of the part whose sum is `own`, for a whole block (every thread gets it);
 // publishes the part's words.  256 predecessors are examined at a time: with several hundred
 // parts in flight most of them hold only their own sum yet.
-__device__ __forceinline__ uint32_t block_look_back(uint64_t *words, int part, uint32_t own, uint32_t *status) {
+__device__ __forceinline__ uint32_t block_look_back(uint64_t *words, int part, uint32_t own, const StepWaits &sw) {
     __shared__ uint32_t s_sum[kScanThreads / 32];
     __shared__ bool s_has[kScanThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) store_word(words + part, (part == 0 ? kPrefix : kAggregate) | own);
+    if (threadIdx.x == 0 && !(sw.withhold && part == 0)) store_word(words + part, (part == 0 ? kPrefix : kAggregate) | own);
     uint32_t sum = 0;
     bool found = part == 0;
     for (int p = part - 1; !found; p -= kScanThreads) {  // (block-uniform)
         const int q = p - (int)threadIdx.x;
         uint64_t w = kPrefix;  // before the first part: an empty prefix
-        if (q >= 0) w = wait_word(words + q, load_word(words + q), status);
+        if (q >= 0) w = wait_word(words + q, load_word(words + q), sw);
         const uint32_t pre = __ballot_sync(SG_FULL_MASK, (w & kPrefix) != 0);
         // lanes past the nearest prefix do not count
         const int stop = pre ? __ffs(pre) - 1 : 31;
@@ -143,9 +166,10 @@ __device__ __forceinline__ uint32_t block_look_back(uint64_t *words, int part, u
 // thread's sum has been published in words[part * stride]; four predecessors' words are
 // requested at a time.  Called by whole warps, and the warp stays together: the waits and the
 // loop end for all lanes at once (inactive lanes sum nothing), so that no lane runs ahead to the
-// caller's block barrier while others still look back.
+// caller's block barrier while others still look back.  late: set when a wait gave up (for all
+// lanes of the warp).
 __device__ __forceinline__ uint32_t look_back(const uint64_t *words, int stride, int part, bool active,
-                                              uint32_t *status) {
+                                              const StepWaits &sw, bool &late) {
     uint32_t sum = 0;
     bool done = !active;
     for (int p = part - 1; p >= 0 && !__all_sync(SG_FULL_MASK, done); p -= 4) {
@@ -157,8 +181,9 @@ __device__ __forceinline__ uint32_t look_back(const uint64_t *words, int stride,
 #pragma unroll
             for (int i = 0; i < 4; ++i) missing |= !(w[i] >> 32);
             if (!__any_sync(SG_FULL_MASK, missing)) break;
-            if (polls >= kSpinLimit) {  // (warp-uniform)
-                if (missing) atomicOr(status, SG_STATUS_TIMEOUT);
+            if (polls >= sw.polls) {  // (warp-uniform)
+                if (missing) sw.gave_up();
+                late = true;
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
                     if (!(w[i] >> 32)) w[i] = kPrefix;
@@ -216,8 +241,7 @@ __global__ void __launch_bounds__(kScanThreads) compact_kernel(const uint2 *__re
                                                                uint64_t *__restrict__ words, int *__restrict__ counter,
                                                                uint32_t *__restrict__ key, uint32_t *__restrict__ val,
                                                                int *__restrict__ total, uint32_t *__restrict__ hist,
-                                                               int *__restrict__ instances,
-                                                               uint32_t *__restrict__ status) {
+                                                               int *__restrict__ instances, StepWaits sw) {
     pdl_begin();
     constexpr int E = kCompactPerThread;
     __shared__ uint32_t s_h[4 * 256];
@@ -262,7 +286,7 @@ __global__ void __launch_bounds__(kScanThreads) compact_kernel(const uint2 *__re
                 s_val[o] = (uint32_t)(i0 + q);
                 ++o;
             }
-        const uint32_t off = block_look_back(words, part, tot, status);
+        const uint32_t off = block_look_back(words, part, tot, sw);
         if (part == parts - 1 && threadIdx.x == 0) *total = (int)(off + tot);
         __syncthreads();
         for (uint32_t j = threadIdx.x; j < ((tot + 31) & ~31u); j += kScanThreads) {
@@ -468,10 +492,10 @@ __global__ void __launch_bounds__(kScanThreads) slot_prefix_kernel(const uint2 *
                                                                    uint64_t *__restrict__ words, int *__restrict__ counter,
                                                                    uint32_t *__restrict__ P,
                                                                    uint32_t *__restrict__ first_rec,
-                                                                   int *__restrict__ total, uint32_t *__restrict__ status) {
+                                                                   int *__restrict__ total, StepWaits sw) {
     pdl_begin();
     constexpr int E = kCompactPerThread;
-    const int n = *m_ptr;
+    const int n = sw.broken() ? 0 : *m_ptr;
     const int parts = (n + kCompactPart - 1) / kCompactPart;
     for (int part; (part = next_part(counter)) < parts;) {
         // thread t takes records base + 32 (8 warp + q) + lane: coalesced loads, and the scan runs
@@ -496,7 +520,7 @@ __global__ void __launch_bounds__(kScanThreads) slot_prefix_kernel(const uint2 *
         }
         uint32_t tot;
         const uint32_t ex = block_exclusive_scan(lane == 0 ? sum : 0u, tot);
-        const uint32_t off = block_look_back(words, part, tot, status) + __shfl_sync(SG_FULL_MASK, ex, 0);
+        const uint32_t off = block_look_back(words, part, tot, sw) + __shfl_sync(SG_FULL_MASK, ex, 0);
         if (part == parts - 1 && threadIdx.x == 0) *total = (int)(off + tot);
 #pragma unroll
         for (int q = 0; q < E; ++q) {
@@ -551,7 +575,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) cull_kernel(
     int *__restrict__ counter, int N, const sg_view *__restrict__ views, int n_views, int tile_w, int tile_h,
     uint32_t *__restrict__ tkey, uint32_t *__restrict__ tval, int capacity, int *__restrict__ total, Digits dg,
     uint32_t *__restrict__ hist, uint64_t *__restrict__ sweep_words, int sweep_part, uint32_t *__restrict__ slot_tf,
-    uint32_t *__restrict__ slot_cnt, uint32_t *__restrict__ slot_half, uint32_t *__restrict__ status) {
+    uint32_t *__restrict__ slot_cnt, uint32_t *__restrict__ slot_half, StepWaits sw) {
     pdl_begin();
     __shared__ uint32_t s_P[kScanThreads], s_ex[kScanThreads], s_tf[kScanThreads], s_or[kScanThreads],
         s_hf[HALVES ? kScanThreads : 1];
@@ -561,8 +585,9 @@ __global__ void __launch_bounds__(kScanThreads, 6) cull_kernel(
     for (int v = threadIdx.x; v < n_views; v += kScanThreads)
         s_vw[v] = make_int4(views[v].W, views[v].H, views[v].tile_offset, views[v].tiles_x);
     for (int i = threadIdx.x; i < 4 * 256; i += kScanThreads) s_h[i] = 0;
-    const int n = *m_ptr;
-    const uint32_t S = (uint32_t)*s_ptr;
+    const bool broken = sw.broken();
+    const int n = broken ? 0 : *m_ptr;
+    const uint32_t S = broken ? 0u : (uint32_t)*s_ptr;
     const int chunks = (int)(((uint64_t)S + 255) / 256);
     // chunks of a part: at most two parts per block, one chunk for small inputs
     const int per = max(1, max((chunks + kMaxChunks - 1) / kMaxChunks, (chunks + 2 * (int)gridDim.x - 1) / (2 * (int)gridDim.x)));
@@ -682,7 +707,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) cull_kernel(
         if (per == 1) {
             const uint32_t cnt = slot((uint64_t)b0 * 256, i0, k, orec, tfirst, half, false, false);
             const uint32_t ex = block_exclusive_scan(cnt, tot);
-            run = block_look_back(words, part, tot, status);
+            run = block_look_back(words, part, tot, sw);
             sum = tot;
             emit(run, ex, cnt, tot, orec, tfirst, half);
         } else {
@@ -694,7 +719,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) cull_kernel(
                 ic = s_next;
             }
             block_exclusive_scan(kept, sum);
-            run = block_look_back(words, part, sum, status);
+            run = block_look_back(words, part, sum, sw);
             ic = i0;
             uint32_t at = run;
             for (int b = b0; b < b1; ++b) {
@@ -711,7 +736,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) cull_kernel(
             sweep_words[q * 256 + threadIdx.x] = 0;
     }
     flush_hist(s_h, 256 * dg.n, hist);
-    if (overflow) atomicOr(status, SG_STATUS_CAPACITY);
+    if (overflow) atomicOr(sw.status, SG_STATUS_CAPACITY);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -732,7 +757,7 @@ __global__ void __launch_bounds__(kScanThreads, 4) sweep_kernel(
     const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin, uint32_t *__restrict__ kout,
     uint32_t *__restrict__ vout, const int *__restrict__ n_ptr, int cap, int shift, uint32_t mask,
     const uint32_t *__restrict__ hist, uint64_t *__restrict__ words, uint64_t *__restrict__ clear,
-    int *__restrict__ counter, uint32_t *__restrict__ status) {
+    int *__restrict__ counter, StepWaits sw) {
     pdl_begin();
     constexpr int kWarps = kScanThreads / 32, IPT = kSweepIpt, CH = kSweepPart;
     __shared__ uint32_t to[256];            // output position of the part's slot 0 if it had digit d
@@ -740,7 +765,7 @@ __global__ void __launch_bounds__(kScanThreads, 4) sweep_kernel(
     __shared__ uint32_t wcnt[kWarps][256];  // per-warp digit counts, then per-warp offsets
     __shared__ uint32_t skey[CH], sval[CH];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n = min(*n_ptr, cap);
+    const int n = sw.broken() ? 0 : min(*n_ptr, cap);
     const int parts = (int)(((int64_t)n + CH - 1) / CH);
     uint32_t unused;
     const uint32_t first = block_exclusive_scan(hist[tid], unused);  // digit tid's first output position
@@ -783,7 +808,7 @@ __global__ void __launch_bounds__(kScanThreads, 4) sweep_kernel(
         }
         uint64_t *word = words + (size_t)part * 256 + tid;
         const bool digit = tid <= (int)mask;  // (the other threads' counts are 0)
-        if (digit) store_word(word, (part == 0 ? kPrefix : kAggregate) | cnt);
+        if (digit && !(sw.withhold && part == 0)) store_word(word, (part == 0 ? kPrefix : kAggregate) | cnt);
         const uint32_t slot0 = block_exclusive_scan(cnt, unused);
         loc[tid] = slot0;
         __syncthreads();
@@ -798,7 +823,8 @@ __global__ void __launch_bounds__(kScanThreads, 4) sweep_kernel(
         }
         uint32_t before = 0;
         if (part > 0 && (tid & ~31) <= (int)mask) {  // (warp-uniform)
-            before = look_back(words + tid, 256, part, digit, status);
+            bool late = false;
+            before = look_back(words + tid, 256, part, digit, sw, late);
             if (digit) store_word(word, kPrefix | (uint64_t)(before + cnt));
             __syncwarp();
         }
@@ -834,17 +860,17 @@ static Digits split_digits(int bits, int max_bits) {
 // (kout, vout) using (ktmp, vtmp) as ping-pong; kin/vin are not modified.  hist: the digits'
 // histograms (256 words each); words[0]: the first pass's chained-scan words, cleared for every
 // part; words[1]: the second pass's (the passes alternate between the two and each clears its
-// successor's); counters: one per pass, zero.
+// successor's); counters: one per pass, zero; waits: one per pass.
 static void radix_sort(const uint32_t *kin, const uint32_t *vin, uint32_t *kout, uint32_t *vout, uint32_t *ktmp,
                        uint32_t *vtmp, const int *n_ptr, int cap, const Digits &dg, const uint32_t *hist,
-                       uint64_t *const words[2], int *counters, int grid, uint32_t *status, cudaStream_t st) {
+                       uint64_t *const words[2], int *counters, int grid, const StepWaits *waits, cudaStream_t st) {
     const uint32_t *ks = kin, *vs = vin;
     for (int p = 0; p < dg.n; ++p) {
         uint32_t *kd = ((dg.n - 1 - p) % 2 == 0) ? kout : ktmp;
         uint32_t *vd = ((dg.n - 1 - p) % 2 == 0) ? vout : vtmp;
         launch_pdl(sweep_kernel, grid, kScanThreads, 0, st, ks, vs, kd, vd, n_ptr, cap, dg.shift[p], dg.mask[p],
                    hist + 256 * p, words[p & 1], p + 1 < dg.n ? words[(p + 1) & 1] : (uint64_t *)nullptr, counters + p,
-                   status);
+                   waits[p]);
         count_launches(1);
         ks = kd;
         vs = vd;
@@ -892,15 +918,19 @@ __device__ __forceinline__ uint32_t length_bucket(int2 r) {
 
 // [start, end) of every tile by search in the sorted tile ids ((0, 0) for a tile with no
 // instance): one warp per 32 tiles finds its first and its last bound together, then each lane
-// its own bound in between.  hist (or null): counts of the length buckets.
+// its own bound in between.  hist (or null): counts of the length buckets.  *failed: the last
+// step's flag.
 __global__ void __launch_bounds__(kScanThreads) ranges_kernel(const uint32_t *__restrict__ tile,
-                                                              const int *__restrict__ k_ptr, int cap, int n_tiles,
-                                                              int2 *__restrict__ ranges, uint32_t *__restrict__ hist) {
+                                                              int *__restrict__ k_ptr, int cap, int n_tiles,
+                                                              int2 *__restrict__ ranges, uint32_t *__restrict__ hist,
+                                                              const int *__restrict__ failed) {
     pdl_begin();
+    const bool broken = *failed != 0;  // (a step gave up: no instances)
+    if (broken && blockIdx.x == 0 && threadIdx.x == 0) *k_ptr = 0;
     __shared__ uint32_t s_h[64];
     if (threadIdx.x < 64) s_h[threadIdx.x] = 0;
     __syncthreads();
-    const int K = min(*k_ptr, cap), lane = threadIdx.x & 31;
+    const int K = broken ? 0 : min(*k_ptr, cap), lane = threadIdx.x & 31;
     const int t = blockIdx.x * kScanThreads + (int)threadIdx.x, t0 = t - lane;
     if (t0 < n_tiles) {  // (warp-uniform)
         const int wlo = warp_lower_bound_u32(tile, K, (uint32_t)t0);
@@ -919,11 +949,12 @@ __global__ void __launch_bounds__(kScanThreads) ranges_kernel(const uint32_t *__
 
 // The work order: a stable counting sort of the tiles by length bucket.  A block's part is a
 // contiguous range of tiles (grid parts, 256 tiles at a time), counted, placed by the chained
-// scan (64 words per part) and written.
+// scan (64 words per part) and written.  A part whose wait gives up counts the tiles before it
+// itself, so that the order always holds every tile.
 __global__ void __launch_bounds__(kScanThreads) order_kernel(const int2 *__restrict__ ranges, int n_tiles,
                                                              const uint32_t *__restrict__ hist,
                                                              uint64_t *__restrict__ words, int *__restrict__ counter,
-                                                             int *__restrict__ order, uint32_t *__restrict__ status) {
+                                                             int *__restrict__ order, StepWaits sw) {
     pdl_begin();
     constexpr int kWarps = kScanThreads / 32;
     __shared__ uint32_t s_cnt[64], s_run[64], s_w[kWarps][64];
@@ -940,10 +971,15 @@ __global__ void __launch_bounds__(kScanThreads) order_kernel(const int2 *__restr
     __syncthreads();
     if (tid < 64) {
         uint64_t *word = words + (size_t)part * 64 + tid;
-        store_word(word, (part == 0 ? kPrefix : kAggregate) | s_cnt[tid]);
+        if (!(sw.withhold && part == 0)) store_word(word, (part == 0 ? kPrefix : kAggregate) | s_cnt[tid]);
         uint32_t before = 0;
         if (part > 0) {
-            before = look_back(words + tid, 64, part, true, status);
+            bool late = false;
+            before = look_back(words + tid, 64, part, true, sw, late);
+            if (late) {
+                before = 0;
+                for (int64_t i = 0; i < beg; ++i) before += length_bucket(ranges[i]) == (uint32_t)tid;
+            }
             store_word(word, kPrefix | (uint64_t)(before + s_cnt[tid]));
         }
         s_run[tid] = first + before;
@@ -971,7 +1007,7 @@ __global__ void __launch_bounds__(kScanThreads) order_kernel(const int2 *__restr
         __syncthreads();
         if (d < 64u) {
             const uint32_t pos = s_w[warp][d] + below;
-            if (pos < (uint32_t)n_tiles) order[pos] = (int)i;  // (beyond only after a timeout)
+            order[pos] = (int)i;
         }
         __syncthreads();
     }
@@ -981,7 +1017,7 @@ __global__ void __launch_bounds__(kScanThreads) order_kernel(const int2 *__restr
 // Workspace layout
 // ---------------------------------------------------------------------------------------
 
-// Chained-scan part counters (one per kernel of a list build).
+// Steps of a list build: its kernels with a chained scan (each has a part counter and a flag).
 enum { kCtrCompact = 0, kCtrDepth = 1, kCtrSlots = 5, kCtrCull = 6, kCtrTile = 7, kCtrOrder = 11, kCtrs = 12 };
 
 struct TileWorkspace {
@@ -994,6 +1030,7 @@ struct TileWorkspace {
     size_t zero_bytes;
     int *counts;    // [0] visible records M, [1] slots S
     int *counters;  // kCtrs part counters
+    int *failed;    // kCtrs flags of steps that gave up
     uint32_t *dhist, *thist, *ohist;                      // 4 x 256, 4 x 256, 64
     uint64_t *cwords, *swords, *kwords, *owords;  // chained-scan words: compaction, slots, culling, order
     uint64_t *sweep[2];  // radix passes: [0] is cleared for the depth sort's parts
@@ -1041,6 +1078,7 @@ static size_t tile_ws_layout(int64_t R, int32_t cap, int G, TileWorkspace *ws, c
     w.zero = take(0);
     w.counts = (int *)take(4 * sizeof(int));
     w.counters = (int *)take(kCtrs * sizeof(int));
+    w.failed = (int *)take(kCtrs * sizeof(int));
     w.dhist = (uint32_t *)take(4 * 256 * 4);
     w.thist = (uint32_t *)take(4 * 256 * 4);
     w.ohist = (uint32_t *)take(64 * 4);
@@ -1063,7 +1101,7 @@ size_t tile_lists_workspace_size(int64_t R, int32_t cap) {
 sg_status launch_build_tile_lists(const sg_projected *proj, int N, int n_views,
                                   const sg_view *views, int n_tiles, int tile_w, int tile_h, sg_tile_lists *lists,
                                   void *workspace, size_t ws_bytes, uint32_t *status,
-                                  cudaStream_t st) {
+                                  cudaStream_t st, int withheld_step, uint32_t polls) {
     const int G = sort_grid();
     const int64_t R = (int64_t)N * n_views;
     TileWorkspace w;
@@ -1076,18 +1114,22 @@ sg_status launch_build_tile_lists(const sg_projected *proj, int N, int n_views,
     const float4 *geo = reinterpret_cast<const float4 *>(proj->geo);
     const float2 *ext = reinterpret_cast<const float2 *>(proj->ext);
     auto grid = [G](int64_t parts) { return (int)std::max<int64_t>(1, std::min<int64_t>(G, parts)); };
+    if (!polls) polls = kSpinLimit;
+    StepWaits waits[kCtrs];
+    for (int k = 0; k < kCtrs; ++k)
+        waits[k] = {status, k ? w.failed + k - 1 : nullptr, w.failed + k, polls, k == withheld_step};
     cudaMemsetAsync(w.zero, 0, w.zero_bytes, st);
     // 1. compaction of the visible records (count -> counts[0])
     const int cgrid = grid((R + kCompactPart - 1) / kCompactPart);
     launch_pdl(compact_kernel, cgrid, kScanThreads, 0, st, rect, geo, (int)R, w.cwords, w.counters + kCtrCompact,
-               w.dkey_in, w.dval_in, w.counts, w.dhist, lists->count, status);
+               w.dkey_in, w.dval_in, w.counts, w.dhist, lists->count, waits[kCtrCompact]);
     // 2. depth sort (32 bits)
     radix_sort(w.dkey_in, w.dval_in, w.dkey_out, w.dval_out, w.dkey_tmp, w.dval_tmp, w.counts, (int)R,
-               split_digits(32, 8), w.dhist, w.sweep, w.counters + kCtrDepth, grid(sweep_parts(R)), status, st);
+               split_digits(32, 8), w.dhist, w.sweep, w.counters + kCtrDepth, grid(sweep_parts(R)), waits + kCtrDepth, st);
     // 3. slots: the rectangle tile rows of the records in depth order (their number ->
     // counts[1]); culling and emission (K -> lists->count)
     launch_pdl(slot_prefix_kernel, cgrid, kScanThreads, 0, st, rect, w.dval_out, w.counts, w.swords,
-               w.counters + kCtrSlots, w.slot0, w.first_rec, w.counts + 1, status);
+               w.counters + kCtrSlots, w.slot0, w.first_rec, w.counts + 1, waits[kCtrSlots]);
     int bits = 1;
     while ((1ll << bits) < (long long)n_tiles) ++bits;
     const Digits dg = split_digits(bits, kTileDigitBits);
@@ -1095,20 +1137,20 @@ sg_status launch_build_tile_lists(const sg_projected *proj, int N, int n_views,
     launch_pdl(halves ? cull_kernel<true> : cull_kernel<false>, G + G / 2, kScanThreads, 0, st, rect, geo, ext, w.dval_out,
                w.counts, w.counts + 1, w.slot0, w.first_rec, w.kwords, w.counters + kCtrCull, N, views, n_views, tile_w,
                tile_h, w.tkey_in, w.tval_in, lists->capacity, lists->count, dg, w.thist, w.sweep[0], kSweepPart, w.tkey_tmp, w.tval_tmp,
-               lists->tile, status);
+               lists->tile, waits[kCtrCull]);
     // 4. stable sort by tile id
     radix_sort(w.tkey_in, w.tval_in, lists->tile, lists->record, w.tkey_tmp, w.tval_tmp, lists->count,
-               lists->capacity, dg, w.thist, w.sweep, w.counters + kCtrTile, grid(sweep_parts(lists->capacity)), status,
-               st);
+               lists->capacity, dg, w.thist, w.sweep, w.counters + kCtrTile, grid(sweep_parts(lists->capacity)),
+               waits + kCtrTile, st);
     // 5. tile ranges; 6. work order
     int2 *ranges = reinterpret_cast<int2 *>(lists->ranges);
     const int tblocks = (int)(((int64_t)n_tiles + kScanThreads - 1) / kScanThreads);
     launch_pdl(ranges_kernel, tblocks, kScanThreads, 0, st, lists->tile, lists->count, lists->capacity, n_tiles, ranges,
-               lists->order ? w.ohist : (uint32_t *)nullptr);
+               lists->order ? w.ohist : (uint32_t *)nullptr, w.failed + kCtrTile + dg.n - 1);
     count_launches(4);  // compaction, slots, culling, ranges
     if (lists->order) {
         launch_pdl(order_kernel, std::min(G, tblocks), kScanThreads, 0, st, ranges, n_tiles, w.ohist,
-                   w.owords, w.counters + kCtrOrder, lists->order, status);
+                   w.owords, w.counters + kCtrOrder, lists->order, waits[kCtrOrder]);
         count_launches(1);
     }
     return check_launch("build_tile_lists");

@@ -182,3 +182,20 @@ def test_loss_workspace_must_be_16_byte_aligned():
     assert lib.sg_pyramid_loss(C.byref(imgs), C.byref(gt), views, views, 1, 8, C.byref(lc), a, C.byref(dl),
                                base + 4, 128, None, None) == 1
     assert b"16-byte" in lib.sg_last_error()
+
+
+def test_tile_list_timeout_probe_validates_on_the_host():
+    from paper_2412_01217_gb300 import _lib
+    lib = _lib.load()
+    cfg, proj, lists = _lib.SgConfig(), _lib.SgProjected(), _lib.SgTileLists()
+    lib.sg_default_config(C.byref(cfg))
+    buf = (C.c_uint32 * 1024)()
+    at = C.addressof(buf) + (-C.addressof(buf)) % 16
+    proj.geo = proj.rect = proj.ext = lists.tile = lists.record = lists.ranges = lists.count = at
+    lists.capacity = 1
+    probe = lambda step, polls, ws=at: lib.sg_tile_lists_timeout_probe(
+        C.byref(proj), 1, 1, at, 1, C.byref(cfg), C.byref(lists), ws, 16, step, polls, at, None)
+    assert probe(-1, 10) == 1 and probe(12, 10) == 1
+    assert probe(0, 0) == 1 and probe(0, (1 << 20) + 1) == 1
+    assert probe(0, 10, None) == 1
+    assert probe(0, 10) == 2  # workspace of 16 bytes: too small
