@@ -965,15 +965,16 @@ struct PairSum {
         add(h);
         lo += l;
     }
-    // (an infinite sum has no error term)
-    __device__ __forceinline__ double value() const { return isinf(hi) ? (double)hi : (double)hi + (double)lo; }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
 // A view's partial sums and its loss terms by a cluster of kFinalCtas CTAs, their shares added
 // in rank order through distributed shared memory.  Bound by the latency of the partials'
 // loads; the sums over a CTA are pairs of floats, because an SM does only a few double additions
 // per clock (12.7 us with doubles, 637x477 x 3 levels 9.7 -> 7.2): 1200x680 x 3 levels with
-// one CTA per view took 38 us (25 us less of the loss with a 32-class decoder).
+// one CTA per view took 38 us (25 us less of the loss with a 32-class decoder).  A warp whose pairs
+// leave the range of a float (sums beyond it, or a partial that is not finite) sums again in
+// double.
 constexpr int kFinalCtas = 8;
 __global__ void __cluster_dims__(kFinalCtas, 1, 1) __launch_bounds__(kLossThreads) loss_finalize_kernel(FinalArgs a) {
     pdl_begin();
@@ -984,19 +985,19 @@ __global__ void __cluster_dims__(kFinalCtas, 1, 1) __launch_bounds__(kLossThread
     constexpr int kStride = kFinalCtas * kLossThreads;
     const sg_view &vw = a.views[v];
     const double HW = (double)vw.W * vw.H;
-    __shared__ PairSum s_w[kLossThreads / 32][4];
+    __shared__ double s_w[kLossThreads / 32][4];
     __shared__ double s_part[kFinalCtas][4];  // (rank 0's holds the shares)
-    PairSum part[4];  // colour, semantics, depth L1, CE
-    for (int i = a.lv.tile_off[v] + first; i < a.lv.tile_off[v + 1]; i += kStride)
+    // add(k, x) for the thread's partials: colour, semantics, depth L1, CE
+    auto gather = [&](auto add) {
+        for (int i = a.lv.tile_off[v] + first; i < a.lv.tile_off[v + 1]; i += kStride)
 #pragma unroll
-        for (int g = 0; g < kSsimGroups; ++g)
-            if (g < a.rgb_groups + a.sem_groups) {
-                const float t = a.ssim[(size_t)g * a.n_tiles + i];
-                if (g < a.rgb_groups) part[0].add(t); else part[1].add(t);
-            }
-    // the per-unit (depth L1, CE) sums: two units per 16-byte load, four loads in flight per
-    // thread, summed in a fixed order
-    {
+            for (int g = 0; g < kSsimGroups; ++g)
+                if (g < a.rgb_groups + a.sem_groups) {
+                    const float t = a.ssim[(size_t)g * a.n_tiles + i];
+                    if (g < a.rgb_groups) add(0, t); else add(1, t);
+                }
+        // the per-unit (depth L1, CE) sums: two units per 16-byte load, four loads in flight per
+        // thread, summed in a fixed order
         const float4 *p4 = reinterpret_cast<const float4 *>(a.pix);
         const int s1 = kPixSlots * a.lv.pix_blk_off[v + 1] / 2;
         for (int i = kPixSlots * a.lv.pix_blk_off[v] / 2 + first; i < s1; i += 4 * kStride) {
@@ -1006,29 +1007,46 @@ __global__ void __cluster_dims__(kFinalCtas, 1, 1) __launch_bounds__(kLossThread
                 q[k] = i + k * kStride < s1 ? p4[i + k * kStride] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                part[2].add(q[k].x);
-                part[2].add(q[k].z);
-                part[3].add(q[k].y);
-                part[3].add(q[k].w);
+                add(2, q[k].x);
+                add(2, q[k].z);
+                add(3, q[k].y);
+                add(3, q[k].w);
             }
         }
-    }
+    };
     // the four sums side by side: warp trees, then one thread each over the warps and the CTAs, in
     // order and in double
+    PairSum part[4];
+    gather([&](int k, float x) { part[k].add(x); });
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             part[k].add(__shfl_down_sync(SG_FULL_MASK, part[k].hi, o), __shfl_down_sync(SG_FULL_MASK, part[k].lo, o));
+    double sum[4];
+    bool finite = true;  // (lane 0's sums take in every lane's: one that is not finite stays so)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        sum[k] = part[k].value();
+        finite = finite && isfinite(part[k].hi);
+    }
+    if (!__shfl_sync(SG_FULL_MASK, (int)finite, 0)) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) sum[k] = 0.0;
+        gather([&](int k, float x) { sum[k] += x; });
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sum[k] += __shfl_down_sync(SG_FULL_MASK, sum[k], o);
+    }
     if ((threadIdx.x & 31) == 0)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) s_w[threadIdx.x >> 5][k] = part[k];
+        for (int k = 0; k < 4; ++k) s_w[threadIdx.x >> 5][k] = sum[k];
     cluster.sync();  // (rank 0 runs: its shared memory can be written)
     const int k = threadIdx.x;
     if (k < 4) {
         double t = 0.0;
 #pragma unroll
-        for (int w = 0; w < kLossThreads / 32; ++w) t += s_w[w][k].value();
+        for (int w = 0; w < kLossThreads / 32; ++w) t += s_w[w][k];
         *cluster.map_shared_rank(&s_part[rank][k], 0) = t;
     }
     cluster.sync();
