@@ -156,8 +156,7 @@ typedef struct {
                        (u_int + u_frac, v_int + v_frac) and
                        1/2 d^T Sigma2D^{-1} d = (m00 dx)^2 + (m10 dx + m11 dy)^2            */
     uint32_t *rect; /* R x 2: tile rectangle [tx0,tx1) x [ty0,ty1) as (tx0|ty0<<16, tx1|ty1<<16);
-                       an empty rectangle means the record is culled (its geo and ext
-                       entries are left unwritten)                                      */
+                       an empty rectangle means the record is culled                    */
     float *ext;     /* R x 2: half extents (pixels) of the region where alpha can reach
                        alpha_min, with margin (8-B aligned)                             */
     float *rgb;     /* R x 3: colour of each record seen from its view-level, written by

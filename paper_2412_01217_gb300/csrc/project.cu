@@ -307,10 +307,9 @@ __global__ void __launch_bounds__(256) __maxnreg__((D == 0 ? 64 : D <= 2 ? 128 :
         }
         ViewGeom q;
         level_geom(vw, pose, s_lim[v], q);
-        // an empty rectangle marks a culled record; nothing reads its geometry, which is written
-        // for visible records only: on a large map most are culled (batched workload: 12M records,
-        // 2.1M visible), and zeros for them would be most of the kernel's traffic
+        float4 g0 = make_float4(0.f, 0.f, 0.f, 0.f), g1 = g0;
         uint2 rc = make_uint2(0u, 0u);
+        float2 e2 = make_float2(0.f, 0.f);
         const float tz = q.t[2];
         if (tz > pc.z_near && o >= pc.alpha_min) {
             // the 2D mean in double-float: t = R mu + t_cw and (fx t_x / t_z + cx, ...)
@@ -355,14 +354,14 @@ __global__ void __launch_bounds__(256) __maxnreg__((D == 0 ? 64 : D <= 2 ? 128 :
                     const float ui = rintf(u), vi = rintf(vv);
                     const float uf = __fadd_rn(__fsub_rn(udf.hi, ui), udf.lo);
                     const float vf = __fadd_rn(__fsub_rn(vdf.hi, vi), vdf.lo);
-                    geo[2 * r] = make_float4(uf, vf, tz, o);
+                    g0 = make_float4(uf, vf, tz, o);
                     // conditional form of 1/2 d^T Sigma2D^{-1} d (see eval_alpha)
                     const float m00 = rsqrtf(2.f * s00);
                     const float m11 = sqrtf(s00 / (2.f * det));
                     const float m10 = -s01 / sqrtf(2.f * s00 * det);
                     const uint32_t packed = ((uint32_t)(int)ui & 0xffffu) | (((uint32_t)(int)vi & 0xffffu) << 16);
-                    geo[2 * r + 1] = make_float4(m00, m10, m11, __uint_as_float(packed));
-                    ext[r] = make_float2(ex, ey);
+                    g1 = make_float4(m00, m10, m11, __uint_as_float(packed));
+                    e2 = make_float2(ex, ey);
                     if constexpr (D > 0) {
                         // colour = rgb + sum_k sh_k Y_k(d), d = (mu - c) / |mu - c|; the same
                         // for the semantic feature with sem_sh
@@ -401,7 +400,10 @@ __global__ void __launch_bounds__(256) __maxnreg__((D == 0 ? 64 : D <= 2 ? 128 :
                 }
             }
         }
+        geo[2 * r] = g0;
+        geo[2 * r + 1] = g1;
         rect[r] = rc;
+        ext[r] = e2;
     }
 }
 
