@@ -26,12 +26,12 @@
 // Parts are drawn in order, so the predecessors of a part are held by blocks that already run;
 // every wait is bounded all the same (SG_STATUS_TIMEOUT), and a step whose predecessor gave up
 // takes its input as empty: what the failed step left behind (places never written) is not read,
-// and the lists come out empty.  The steps were three kernels each
-// before (count, scan of the counts, apply): 33 launches per list build, now 12 or 13 and one
-// memset, and the keys and footprints are read once instead of twice.  What that gives is
-// the launches and their latencies (320x180 x 3 levels with 30k Gaussians: 110 -> 70 us of
-// kernels and 21 launch gaps); on the batched workload (2.1M visible records, 19M instances)
-// the kernels take the same time as before (1.0 ms).
+// and the lists come out empty.  The steps were three kernels each before (count, scan of the
+// counts, apply): 33 launches per list build, now 10 to 12 (by the width of the tile ids) and one
+// memset, and the keys and footprints are read once instead of twice.  What that gives is the
+// launches and their latencies (320x180 x 3 levels with 30k Gaussians: 110 -> 70 us of kernels
+// and 21 launch gaps); on the batched workload (2.1M visible records, 19M instances) the kernels
+// take the same time as before (1.0 ms).
 #include <cstdio>
 
 #include <algorithm>
@@ -100,11 +100,12 @@ struct StepWaits {
         atomicOr(status, SG_STATUS_TIMEOUT);
         *own = 1;
     }
-    // Whether an earlier step gave up (uniform over the grid: their kernels are done).
-    __device__ __forceinline__ bool broken() const {
-        if (!before || !*before) return false;
+    // n, or 0 if an earlier step gave up (uniform over the grid: their kernels are done; the flag
+    // and n, which the caller has read, are in flight together).
+    __device__ __forceinline__ int input(int n) const {
+        if (!before || !*before) return n;
         *own = 1;
-        return true;
+        return 0;
     }
 };
 
@@ -495,7 +496,7 @@ __global__ void __launch_bounds__(kScanThreads) slot_prefix_kernel(const uint2 *
                                                                    int *__restrict__ total, StepWaits sw) {
     pdl_begin();
     constexpr int E = kCompactPerThread;
-    const int n = sw.broken() ? 0 : *m_ptr;
+    const int n = sw.input(*m_ptr);
     const int parts = (n + kCompactPart - 1) / kCompactPart;
     for (int part; (part = next_part(counter)) < parts;) {
         // thread t takes records base + 32 (8 warp + q) + lane: coalesced loads, and the scan runs
@@ -585,9 +586,8 @@ __global__ void __launch_bounds__(kScanThreads, 6) cull_kernel(
     for (int v = threadIdx.x; v < n_views; v += kScanThreads)
         s_vw[v] = make_int4(views[v].W, views[v].H, views[v].tile_offset, views[v].tiles_x);
     for (int i = threadIdx.x; i < 4 * 256; i += kScanThreads) s_h[i] = 0;
-    const bool broken = sw.broken();
-    const int n = broken ? 0 : *m_ptr;
-    const uint32_t S = broken ? 0u : (uint32_t)*s_ptr;
+    const int n = *m_ptr;
+    const uint32_t S = (uint32_t)sw.input(*s_ptr);  // (without slots no record is read)
     const int chunks = (int)(((uint64_t)S + 255) / 256);
     // chunks of a part: at most two parts per block, one chunk for small inputs
     const int per = max(1, max((chunks + kMaxChunks - 1) / kMaxChunks, (chunks + 2 * (int)gridDim.x - 1) / (2 * (int)gridDim.x)));
@@ -765,7 +765,7 @@ __global__ void __launch_bounds__(kScanThreads, 4) sweep_kernel(
     __shared__ uint32_t wcnt[kWarps][256];  // per-warp digit counts, then per-warp offsets
     __shared__ uint32_t skey[CH], sval[CH];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n = sw.broken() ? 0 : min(*n_ptr, cap);
+    const int n = sw.input(min(*n_ptr, cap));
     const int parts = (int)(((int64_t)n + CH - 1) / CH);
     uint32_t unused;
     const uint32_t first = block_exclusive_scan(hist[tid], unused);  // digit tid's first output position
@@ -925,12 +925,13 @@ __global__ void __launch_bounds__(kScanThreads) ranges_kernel(const uint32_t *__
                                                               int2 *__restrict__ ranges, uint32_t *__restrict__ hist,
                                                               const int *__restrict__ failed) {
     pdl_begin();
+    const int found = *k_ptr;
     const bool broken = *failed != 0;  // (a step gave up: no instances)
     if (broken && blockIdx.x == 0 && threadIdx.x == 0) *k_ptr = 0;
     __shared__ uint32_t s_h[64];
     if (threadIdx.x < 64) s_h[threadIdx.x] = 0;
     __syncthreads();
-    const int K = broken ? 0 : min(*k_ptr, cap), lane = threadIdx.x & 31;
+    const int K = broken ? 0 : min(found, cap), lane = threadIdx.x & 31;
     const int t = blockIdx.x * kScanThreads + (int)threadIdx.x, t0 = t - lane;
     if (t0 < n_tiles) {  // (warp-uniform)
         const int wlo = warp_lower_bound_u32(tile, K, (uint32_t)t0);
