@@ -128,8 +128,8 @@ typedef struct {
     int32_t persistent;     /* 1: persistent grid with an atomic work queue           */
     int32_t pixels_per_thread;     /* forward: 1, 2 or 4 pixels per thread (rows 4 apart);
                                       tile_h % (4 * it) == 0, tile pixels >= 32 * it       */
-    int32_t pixels_per_thread_bwd; /* at most so many for the backward kernel (1, 2 or 4 with
-                                      the same conditions); it runs one, the fastest      */
+    int32_t pixels_per_thread_bwd; /* checked (1, 2 or 4 with the same conditions) but without
+                                      effect: the backward kernel runs one, the fastest   */
     int32_t batch_bwd;      /* batch of the backward kernel; 0: the same as `batch`    */
     int32_t isotropic;      /* 0: EWA projection of the anisotropic Gaussian (log_scale,
                                quat); 1: Eq. 2 as printed: an isotropic Gaussian of radius

@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(256) __maxnreg__((D == 0 ? 64 : D <= 2 ? 128 :
                     const float uf = __fadd_rn(__fsub_rn(udf.hi, ui), udf.lo);
                     const float vf = __fadd_rn(__fsub_rn(vdf.hi, vi), vdf.lo);
                     g0 = make_float4(uf, vf, tz, o);
-                    // conditional form of 1/2 d^T Sigma2D^{-1} d (see eval_alpha)
+                    // conditional form of 1/2 d^T Sigma2D^{-1} d (see entry_alpha)
                     const float m00 = rsqrtf(2.f * s00);
                     const float m11 = sqrtf(s00 / (2.f * det));
                     const float m10 = -s01 / sqrtf(2.f * s00 * det);

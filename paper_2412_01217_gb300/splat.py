@@ -69,7 +69,7 @@ class RenderConfig:
     batch: int = 256
     persistent: bool = True
     pixels_per_thread: int = 1
-    pixels_per_thread_bwd: int = 2  # an upper bound: the adjoint runs one pixel per thread
+    pixels_per_thread_bwd: int = 2  # checked but without effect: the adjoint runs one pixel per thread
     batch_bwd: int = 0  # 0: same as batch
     isotropic: bool = False  # Eq. 2 projection (radius f r / d) instead of EWA
     check_numeric: bool = False  # flag non-finite Gaussian parameters in the status word
